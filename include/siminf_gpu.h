@@ -310,17 +310,18 @@ int sg_set_replicate_range(sg_model *m, int32_t rep0, int32_t rep_total);
 
 /* Work split of the SSA day kernel.  With nodes_per_block in 1..128 each
  * block of 128 threads owns that many (replicate, node) pairs, one per
- * thread, kept in registers for a run of days; a node whose SSA needs more
- * than heavy_after draws in a day is handed to one of the block's warps,
- * whose 32 lanes compute 32 draws' random numbers at once.  With
+ * thread, kept in registers for a run of days; a node that expects
+ * heavy_after transitions or more in a day (a rate at the day's start; for
+ * S or G other than the kind's own and for aem: that has taken heavy_after
+ * draws) is handed to one of the block's warps, whose 32 lanes evaluate 32
+ * draws at once.  With
  * nodes_per_block > 128 (up to 2^22; the direct method on the built-in
  * kinds without emulator or persistent schedule -- elsewhere it
  * means 128) the sparse-activity schedule runs instead: each block of 256
  * threads owns nodes_per_block pairs in device memory, skips the days that
  * are certainly empty (no infected animal and phi == +0, with finite model
  * parameters), and runs the SSA of the pairs with a positive total rate from
- * a compact list, one thread each, handing those that need more than
- * heavy_after draws to warps.  When nodes_per_block is also a multiple of
+ * a compact list, one thread each, handing over to warps as above.  When nodes_per_block is also a multiple of
  * the node count (every block holds whole replicates) the whole run is one
  * launch: each block runs its replicates' external transfers itself and no
  * block waits for another.  Results are identical for every setting (the
@@ -328,10 +329,11 @@ int sg_set_replicate_range(sg_model *m, int32_t rep0, int32_t rep_total);
  * only speed changes.  nodes_per_block <= 0 or heavy_after < 0 restore the
  * size-based defaults: where the sparse-activity schedule applies and the
  * pairs exceed two full 128-pair blocks per SM, one replicate per block
- * and heavy_after 32 when there are at least as many replicates as SMs
- * (and more than 128 nodes), else two blocks per SM and heavy_after 8;
- * otherwise 128 pairs per block (fewer for small problems, so that about
- * two blocks per SM exist) and heavy_after 2. */
+ * when there are at least as many replicates as SMs (and more than 128
+ * nodes), else two blocks per SM; otherwise 128 pairs per block (fewer for
+ * small problems, so that about two blocks per SM exist).  By default no
+ * node is handed over (S, G other than the kind's own: after 32, 8 and 2
+ * draws in these three cases; aem: after 2). */
 int sg_set_tuning(sg_model *m, int32_t nodes_per_block, int32_t heavy_after);
 
 /* Autotuner: for each of nodes_per_block in {4, 8, 16, 32, 64, 128} x
@@ -615,11 +617,16 @@ int sg_emulator_set_fp8(sg_model *m, const void *const *W8, const float *const *
  *                    for i < n  (Salmon et al., SC'11)
  *   sg_log_batch:    y[i] = the library's natural logarithm of x[i]
  *   sg_u01_batch:    y[i] = open-interval uniform of words w[2 i], w[2 i+1]
+ *   sg_filter_bounds_batch: FP32 bounds as the SSA's interval decisions use
+ *                    them: out[4 i], out[4 i + 1] of -log r1 of words w[2 i],
+ *                    w[2 i + 1]; out[4 i + 2], out[4 i + 3] of 1 / x[i]
  * All pointers are device pointers. */
 int sg_philox_batch(const uint32_t *d_ctr, uint64_t key, uint32_t *d_out,
                     int64_t n, void *stream);
 int sg_log_batch(const double *d_x, double *d_y, int64_t n, void *stream);
 int sg_u01_batch(const uint32_t *d_w, double *d_y, int64_t n, void *stream);
+int sg_filter_bounds_batch(const uint32_t *d_w, const float *d_x, float *d_out,
+                           int64_t n, void *stream);
 
 /* FP64 throughput probe for roofline statements: runs independent chains of
  * fused multiply-adds on every SM for about `iters` steps and returns the

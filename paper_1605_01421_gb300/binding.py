@@ -23,13 +23,13 @@ _BUILD = os.path.join(_PKG, "_build")
 LIB_PATH = os.path.join(_BUILD, "libsiminf_gpu.so")
 
 SOURCES = ["sg_engine.cu", "sg_plan.cpp", "sg_mlp.cu", "sg_mparse.cpp"]
-HEADERS = ["sg_common.h", "sg_device.cuh", "sg_kernels.cuh", "sg_plan.h", "sg_mlp.h", "sg_tc.cuh",
+HEADERS = ["sg_common.h", "sg_device.cuh", "sg_filter.cuh", "sg_kernels.cuh", "sg_plan.h", "sg_mlp.h", "sg_tc.cuh",
            "sg_mparse.h"]
 # The headers the run-time compiler (NVRTC) sees for a model from transition
 # strings, embedded into the library; NVRTC has no C library, so the two
 # standard headers they include are replaced by minimal ones.
 JIT_HEADERS = [("siminf_gpu.h", "include"), ("sg_common.h", "csrc"), ("sg_device.cuh", "csrc"),
-               ("sg_kernels.cuh", "csrc")]
+               ("sg_filter.cuh", "csrc"), ("sg_kernels.cuh", "csrc")]
 _JIT_STDINT = """#pragma once
 typedef signed char int8_t;
 typedef unsigned char uint8_t;
@@ -167,7 +167,7 @@ class Stats(ctypes.Structure):
 
 EXPORTS = ["sg_model_create", "sg_set_events", "sg_run", "sg_run_host",
            "sg_model_destroy", "sg_strerror", "sg_philox_batch", "sg_log_batch",
-           "sg_u01_batch", "sg_set_kernel_timing", "sg_fp64_fma_probe",
+           "sg_u01_batch", "sg_filter_bounds_batch", "sg_set_kernel_timing", "sg_fp64_fma_probe",
            "sg_run_noalloc", "sg_set_tuning", "sg_autotune", "sg_set_graphs",
            "sg_gemm_bf16", "sg_mlp_ce_loss", "sg_gelu_backward", "sg_transpose_bf16",
            "sg_colsum_bf16", "sg_adam_step", "sg_emu_features", "sg_emu_targets",
@@ -214,6 +214,8 @@ def lib(path: str | None = None):
         L.sg_log_batch.restype = ctypes.c_int
         L.sg_u01_batch.argtypes = [vp, vp, i64, vp]
         L.sg_u01_batch.restype = ctypes.c_int
+        L.sg_filter_bounds_batch.argtypes = [vp, vp, vp, i64, vp]
+        L.sg_filter_bounds_batch.restype = ctypes.c_int
         L.sg_set_kernel_timing.argtypes = [vp, ctypes.c_int]
         L.sg_set_kernel_timing.restype = ctypes.c_int
         L.sg_fp64_fma_probe.argtypes = [i32, ctypes.POINTER(ctypes.c_double), vp]
@@ -810,3 +812,18 @@ def u01_batch(words, stream=None):
     if rc:
         raise SimInfError(rc)
     return y.cpu().numpy()
+
+
+def filter_bounds_batch(words, x, stream=None):
+    """FP32 bounds (lo, hi) of -log r1 for Philox words (n, 2) and of 1 / x
+    for x in [2^-100, 2^100], as the day kernels use them; float32 (n, 4)."""
+    import torch
+    w = torch.as_tensor(np.ascontiguousarray(words, dtype=np.uint32).view(np.int32),
+                        device="cuda")
+    t = torch.as_tensor(np.ascontiguousarray(x, dtype=np.float32), device="cuda")
+    out = torch.empty((t.numel(), 4), dtype=torch.float32, device="cuda")
+    rc = lib().sg_filter_bounds_batch(_dev_ptr(w), _dev_ptr(t), _dev_ptr(out), t.numel(),
+                                      _stream_handle(stream))
+    if rc:
+        raise SimInfError(rc)
+    return out.cpu().numpy()

@@ -24,6 +24,7 @@ struct SgTables {
   uint32_t Emask[SG_MAX_SELECT];         // bit p: compartment p in E[, s]
   int8_t Nsh[SG_MAX_SHIFT][SG_MAX_COMP]; // Nsh[q][p] = N[p, q]
   double gdata[SG_MAX_GDATA];
+  float g_lo[SG_MAX_GDATA], g_hi[SG_MAX_GDATA];  // FP32 neighbours: g_lo <= gdata <= g_hi
 };
 
 // Scheduled events in planned order, structure of arrays on the device.

@@ -67,6 +67,11 @@ __device__ __forceinline__ double i2d(int n) {
   return __longlong_as_double((long long)(((unsigned long long)(p + 1023) << 52) | frac));
 }
 
+// (double)n of a sum of counts.
+__device__ __forceinline__ double l2d(long long n) {
+  return n == (long long)(int)n ? i2d((int)n) : (double)n;
+}
+
 // Order-preserving integer key of a double (for non-NaN values, including
 // negatives): a < b  <=>  key(a) < key(b), except that -0 orders below +0.
 __device__ __forceinline__ long long order_key(double x) {
@@ -363,20 +368,16 @@ __device__ __forceinline__ double season_decay(int t, const int *ends, const dou
 template <int KIND>
 __device__ __forceinline__ int post_step(double *v, const int *u, const int *ends,
                                          const double *g, int t) {
+  // sums of counts: exact in FP64, so taken in integers
   double I_tot, N_tot;
   const double *pg;
   if (KIND == SG_SISE) {
     I_tot = i2d(u[1]);
-    N_tot = i2d(u[0]) + i2d(u[1]);
+    N_tot = l2d((long long)u[0] + u[1]);
     pg = g + 2;
   } else if (KIND == SG_SISE3) {
-    I_tot = 0.0;
-    N_tot = 0.0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      I_tot = I_tot + i2d(u[2 * a + 1]);
-      N_tot = N_tot + i2d(u[2 * a]) + i2d(u[2 * a + 1]);
-    }
+    I_tot = l2d((long long)u[1] + u[3] + u[5]);
+    N_tot = l2d((long long)u[0] + u[1] + u[2] + u[3] + u[4] + u[5]);
     pg = g + 6;
   } else {
     return 0;

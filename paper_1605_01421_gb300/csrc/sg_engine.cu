@@ -182,6 +182,19 @@ __global__ void k_u01_batch(const uint32_t *w, double *y, long long n) {
     y[i] = u01_open(w[2 * i], w[2 * i + 1]);
 }
 
+// The intervals of sg_filter.cuh for test: bounds of -log r1 for the words
+// w[2i], w[2i + 1], and of the reciprocal of x[i].
+__global__ void k_filter_bounds(const uint32_t *w, const float *x, float *out, long long n) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    const Itv e = itv_neglog(w[2 * i], w[2 * i + 1]);
+    out[4 * i] = e.lo;
+    out[4 * i + 1] = e.hi;
+    out[4 * i + 2] = rcp_lo(x[i]);
+    out[4 * i + 3] = rcp_hi(x[i]);
+  }
+}
+
 // Independent fused multiply-add chains (8 per thread) for the FP64
 // throughput probe; the result is stored so the chains are not removed.
 __global__ void k_fp64_fma(double *out, int iters) {
@@ -464,6 +477,46 @@ static const int kKindNv[5] = {0, 0, 1, 1, 1};
 static const int kKindGdata[5] = {2, 2, 7, 11, 8};
 static const int kKindLdata[5] = {0, 0, 4, 4, 4};
 
+// Global data and their FP32 neighbours (NaN where there are none).
+static void set_gdata(SgTables &tb, const sg_desc *d) {
+  for (int i = 0; i < d->n_gdata; ++i) {
+    const double x = d->gdata[i];
+    const float f = (float)x;
+    tb.gdata[i] = x;
+    tb.g_lo[i] = (double)f <= x ? f : std::nextafterf(f, -INFINITY);
+    tb.g_hi[i] = (double)f >= x ? f : std::nextafterf(f, INFINITY);
+    if (!std::isfinite(tb.g_lo[i]) || !std::isfinite(tb.g_hi[i]))
+      tb.g_lo[i] = tb.g_hi[i] = NAN;
+  }
+}
+
+// Whether the day kernels may decide draws from intervals (sg_filter.cuh):
+// the transitions are the kind's own, G marks at least the rates that each
+// one changes (then every rate equals its value at the current counts), and
+// the rate parameters are not negative (NaN intervals catch the rest).
+// Models from transition strings derive both from the strings.
+static bool filter_applies(const SgTables &tb) {
+  if (tb.kind == SG_GENERIC) return true;
+  const bool three = tb.kind == SG_SISE3;
+  const int n_rates = three ? 6 : 2;
+  for (int j = 0; j < tb.n_trans; ++j) {
+    int8_t want[SG_MAX_COMP] = {};
+    if (tb.kind == SG_SIR) {
+      want[j] = -1;
+      want[j + 1] = 1;
+    } else {
+      want[j] = -1;
+      want[j ^ 1] = 1;
+    }
+    if (std::memcmp(want, tb.S[j], sizeof want) != 0) return false;
+    const uint32_t need = three ? 3u << (j & ~1) : 3u;
+    if ((tb.dep[j] & need) != need) return false;
+  }
+  for (int i = 0; i < n_rates; ++i)
+    if (!(tb.g_lo[i] >= 0.0f)) return false;
+  return true;
+}
+
 static int model_create(const sg_desc *d, sg_model **out, bool generic);
 
 extern "C" int sg_model_create(const sg_desc *d, sg_model **out) {
@@ -525,7 +578,7 @@ static int model_create(const sg_desc *d, sg_model **out, bool generic) {
       if (x < -127 || x > 127) { delete m; return SG_ERR_ARG; }
       tb.Nsh[q][p] = (int8_t)x;
     }
-  for (int i = 0; i < d->n_gdata; ++i) tb.gdata[i] = d->gdata[i];
+  set_gdata(tb, d);
   const size_t nl = (size_t)d->n_ldata * d->n_nodes;
   std::vector<double> ld(d->ldata ? d->ldata : nullptr, d->ldata ? d->ldata + nl : nullptr);
   int rc = upload(m->ldata, ld);
@@ -1462,6 +1515,8 @@ extern "C" int sg_run(sg_model *m, const int32_t *tspan, int32_t n_tspan, uint64
   da.slots = slots;
   da.rep0 = m->rep0;
   da.heavy_after = m->heavy_after >= 0 ? m->heavy_after : 2;
+  da.fast = filter_applies(tb) ? 1 : 0;
+  da.warp_rate = m->heavy_after >= 0 ? (float)std::max(1, m->heavy_after) : INFINITY;
   da.npb = m->npb > 0 ? m->npb : default_npb((long long)Nn * n_rep);
   // the sparse-activity schedule (nodes_per_block > kDayBlock) is for the
   // direct method on the built-in kinds with the day / E2 kernel pair;
@@ -1552,7 +1607,7 @@ extern "C" int sg_run(sg_model *m, const int32_t *tspan, int32_t n_tspan, uint64
                      t0,
                      t_end,
                      da.npb,
-                     da.heavy_after,
+                     m->heavy_after,
                      m->rep0,
                      (m->plan_version * 1000003ull + (m->emu_on ? m->emu_version + 1 : 0)) *
                              1000033ull +
@@ -1729,6 +1784,19 @@ extern "C" int sg_u01_batch(const uint32_t *d_w, double *d_y, int64_t n, void *s
   return SG_OK;
 }
 
+extern "C" int sg_filter_bounds_batch(const uint32_t *d_w, const float *d_x, float *d_out,
+                                      int64_t n, void *stream) {
+  if (n < 0 || (n > 0 && (!d_w || !d_x || !d_out))) return SG_ERR_ARG;
+  if (n == 0) return SG_OK;
+  k_filter_bounds<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>(d_w, d_x, d_out, n);
+  if (cudaGetLastError() != cudaSuccess ||
+      cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) {
+    cudaGetLastError();
+    return SG_ERR_CUDA;
+  }
+  return SG_OK;
+}
+
 extern "C" int sg_set_kernel_timing(sg_model *m, int enable) {
   if (!m) return SG_ERR_ARG;
   m->timing = enable != 0;
@@ -1859,7 +1927,7 @@ extern "C" int sg_run_noalloc(const sg_desc *d, const double *d_ldata, const int
       if (d->G[(size_t)j * T + kk] != 0) dep |= 1u << kk;
     tb.dep[j] = dep;
   }
-  for (int i = 0; i < d->n_gdata; ++i) tb.gdata[i] = d->gdata[i];
+  set_gdata(tb, d);
 
   // scratch layout: error word | counters | tspan | rec | u | v
   const int32_t t0 = tspan[0], t_end = tspan[n_tspan - 1], days = t_end - t0;
@@ -1921,6 +1989,8 @@ extern "C" int sg_run_noalloc(const sg_desc *d, const double *d_ldata, const int
       da.n_rep = n_rep;
       da.slots = 1;
       da.heavy_after = 2;
+      da.fast = filter_applies(tb) ? 1 : 0;
+      da.warp_rate = INFINITY;
       da.npb = default_npb((long long)Nn * n_rep);
       da.emu = nullptr;
       da.T_begin = t0 + 1;

@@ -9,6 +9,7 @@
 
 #include "sg_common.h"
 #include "sg_device.cuh"
+#include "sg_filter.cuh"
 
 namespace sg {
 
@@ -167,6 +168,10 @@ struct DayArgs {
   int32_t finish_first;    // finish unit step T_begin - 1 before the SSA
   int32_t finish_last;     // finish unit step T_end - 1 after the SSA
   int32_t heavy_after;     // draws a thread takes before its warp takes over
+  // 1: the model's S and G are its kind's own and its parameters finite and
+  // not negative, so the intervals of sg_filter.cuh apply
+  int32_t fast;
+  float warp_rate;         // expected transitions from which a unit's day goes to a warp
   int32_t npb;             // nodes per block (<= kDayBlock); the other
                            // threads of the block only serve heavy nodes
   const int32_t *emu;      // [R][Nn][4]: emulated increments of I_1..I_3 and
@@ -471,564 +476,330 @@ __device__ __forceinline__ int select_prefix(const double *w, const double *P, d
   return n < 0 ? last : n;
 }
 
-enum { SSA_DONE = 0, SSA_HEAVY = 1 };
+enum { SSA_DONE = 0, SSA_REDO = 1 };
 
-// Direct SSA of one node toward the unit time Tn in its own thread, for at
-// most `budget` draws (Appendix A, one iteration per draw).  Returns SSA_DONE,
-// SSA_HEAVY (budget spent, state and counter ready for the warp) or an error.
+// Direct SSA of one unit's day toward Td in its own thread, every operation
+// in FP64 (Appendix A, one iteration per draw).  Returns SSA_DONE, SSA_REDO
+// (counts unchanged: more than `budget` draws were due, the day is left to a
+// warp, which starts it again because rates kept by a caller's own G depend
+// on the way to a state) or an error.
 template <int KIND>
-__device__ __forceinline__ int ssa_thread(int *u, double *w, const double *kf, double &t,
-                                          uint32_t &c, double Tn, uint32_t node, uint32_t Td,
-                                          uint32_t tag, uint32_t k0, uint32_t k1, int budget,
-                                          const SgTables &tb, unsigned long long &fired) {
+__device__ __forceinline__ int ssa_exact(int *u0, const double *kf, uint32_t node, uint32_t Td,
+                                         uint32_t tag, uint32_t k0, uint32_t k1, int budget,
+                                         const SgTables &tb, unsigned long long &fired,
+                                         unsigned long long &drawn) {
   using M = ModelTraits<KIND>;
+  const double Tn = (double)(int)Td;
   const long long Tkey = order_key(Tn);
-  for (int b = 0;; ++b) {
+  double t = (double)((int)Td - 1);
+  uint32_t c = 0, f = 0;
+  int code = SSA_DONE;
+  int u[M::C];
+  double w[M::T];
+#pragma unroll
+  for (int p = 0; p < M::C; ++p) u[p] = u0[p];
+#pragma unroll
+  for (int j = 0; j < M::T; ++j) {
+    w[j] = M::rate_k(j, u, kf, tb.gdata);
+    if (bad_rate(w[j])) code = SG_ERR_RATE;
+  }
+  while (code == SSA_DONE) {
     // lambda = ((0 + w_1) + w_2) + ...; the leading 0 + w_1 changes no
     // decision or value, so the sum starts at w_1
     double lam = w[0];
 #pragma unroll
     for (int j = 1; j < M::T; ++j) lam = lam + w[j];
-    if (!gt0(lam)) return SSA_DONE;  // nothing can fire: jump to Tn
-    if (c >= SG_MAX_DRAWS) return SG_ERR_STEP_LIMIT;
-    if (b == budget) return SSA_HEAVY;
-    const U4 x = philox10(U4{c, node, Td, tag}, k0, k1);
-    ++c;
-    const double r1 = u01_open(x.x, x.y);
-    const double r2 = u01_open(x.z, x.w);
-    const double tau = -log_pos(r1) / lam;
-    const double tt = t + tau;
-    if (order_key(tt) >= Tkey) return SSA_DONE;
-    t = tt;
-    const int rc = fire<KIND>(u, w, lam * r2, kf, tb);
-    ++fired;
-    if (rc) return rc;
-  }
-}
-
-// One iteration of ssa_thread's loop (one draw of the direct method,
-// Appendix A): returns SSA_STEP_FIRED (a transition fired, t and u moved on),
-// SSA_DONE (lambda = 0 or the next event falls at or after Tn),
-// SSA_HEAVY (hand_off set and a draw is due: state unchanged, for a warp) or
-// an error.  The same operations in the same order as ssa_thread.
-enum { SSA_STEP_FIRED = 2 };
-template <int KIND>
-__device__ __forceinline__ int ssa_step(int *u, double *w, const double *kf, double &t,
-                                        uint32_t &c, long long Tkey, uint32_t node, uint32_t Td,
-                                        uint32_t tag, uint32_t k0, uint32_t k1, bool hand_off,
-                                        const SgTables &tb, unsigned long long &fired) {
-  using M = ModelTraits<KIND>;
-  double lam = w[0];
-#pragma unroll
-  for (int j = 1; j < M::T; ++j) lam = lam + w[j];
-  if (!gt0(lam)) return SSA_DONE;
-  if (c >= SG_MAX_DRAWS) return SG_ERR_STEP_LIMIT;
-  if (hand_off) return SSA_HEAVY;
-  const U4 x = philox10(U4{c, node, Td, tag}, k0, k1);
-  ++c;
-  const double r1 = u01_open(x.x, x.y);
-  const double r2 = u01_open(x.z, x.w);
-  const double tau = -log_pos(r1) / lam;
-  const double tt = t + tau;
-  if (order_key(tt) >= Tkey) return SSA_DONE;
-  t = tt;
-  const int rc = fire<KIND>(u, w, lam * r2, kf, tb);
-  ++fired;
-  return rc ? rc : SSA_STEP_FIRED;
-}
-
-// A node handed from its thread to a warp.
-template <int C, int NK>
-struct HeavySlot {
-  double t;
-  double kf[NK];
-  uint32_t c;
-  int32_t node, rep, code;
-  int32_t u[C];
-};
-
-// SISe3 heavy node-days, three draws per parallel round (see the comment
-// inside); returns false, doing nothing, for other kinds or another
-// dependency graph (the caller then takes the sequential loop).
-template <int KIND>
-__device__ __forceinline__ bool ssa_window3(int *u, double *w, const double *kf, double &t,
-                                            uint32_t &c, uint32_t &c0, double &nE, double &r2,
-                                            bool &have, unsigned long long &f, int &code,
-                                            uint32_t node, uint32_t Td, uint32_t tag, uint32_t k0,
-                                            uint32_t k1, long long Tkey, const SgTables &tb) {
-  if constexpr (KIND != SG_SISE3) {
-    return false;
-  } else {
-    using M = ModelTraits<KIND>;
-    constexpr int C = M::C, T = M::T;
-    if (!(tb.dep[0] == 3u && tb.dep[1] == 3u && tb.dep[2] == 12u && tb.dep[3] == 12u &&
-          tb.dep[4] == 48u && tb.dep[5] == 48u))
-      return false;
-    const int lane = threadIdx.x & 31;
-    // SISe3 with its block-diagonal dependency graph (each transition changes
-    // and is changed by its own age class only), so the rates of a state are
-    // the same however it was reached.  The states reachable within the next
-    // J = 3 draws are u plus at most two columns of S: the root (lane 0), one
-    // transition n (lanes 1 + n) and two transitions a <= b (lanes 7 +
-    // pair(a, b)), 28 in all.  Every lane evaluates its state's draw (draw
-    // c + depth): rates, lambda in index order, waiting-time divide and
-    // inversion; the walk then follows the fired transitions through the
-    // table.  Same operations and order as the sequential loop.
-    constexpr int J = 3;
-    constexpr int kT = ModelTraits<SG_SISE3>::T;  // 6
-    auto pair = [](int a, int b) { return a * kT - a * (a - 1) / 2 + (b - a); };
-    int depth = 0, ma = -1, mb = -1;  // this lane's state: root, {ma}, {ma, mb}
-    if (lane >= 1 && lane <= kT) {
-      depth = 1;
-      ma = lane - 1;
-    } else if (lane > kT && lane < 1 + kT + kT * (kT + 1) / 2) {
-      depth = 2;
-      int l = lane - 1 - kT, a = 0;
-      while (l >= kT - a) {
-        l -= kT - a;
-        ++a;
-      }
-      ma = a;
-      mb = a + l;
-    }
-    bool done = false;
-    while (!done && code == 0) {
-      if (!have || c + (uint32_t)J - c0 > 32u) {
-        c0 = c;
-        const U4 x = philox10(U4{c0 + (uint32_t)lane, node, Td, tag}, k0, k1);
-        nE = -log_pos(u01_open(x.x, x.y));
-        r2 = u01_open(x.z, x.w);
-        have = true;
-      }
-      int us[C];
-#pragma unroll
-      for (int p = 0; p < C; ++p) {
-        int x = u[p];
-        if (ma >= 0) x += tb.S[ma][p];
-        if (mb >= 0) x += tb.S[mb][p];
-        us[p] = x;
-      }
-      double ws[T];
-      bool bad = false;
-#pragma unroll
-      for (int j = 0; j < T; ++j) {
-        ws[j] = M::rate_k(j, us, kf, tb.gdata);
-        bad = bad || bad_rate(ws[j]);
-      }
-      const int src = (int)(c - c0) + depth;  // lane holding draw c + depth
-      const double E = __shfl_sync(0xffffffffu, nE, src);
-      const double R2 = __shfl_sync(0xffffffffu, r2, src);
-      double lam = ws[0];
-#pragma unroll
-      for (int j = 1; j < T; ++j) lam = lam + ws[j];
-      const double tau = E / lam;
-      const double target = lam * R2;
-      // inversion exactly as fire(): running sum over the positive rates
-      double cum = 0.0;
-      int nsel = -1, last = -1;
-#pragma unroll
-      for (int j = 0; j < T; ++j) {
-        if (nsel < 0 && gt0(ws[j])) {
-          cum = last < 0 ? ws[j] : cum + ws[j];
-          last = j;
-          if (le_nonneg(target, cum)) nsel = j;
-        }
-      }
-      if (nsel < 0) nsel = last;
-      const unsigned pos_mask = __ballot_sync(0xffffffffu, gt0(lam));
-      const unsigned bad_mask = __ballot_sync(0xffffffffu, bad);
-      int L = 0, n1 = -1, j = 0;
-      for (; j < J; ++j) {
-        if (j > 0 && ((bad_mask >> L) & 1u)) {
-          code = SG_ERR_RATE;  // the transition into this state gave a bad rate
-          break;
-        }
-        if (!((pos_mask >> L) & 1u)) {
-          done = true;  // nothing can fire: jump to Tn
-          break;
-        }
-        if (c >= SG_MAX_DRAWS) {
-          code = SG_ERR_STEP_LIMIT;
-          break;
-        }
-        const double tauL = __shfl_sync(0xffffffffu, tau, L);
-        const int n = __shfl_sync(0xffffffffu, nsel, L);
-        ++c;
-        const double tt = t + tauL;
-        if (order_key(tt) >= Tkey) {
-          done = true;
-          break;
-        }
-        t = tt;
-#pragma unroll
-        for (int p = 0; p < C; ++p) u[p] += tb.S[n][p];
-        ++f;
-        if (j == 0) {
-          n1 = n;
-          L = 1 + n;
-        } else if (j == 1) {
-          L = 1 + kT + (n1 <= n ? pair(n1, n) : pair(n, n1));
-        }
-      }
-      if (!done && code == 0) {
-        // j == J: a new window starts from the state after J transitions
-#pragma unroll
-        for (int k = 0; k < T; ++k) {
-          w[k] = M::rate_k(k, u, kf, tb.gdata);
-          if (bad_rate(w[k])) code = SG_ERR_RATE;
-        }
-      }
-    }
-    return true;
-  }
-}
-
-// Speculative window for heavy node-days of models from transition strings,
-// whose dependency graph is complete (the parser derives it from what each
-// propensity reads, so recomputing the rates G marks after a transition gives
-// the same rates as recomputing every rate from the counts).  The states reachable
-// within the next J draws are u plus a multiset of at most J - 1 columns of
-// S; lane l holds one such multiset (sorted transition indices a_1 <= ... ),
-// with J the largest for which they fit in a warp (T = 3: 4; T = 4..6: 3;
-// T = 7..31: 2).  Every lane evaluates its state's draw (draw c + depth):
-// rates from the counts, lambda in index order, waiting-time divide and
-// inversion; the walk then follows the fired transitions, finding the lane
-// of the state reached with a ballot, so J draws cost one parallel round
-// instead of J dependent rate updates and divides.  Same operations and
-// order as the sequential loop.  (SISe3 has a dedicated window with an
-// arithmetic walk, ssa_window3.)  Returns false, doing nothing, for other
-// kinds (the caller then takes the sequential loop).
-template <int KIND>
-__device__ __forceinline__ bool ssa_window(int *u, double *w, const double *kf, double &t,
-                                           uint32_t &c, uint32_t &c0, double &nE, double &r2,
-                                           bool &have, unsigned long long &f, int &code,
-                                           uint32_t node, uint32_t Td, uint32_t tag, uint32_t k0,
-                                           uint32_t k1, long long Tkey, const SgTables &tb) {
-  using M = ModelTraits<KIND>;
-  constexpr int C = M::C, T = M::T;
-  if constexpr (KIND != SG_GENERIC || T < 3 || T > 31) {
-    return false;
-  } else {
-    constexpr int J = T == 3 ? 4 : (T <= 6 ? 3 : 2);
-    constexpr int D = J - 1;  // largest multiset held by a lane
-    const int lane = threadIdx.x & 31;
-    // this lane's multiset: enumerate by depth, then lexicographically
-    int depth = 0, a[D > 0 ? D : 1];
-#pragma unroll
-    for (int i = 0; i < D; ++i) a[i] = -1;
-    {
-      int l = lane, d = 0, cur[D > 0 ? D : 1];
-      bool found = false;
-      // depth 0: lane 0
-      if (l == 0) {
-        found = true;
-      } else {
-        l -= 1;
-        for (d = 1; d <= D && !found; ++d) {
-          // multisets of size d in lexicographic order
-#pragma unroll
-          for (int i = 0; i < D; ++i) cur[i] = 0;
-          for (;;) {
-            if (l == 0) {
-              found = true;
-              depth = d;
-#pragma unroll
-              for (int i = 0; i < D; ++i) a[i] = i < d ? cur[i] : -1;
-              break;
-            }
-            --l;
-            // next non-decreasing tuple of length d over 0..T-1
-            int i = d - 1;
-            while (i >= 0 && cur[i] == T - 1) --i;
-            if (i < 0) break;
-            const int v = cur[i] + 1;
-            for (int k = i; k < d; ++k) cur[k] = v;
-          }
-        }
-      }
-      if (!found) depth = -1;  // a spare lane: evaluates nothing used
-    }
-    const int ev_depth = depth < 0 ? 0 : depth;
-    bool done = false;
-    while (!done && code == 0) {
-      if (!have || c + (uint32_t)J - c0 > 32u) {
-        c0 = c;
-        const U4 x = philox10(U4{c0 + (uint32_t)lane, node, Td, tag}, k0, k1);
-        nE = -log_pos(u01_open(x.x, x.y));
-        r2 = u01_open(x.z, x.w);
-        have = true;
-      }
-      int us[C];
-#pragma unroll
-      for (int p = 0; p < C; ++p) {
-        int x = u[p];
-#pragma unroll
-        for (int i = 0; i < D; ++i)
-          if (a[i] >= 0) x += tb.S[a[i]][p];
-        us[p] = x;
-      }
-      double ws[T];
-      bool bad = false;
-#pragma unroll
-      for (int j = 0; j < T; ++j) {
-        ws[j] = M::rate_k(j, us, kf, tb.gdata);
-        bad = bad || bad_rate(ws[j]);
-      }
-      const int src = (int)(c - c0) + ev_depth;  // lane holding draw c + depth
-      const double E = __shfl_sync(0xffffffffu, nE, src);
-      const double R2 = __shfl_sync(0xffffffffu, r2, src);
-      double lam = ws[0];
-#pragma unroll
-      for (int j = 1; j < T; ++j) lam = lam + ws[j];
-      const double tau = E / lam;
-      const double target = lam * R2;
-      // inversion exactly as fire(): running sum over the positive rates
-      double cum = 0.0;
-      int nsel = -1, last = -1;
-#pragma unroll
-      for (int j = 0; j < T; ++j) {
-        if (nsel < 0 && gt0(ws[j])) {
-          cum = last < 0 ? ws[j] : cum + ws[j];
-          last = j;
-          if (le_nonneg(target, cum)) nsel = j;
-        }
-      }
-      if (nsel < 0) nsel = last;
-      const unsigned pos_mask = __ballot_sync(0xffffffffu, gt0(lam));
-      const unsigned bad_mask = __ballot_sync(0xffffffffu, bad);
-      int L = 0, j = 0;
-      int path[D > 0 ? D : 1];  // sorted transitions fired in this round
-#pragma unroll
-      for (int i = 0; i < D; ++i) path[i] = -1;
-      for (; j < J; ++j) {
-        if (j > 0 && ((bad_mask >> L) & 1u)) {
-          code = SG_ERR_RATE;  // the transition into this state gave a bad rate
-          break;
-        }
-        if (!((pos_mask >> L) & 1u)) {
-          done = true;  // nothing can fire: jump to Tn
-          break;
-        }
-        if (c >= SG_MAX_DRAWS) {
-          code = SG_ERR_STEP_LIMIT;
-          break;
-        }
-        const double tauL = __shfl_sync(0xffffffffu, tau, L);
-        const int n = __shfl_sync(0xffffffffu, nsel, L);
-        ++c;
-        const double tt = t + tauL;
-        if (order_key(tt) >= Tkey) {
-          done = true;
-          break;
-        }
-        t = tt;
-#pragma unroll
-        for (int p = 0; p < C; ++p) u[p] += tb.S[n][p];
-        ++f;
-        if (j + 1 < J) {
-          // insert n into the sorted path, then find the lane holding it
-          int x = n;
-#pragma unroll
-          for (int i = 0; i < D; ++i) {
-            if (i <= j && path[i] >= 0 && path[i] > x) {
-              const int y = path[i];
-              path[i] = x;
-              x = y;
-            } else if (i == j) {
-              path[i] = x;
-            }
-          }
-          bool match = depth == j + 1;
-#pragma unroll
-          for (int i = 0; i < D; ++i) match = match && a[i] == path[i];
-          L = __ffs(__ballot_sync(0xffffffffu, match)) - 1;
-        }
-      }
-      if (!done && code == 0) {
-        // j == J: a new window starts from the state after J transitions
-#pragma unroll
-        for (int k = 0; k < T; ++k) {
-          w[k] = M::rate_k(k, u, kf, tb.gdata);
-          if (bad_rate(w[k])) code = SG_ERR_RATE;
-        }
-      }
-    }
-    return true;
-  }
-}
-
-// Direct SSA of one heavy node by a whole warp.  The draws depend only on
-// (seed, replicate, node, day, draw index), so lane l computes the Philox
-// words, uniforms and logarithm of draw c0 + l for 32 draws at once; the
-// sequential part (waiting time, boundary test, transition) then runs on all
-// lanes in step, reading draw j from lane j.  The transition for a draw is
-// evaluated alongside the waiting-time division and kept only if the draw
-// falls before Tn.  Same operations, in the same order, as ssa_thread.
-template <int KIND>
-__device__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK> &hs, double Tn,
-                         uint32_t Td, uint32_t k0, uint32_t k1, const SgTables &tb,
-                         unsigned long long &fired, unsigned long long &drawn) {
-  using M = ModelTraits<KIND>;
-  constexpr int C = M::C, T = M::T, NK = M::NK;
-  const int lane = threadIdx.x & 31;
-  int u[C];
-  double kf[NK], w[T];
-#pragma unroll
-  for (int p = 0; p < C; ++p) u[p] = hs.u[p];
-#pragma unroll
-  for (int i = 0; i < NK; ++i) kf[i] = hs.kf[i];
-  double t = hs.t;
-  uint32_t c = hs.c;
-  const uint32_t c_in = c, node = (uint32_t)hs.node;
-  const uint32_t tag = (SG_STREAM_SSA << 24) | (uint32_t)hs.rep;
-  int code = 0;
-#pragma unroll
-  for (int j = 0; j < T; ++j) w[j] = M::rate_k(j, u, kf, tb.gdata);
-  uint32_t c0 = c;
-  double nE = 0.0, r2 = 0.0;
-  bool have = false;
-  unsigned long long f = 0;
-  const long long Tkey = order_key(Tn);
-  if (T == 2 && tb.dep[0] == 3u && tb.dep[1] == 3u) {
-    // Two transitions, every rate recomputed after every transition: the
-    // states reachable within the next J = 7 draws are u + (j - b) S0 + b S1,
-    // 0 <= b <= j < 7 (28 of them).  Lane l = j (j + 1) / 2 + b evaluates
-    // draw c + j at state (j, b): rates, lambda, waiting time, inversion.
-    // The walk then follows the fired transitions through the table, so each
-    // draw costs one addition (t + tau) and a branch.  Rates from scratch
-    // equal the incrementally kept ones (pure functions of the counts).
-    constexpr int J = 7;
-    int lj = 0, lb = 0;
-    {
-      int l = lane < J * (J + 1) / 2 ? lane : 0;
-      while (l > lj) { l -= lj + 1; ++lj; }
-      lb = l;
-    }
-    bool done = false;
-    while (!done && code == 0) {
-      if (!have || c + (uint32_t)J - c0 > 32u) {
-        c0 = c;
-        const U4 x = philox10(U4{c0 + (uint32_t)lane, node, Td, tag}, k0, k1);
-        nE = -log_pos(u01_open(x.x, x.y));
-        r2 = u01_open(x.z, x.w);
-        have = true;
-      }
-      // this lane's state and draw
-      int us[C];
-#pragma unroll
-      for (int p = 0; p < C; ++p) us[p] = u[p] + (lj - lb) * tb.S[0][p] + lb * tb.S[1][p];
-      double ws[T];
-      bool bad = false;
-#pragma unroll
-      for (int j = 0; j < T; ++j) {
-        ws[j] = M::rate_k(j, us, kf, tb.gdata);
-        bad = bad || bad_rate(ws[j]);
-      }
-      const int src = (int)(c - c0) + lj;  // lane holding draw c + lj
-      const double E = __shfl_sync(0xffffffffu, nE, src);
-      const double R2 = __shfl_sync(0xffffffffu, r2, src);
-      const double lam = ws[0] + ws[1];
-      const double tau = E / lam;
-      const double target = lam * R2;
-      const int fire0 = gt0(ws[0]) && le_nonneg(target, ws[0]);
-      // inversion: transition 0 if target <= w0 (w0 > 0), else 1 if w1 > 0,
-      // else the last positive one (w0)
-      const int nsel = fire0 ? 0 : (gt0(ws[1]) ? 1 : 0);
-      const unsigned pos_mask = __ballot_sync(0xffffffffu, gt0(lam));
-      const unsigned bad_mask = __ballot_sync(0xffffffffu, bad);
-      const unsigned n1_mask = __ballot_sync(0xffffffffu, nsel == 1);
-      int j = 0, b = 0;
-      for (; j < J; ++j) {
-        const int L = j * (j + 1) / 2 + b;
-        if (j > 0 && ((bad_mask >> L) & 1u)) {
-          code = SG_ERR_RATE;  // the transition into this state gave a bad rate
-          break;
-        }
-        if (!((pos_mask >> L) & 1u)) {
-          done = true;  // nothing can fire: jump to Tn
-          break;
-        }
-        if (c >= SG_MAX_DRAWS) {
-          code = SG_ERR_STEP_LIMIT;
-          break;
-        }
-        const double tauL = __shfl_sync(0xffffffffu, tau, L);
-        ++c;
-        const double tt = t + tauL;
-        if (order_key(tt) >= Tkey) {
-          done = true;
-          break;
-        }
-        t = tt;
-        b += (int)((n1_mask >> L) & 1u);
-        ++f;
-      }
-      // move to the state reached
-#pragma unroll
-      for (int p = 0; p < C; ++p) u[p] = u[p] + (j - b) * tb.S[0][p] + b * tb.S[1][p];
-      if (!done && code == 0) {
-        // j == J: a new window starts from the state after J transitions
-#pragma unroll
-        for (int k = 0; k < T; ++k) {
-          w[k] = M::rate_k(k, u, kf, tb.gdata);
-          if (bad_rate(w[k])) code = SG_ERR_RATE;
-        }
-      }
-    }
-  } else if (!ssa_window3<KIND>(u, w, kf, t, c, c0, nE, r2, have, f, code, node, Td, tag, k0,
-                                 k1, Tkey, tb) &&
-             !ssa_window<KIND>(u, w, kf, t, c, c0, nE, r2, have, f, code, node, Td, tag, k0,
-                               k1, Tkey, tb)) {
-  for (;;) {
-    double lam = w[0];
-#pragma unroll
-    for (int j = 1; j < T; ++j) lam = lam + w[j];
-    if (!gt0(lam)) break;
+    if (!gt0(lam)) break;  // nothing can fire: jump to Tn
     if (c >= SG_MAX_DRAWS) {
       code = SG_ERR_STEP_LIMIT;
       break;
     }
-    if (!have || c - c0 >= 32u) {
-      c0 = c;
-      const U4 x = philox10(U4{c0 + (uint32_t)lane, node, Td, tag}, k0, k1);
-      nE = -log_pos(u01_open(x.x, x.y));
-      r2 = u01_open(x.z, x.w);
-      have = true;
-    }
-    const int jj = (int)(c - c0);
-    const double E = __shfl_sync(0xffffffffu, nE, jj);
-    const double R2 = __shfl_sync(0xffffffffu, r2, jj);
+    if (c == (uint32_t)budget) return SSA_REDO;
+    const U4 x = philox10(U4{c, node, Td, tag}, k0, k1);
     ++c;
-    const double tau = E / lam;
-    int u2[C];
-    double w2[T];
-#pragma unroll
-    for (int p = 0; p < C; ++p) u2[p] = u[p];
-#pragma unroll
-    for (int j = 0; j < T; ++j) w2[j] = w[j];
-    const int rc = fire<KIND>(u2, w2, lam * R2, kf, tb);
+    const double tau = -log_pos(u01_open(x.x, x.y)) / lam;
     const double tt = t + tau;
     if (order_key(tt) >= Tkey) break;
     t = tt;
-#pragma unroll
-    for (int p = 0; p < C; ++p) u[p] = u2[p];
-#pragma unroll
-    for (int j = 0; j < T; ++j) w[j] = w2[j];
+    code = fire<KIND>(u, w, lam * u01_open(x.z, x.w), kf, tb);
     ++f;
-    if (rc) {
-      code = rc;
+  }
+#pragma unroll
+  for (int p = 0; p < M::C; ++p) u0[p] = u[p];
+  fired += f;
+  drawn += c;
+  return code;
+}
+
+// A unit's day left to a warp, from its start.
+template <int C, int NK>
+struct HeavySlot {
+  double kf[NK];
+  int32_t node, rep, code;
+  int32_t u[C];
+};
+
+// The transition that lambda r2 selects with the rates of the counts u in
+// FP64 (the intervals of sg_filter.cuh did not settle it): -1 if no rate is
+// positive.  w2, w3: the draw's third and fourth Philox words.
+template <int KIND>
+__device__ __forceinline__ int select_exact(const int *u, const double *kf, uint32_t w2,
+                                            uint32_t w3, const SgTables &tb) {
+  using M = ModelTraits<KIND>;
+  double w[M::T], P[M::T];
+#pragma unroll
+  for (int j = 0; j < M::T; ++j) w[j] = M::rate_k(j, u, kf, tb.gdata);
+  rate_prefix<M::T>(w, P, 0);
+  if (!gt0(P[M::T - 1])) return -1;
+  return select_prefix<M::T>(w, P, P[M::T - 1] * u01_open(w2, w3));
+}
+
+// Time within the day in units of 2^-31 of it, rounded outward.  FP64's own
+// rounding of t + tau moves the time by at most half an ulp at |T| + 1 per
+// transition: time_slack(T) units.
+constexpr uint32_t kDayUnits = 1u << 31;
+__device__ __forceinline__ uint32_t time_slack(uint32_t Td) {
+  return ((uint32_t)abs((int)Td) >> 22) + 1u;
+}
+
+// Direct SSA of one unit's whole day in its thread, decided from intervals
+// (sg_filter.cuh): same draws, same transitions and same end as ssa_exact.
+// Returns SSA_DONE with the counts after the day in u, or SSA_REDO (counts
+// unchanged) where an interval does not settle the time of
+// an event or applies no more: the day must then run with exact times.
+// `warp_rate`: with an expected number of transitions (lambda at the day's
+// start) of at least this the thread leaves the unit to a warp (SSA_REDO).
+//
+// Cost: a draw is ~150 instructions, none of them FP64 (the FP64 form of it
+// is 55 FP64 instructions of ~76 issue cycles each).  The random numbers of
+// the next draw do not depend on this one's outcome, so they are computed
+// beside it.  Bound by issue where every lane has a unit (100,000 endemic
+// SISe3 herds x 20 days, 130 M draws: 2.9 ms, in FP64 43.0 ms), elsewhere by
+// the latency of the longest unit (100 SIR nodes x 99 days: 0.23 ms, 1.33 ms).
+constexpr uint32_t kFilterDraws = 1u << 16;  // longer days take exact times
+template <int KIND>
+__device__ __forceinline__ int ssa_filter(int *u, const double *kf, uint32_t node, uint32_t Td,
+                                          uint32_t tag, uint32_t k0, uint32_t k1,
+                                          float warp_rate, const SgTables &tb,
+                                          unsigned long long &fired,
+                                          unsigned long long &drawn) {
+  using M = ModelTraits<KIND>;
+  constexpr int T = M::T;
+  Filter<KIND> F;
+  if (!F.load(u, kf, tb)) return SSA_REDO;
+  const uint32_t slack = time_slack(Td);
+  uint32_t s_lo = 0, s_hi = 0;  // time since the day's start
+  uint32_t d = 0;
+  U4 x = philox10(U4{0u, node, Td, tag}, k0, k1);
+  Itv E = itv_neglog(x.x, x.y);
+  for (;; ++d) {
+    const U4 xn = philox10(U4{d + 1u, node, Td, tag}, k0, k1);
+    const Itv En = itv_neglog(xn.x, xn.y);
+    Itv P[T];
+    const bool good = F.sums(P, tb);
+    const float l_lo = P[T - 1].lo, l_hi = P[T - 1].hi;
+    if (good && l_hi == 0.0f) {  // nothing can fire: jump to Tn
+      drawn += d;
       break;
     }
+    if (!(good && l_lo >= kItvMin && l_hi <= kItvMax) || d >= kFilterDraws ||
+        (d == 0 && l_lo >= warp_rate))
+      return SSA_REDO;
+    // tau = E / lambda
+    const float t_lo = __fmul_rd(E.lo, rcp_lo(l_hi)), t_hi = __fmul_ru(E.hi, rcp_hi(l_lo));
+    const uint32_t n_lo = s_lo + __float2uint_rd(fminf(t_lo, 1.0f) * 0x1.0p31f);
+    const uint32_t n_hi = s_hi + __float2uint_ru(fminf(t_hi, 1.5f) * 0x1.0p31f) + slack;
+    if (n_lo >= kDayUnits) {  // at or after Tn: the draw is discarded
+      drawn += d + 1u;
+      break;
+    }
+    if (n_hi >= kDayUnits) return SSA_REDO;
+    s_lo = n_lo > slack ? n_lo - slack : 0u;
+    s_hi = n_hi;
+    int n = itv_select<T>(P, itv_r2(x.w));
+    if (n < 0) {
+      int v[M::C];
+      F.store(v);
+      n = select_exact<KIND>(v, kf, x.z, x.w, tb);
+      if (n < 0) return SSA_REDO;
+    }
+    F.fire(n, tb);
+    x = xn;
+    E = En;
   }
+  F.store(u);
+  fired += d;  // every draw but the one that passed Tn
+  return SSA_DONE;
+}
+
+// Direct SSA of one unit by a whole warp, with exact times.
+//
+// With the kind's own tables (`fast`): the transitions of up to 32 draws are
+// walked first, selected from intervals (they depend on the draws' r2 and
+// the counts, not on the times), and lane l keeps the counts before draw l;
+// then every lane evaluates its draw in FP64 -- rates, lambda and E / lambda,
+// 32 logarithms and divisions for the price of one -- and the times are
+// added up in order, which tells where the day ends.  A draw walked beyond
+// that is dropped.  Same values as one draw after the other, since the rates
+// are functions of the counts.
+//
+// Otherwise (a caller's own S or G): draw by draw, the rates kept as G says;
+// the lanes only compute 32 draws' random numbers at once.
+template <int KIND>
+__device__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK> &hs, double Tn,
+                         uint32_t Td, uint32_t k0, uint32_t k1, bool fast, const SgTables &tb,
+                         unsigned long long &fired, unsigned long long &drawn) {
+  using M = ModelTraits<KIND>;
+  constexpr int C = M::C, T = M::T, NK = M::NK;
+  constexpr unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  int u[C];
+  double kf[NK];
+#pragma unroll
+  for (int p = 0; p < C; ++p) u[p] = hs.u[p];
+#pragma unroll
+  for (int i = 0; i < NK; ++i) kf[i] = hs.kf[i];
+  double t = Tn - 1.0;
+  uint32_t c = 0;
+  const uint32_t node = (uint32_t)hs.node;
+  const uint32_t tag = (SG_STREAM_SSA << 24) | (uint32_t)hs.rep;
+  int code = 0;
+  unsigned long long f = 0;
+  const long long Tkey = order_key(Tn);
+  Filter<KIND> F;
+  if (fast && F.load(u, kf, tb)) {
+    bool done = false;
+    while (!done && code == 0) {
+      const U4 x = philox10(U4{c + (uint32_t)lane, node, Td, tag}, k0, k1);
+      const double nE = -log_pos(u01_open(x.x, x.y));
+      // walk the transitions; stop early once the day is surely over
+      const float e_lo = itv_neglog(x.x, x.y).lo;
+      float left = (float)(Tn - t) * (1.0f + 0x1.0p-20f);
+      int us[C];
+#pragma unroll
+      for (int p = 0; p < C; ++p) us[p] = u[p];
+      int walked = 0;
+      bool open = true;  // a state after the last walked draw exists
+      while (walked < 32) {
+        Itv P[T];
+        const bool good = F.sums(P, tb) && P[T - 1].lo >= kItvMin && P[T - 1].hi <= kItvMax;
+        const uint32_t w2 = __shfl_sync(full, x.z, walked), w3 = __shfl_sync(full, x.w, walked);
+        const float e = __shfl_sync(full, e_lo, walked);
+        int v[C];
+        F.store(v);
+        if (lane == walked) {
+#pragma unroll
+          for (int p = 0; p < C; ++p) us[p] = v[p];
+        }
+        ++walked;
+        int n = good ? itv_select<T>(P, itv_r2(w3)) : -1;
+        if (n < 0) n = select_exact<KIND>(v, kf, w2, w3, tb);
+        if (good) left -= e * rcp_lo(P[T - 1].hi);
+        if (n < 0 || left < 0.0f) {
+          open = false;
+          break;
+        }
+        F.fire(n, tb);
+      }
+      // lane l < walked: draw c + l exactly
+      double w[T];
+      bool bad = false;
+#pragma unroll
+      for (int j = 0; j < T; ++j) {
+        w[j] = M::rate_k(j, us, kf, tb.gdata);
+        bad = bad || bad_rate(w[j]);
+      }
+      double lam = w[0];
+#pragma unroll
+      for (int j = 1; j < T; ++j) lam = lam + w[j];
+      const double tau = nE / lam;
+      const unsigned pos_mask = __ballot_sync(full, gt0(lam));
+      const unsigned bad_mask = __ballot_sync(full, bad);
+      int l = 0;
+      for (; l < walked; ++l) {
+        if ((bad_mask >> l) & 1u) {
+          code = SG_ERR_RATE;  // the transition into this state gave a bad rate
+          break;
+        }
+        if (!((pos_mask >> l) & 1u)) {
+          done = true;  // nothing can fire: jump to Tn
+          break;
+        }
+        if (c >= SG_MAX_DRAWS) {
+          code = SG_ERR_STEP_LIMIT;
+          break;
+        }
+        const double tt = t + __shfl_sync(full, tau, l);
+        ++c;
+        if (order_key(tt) >= Tkey) {
+          done = true;
+          break;
+        }
+        t = tt;
+        ++f;
+      }
+      if (l < walked || !open) {
+        // the counts before draw l (the last walked one if the walk ended
+        // there although its event still falls into the day)
+        const int src = l < walked ? l : walked - 1;
+#pragma unroll
+        for (int p = 0; p < C; ++p) u[p] = __shfl_sync(full, us[p], src);
+        if (l == walked) {
+          // the event of the last draw, which the walk left out
+          const uint32_t w2 = __shfl_sync(full, x.z, src), w3 = __shfl_sync(full, x.w, src);
+          const int n = select_exact<KIND>(u, kf, w2, w3, tb);
+          F.load(u, kf, tb);
+          F.fire(n, tb);
+          F.store(u);
+        }
+      } else {
+        F.store(u);
+      }
+    }
+  } else {
+    double w[T];
+#pragma unroll
+    for (int j = 0; j < T; ++j) {
+      w[j] = M::rate_k(j, u, kf, tb.gdata);
+      if (bad_rate(w[j])) code = SG_ERR_RATE;
+    }
+    uint32_t c0 = c;
+    double nE = 0.0, r2 = 0.0;
+    bool have = false;
+    while (code == 0) {
+      double lam = w[0];
+#pragma unroll
+      for (int j = 1; j < T; ++j) lam = lam + w[j];
+      if (!gt0(lam)) break;
+      if (c >= SG_MAX_DRAWS) {
+        code = SG_ERR_STEP_LIMIT;
+        break;
+      }
+      if (!have || c - c0 >= 32u) {
+        c0 = c;
+        const U4 x = philox10(U4{c0 + (uint32_t)lane, node, Td, tag}, k0, k1);
+        nE = -log_pos(u01_open(x.x, x.y));
+        r2 = u01_open(x.z, x.w);
+        have = true;
+      }
+      const int jj = (int)(c - c0);
+      const double E = __shfl_sync(full, nE, jj);
+      const double R2 = __shfl_sync(full, r2, jj);
+      ++c;
+      const double tt = t + E / lam;
+      if (order_key(tt) >= Tkey) break;
+      t = tt;
+      code = fire<KIND>(u, w, lam * R2, kf, tb);
+      ++f;
+    }
   }
   __syncwarp();
   if (lane == 0) {
 #pragma unroll
     for (int p = 0; p < C; ++p) hs.u[p] = u[p];
-    hs.c = c;
     hs.code = code;
     fired += f;
-    drawn += c - c_in;
+    drawn += c;
   }
   __syncwarp();
 }
@@ -1613,34 +1384,24 @@ k_days(const SgTables tb, const DayArgs a) {
       if (code) bad_day = Td;
     }
     if (!AEM && live && code == 0 && !emulated) {
-      double kf[NK], w[T];
+      double kf[NK];
       M::prepare(v, tb.gdata, kf);
+      const int r = a.fast ? ssa_filter<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, a.k0,
+                                              a.k1, a.warp_rate, tb, fired, drawn)
+                           : ssa_exact<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, a.k0,
+                                             a.k1, a.heavy_after, tb, fired, drawn);
+      if (r == SSA_REDO) {
+        my = atomicAdd(&s_nheavy, 1);
+        HeavySlot<C, NK> &hs = s_heavy[my];
 #pragma unroll
-      for (int j = 0; j < T; ++j) {
-        w[j] = M::rate_k(j, u, kf, tb.gdata);
-        if (bad_rate(w[j])) code = SG_ERR_RATE;
-      }
-      if (code == 0) {
-        double t = (double)(Td - 1);
-        uint32_t c = 0;
-        const int r = ssa_thread<KIND>(u, w, kf, t, c, Tn, (uint32_t)node, (uint32_t)Td, tag,
-                                       a.k0, a.k1, a.heavy_after, tb, fired);
-        drawn += c;
-        if (r == SSA_HEAVY) {
-          my = atomicAdd(&s_nheavy, 1);
-          HeavySlot<C, NK> &hs = s_heavy[my];
-          hs.t = t;
+        for (int i = 0; i < NK; ++i) hs.kf[i] = kf[i];
+        hs.node = node;
+        hs.rep = grep;
+        hs.code = 0;
 #pragma unroll
-          for (int i = 0; i < NK; ++i) hs.kf[i] = kf[i];
-          hs.c = c;
-          hs.node = node;
-          hs.rep = grep;
-          hs.code = 0;
-#pragma unroll
-          for (int p = 0; p < C; ++p) hs.u[p] = u[p];
-        } else if (r < 0) {
-          code = r;
-        }
+        for (int p = 0; p < C; ++p) hs.u[p] = u[p];
+      } else if (r < 0) {
+        code = r;
       }
       if (code) bad_day = Td;
     }
@@ -1648,7 +1409,7 @@ k_days(const SgTables tb, const DayArgs a) {
     if constexpr (!AEM) {
       const int nh = s_nheavy;
       for (int h = warp; h < nh; h += nwarps)
-        ssa_warp<KIND>(s_heavy[h], Tn, (uint32_t)Td, a.k0, a.k1, tb, fired, drawn);
+        ssa_warp<KIND>(s_heavy[h], Tn, (uint32_t)Td, a.k0, a.k1, a.fast, tb, fired, drawn);
     } else {
       const int nh = min(s_nheavy, kAemSlots);
       for (int h = warp; h < nh; h += nwarps)
@@ -1845,9 +1606,8 @@ k_days(const SgTables tb, const DayArgs a) {
 //      parameters every rate is then +-0 and the post time step leaves phi
 //      at +0, so skipping them changes no bit); the other units get their
 //      rates, and those with lambda > 0 go to a shared list;
-//   2. runs the SSA of the listed units, one thread each (dense lanes), a
-//      unit needing more than heavy_after draws handed to a warp (32 draws'
-//      random numbers at once, as above);
+//   2. runs the SSA of the listed units, one thread each (dense lanes);
+//      days that need exact times go to warps;
 //   3. visits every unit again: its E1 events of the day (per-unit cursor)
 //      and, unless the day's external transfers follow in their own kernel,
 //      the post time step and recording.
@@ -2113,9 +1873,6 @@ k_days_sparse(const SgTables tb, const DayArgs a) {
   const bool has_e1 = a.ev.e1_node_off != nullptr;
   const uint32_t k0 = a.k0, k1 = a.k1;
   unsigned long long rated = 0;  // units whose rates this thread evaluated
-  // a unit whose expected transitions in the day (lambda times one day) reach
-  // this goes to a warp at once
-  const double heavy_rate = (double)max(a.heavy_after, 1);
   unsigned long long fired = 0, drawn = 0, applied = 0;
   pdl_wait();
   if (a.finish_first && a.T_begin >= a.T_end &&
@@ -2252,35 +2009,45 @@ k_days_sparse(const SgTables tb, const DayArgs a) {
           }
           if (code == 0 && !(quiet && quiescent<KIND>(u, v))) {
             ++rated;
-            double kf[NK], w[T];
+            double kf[NK];
             M::prepare(v, tb.gdata, kf);
-            bool bad = false;
+            // lambda: an interval, or (a caller's own tables) its value
+            bool bad = false, fires;
+            float lam;
+            Filter<KIND> F;
+            Itv L[T];
+            if (a.fast && F.load(u, kf, tb) && F.sums(L, tb) && L[T - 1].hi <= kItvMax) {
+              fires = L[T - 1].hi > 0.0f;
+              lam = L[T - 1].lo;
+            } else {
+              double w[T];
 #pragma unroll
-            for (int j = 0; j < T; ++j) {
-              w[j] = M::rate_k(j, u, kf, tb.gdata);
-              bad = bad || bad_rate(w[j]);
+              for (int j = 0; j < T; ++j) {
+                w[j] = M::rate_k(j, u, kf, tb.gdata);
+                bad = bad || bad_rate(w[j]);
+              }
+              double l = w[0];
+#pragma unroll
+              for (int j = 1; j < T; ++j) l = l + w[j];
+              fires = gt0(l);
+              lam = (float)l;
             }
-            double lam = w[0];
-#pragma unroll
-            for (int j = 1; j < T; ++j) lam = lam + w[j];
             if (bad) {
               report(a.err, SG_ERR_RATE, a.rep0 + rep, node, Td, -1);
-            } else if (gt0(lam)) {
+            } else if (fires) {
               atomicOr(&s_actbits[(i - c0) >> 5], 1u << ((i - c0) & 31));
               int slot = kSparseHeavy;
-              if (!(lam < heavy_rate)) slot = atomicAdd(&s_nheavy, 1);
+              if (!(lam < a.warp_rate)) slot = atomicAdd(&s_nheavy, 1);
               if (slot < kSparseHeavy) {
                 HeavySlot<C, NK> &hs = s_heavy[slot];
-                hs.t = (double)(Td - 1);
 #pragma unroll
                 for (int q = 0; q < NK; ++q) hs.kf[q] = kf[q];
-                hs.c = 0;
                 hs.node = node;
                 hs.rep = a.rep0 + rep;
                 hs.code = i;  // the unit, until the warp reports
 #pragma unroll
                 for (int p = 0; p < C; ++p) hs.u[p] = u[p];
-              } else if (lam < 2.0) {
+              } else if (lam < 2.0f) {
                 // the thread list: units expecting two transitions or more
                 // from the front, the others from the back, so that the
                 // longer chains start first
@@ -2296,13 +2063,13 @@ k_days_sparse(const SgTables tb, const DayArgs a) {
       const int n_long = s_nact;
       const int na = n_long + s_nshort;
       const int n_direct = min(s_nheavy, kSparseHeavy);
-      const int list_warps = min(nwarps, (na + 63) >> 6);
+      const int list_warps = min(nwarps, (na + 31) >> 5);
       if (warp >= list_warps) {
         for (int h = warp - list_warps; h < n_direct; h += nwarps - list_warps) {
           HeavySlot<C, NK> &hs = s_heavy[h];
           const long long gid = g0 + hs.code;
           __syncwarp();
-          ssa_warp<KIND>(hs, Tn, (uint32_t)Td, k0, k1, tb, fired, drawn);
+          ssa_warp<KIND>(hs, Tn, (uint32_t)Td, k0, k1, a.fast, tb, fired, drawn);
           if (lane == 0) {
             if (hs.code) report(a.err, hs.code, hs.rep, hs.node, Td, -1);
 #pragma unroll
@@ -2311,153 +2078,45 @@ k_days_sparse(const SgTables tb, const DayArgs a) {
           __syncwarp();
         }
       } else {
-        const long long Tkey = order_key(Tn);
-        bool busy = false, drained = false;
-        long long gid = 0;
-        int rep = 0, node = 0, nb = 0;
-        uint32_t tag = 0, c = 0;
-        int u[C];
-        double kf[NK], w[T];
-        double t = 0.0;
-        // draw buffer shared by the warp: after a refill with k busy lanes,
-        // the busy lane of rank r finds draw cb + j of its unit in lane
-        // r + j k (j < nbuf = 32 / k); bufE / bufR are this lane's entry
-        uint32_t cb = 0;
-        int nbuf = 0, rank = 0, kref = 1;
-        double bufE = 0.0, bufR = 0.0;
-        double P[T];  // prefix sums of w (rate_prefix)
-#pragma unroll
-        for (int j = 0; j < T; ++j) P[j] = 0.0;
-#pragma unroll
-        for (int p = 0; p < C; ++p) u[p] = 0;
-#pragma unroll
-        for (int q = 0; q < NK; ++q) kf[q] = 0.0;
-#pragma unroll
-        for (int j = 0; j < T; ++j) w[j] = 0.0;
         for (;;) {
-          if (!busy && !drained) {
-            const int i = atomicAdd(&s_next, 1);
-            if (i < na) {
-              gid = g0 + c0 + s_act[i < n_long ? i : kSparseChunk - 1 - (i - n_long)];
-              rep = (int)(gid / Nn);
-              node = (int)(gid - (long long)rep * Nn);
-              tag = (SG_STREAM_SSA << 24) | (uint32_t)(a.rep0 + rep);
-              double v[NV > 0 ? NV : 1];
-              v[0] = 0.0;
+          const int li = atomicAdd(&s_next, 1);
+          if (li >= na) break;
+          const long long gid = g0 + c0 + s_act[li < n_long ? li : kSparseChunk - 1 - (li - n_long)];
+          const int rep = (int)(gid / Nn);
+          const int node = (int)(gid - (long long)rep * Nn);
+          const uint32_t tag = (SG_STREAM_SSA << 24) | (uint32_t)(a.rep0 + rep);
+          int u[C];
+          double v[NV > 0 ? NV : 1], kf[NK];
+          v[0] = 0.0;
 #pragma unroll
-              for (int p = 0; p < C; ++p) u[p] = a.u[gid * C + p];
+          for (int p = 0; p < C; ++p) u[p] = a.u[gid * C + p];
 #pragma unroll
-              for (int q = 0; q < NV; ++q) v[q] = a.v[gid * NV + q];
-              M::prepare(v, tb.gdata, kf);
-#pragma unroll
-              for (int j = 0; j < T; ++j) w[j] = M::rate_k(j, u, kf, tb.gdata);
-              rate_prefix<T>(w, P, 0);
-              t = (double)(Td - 1);
-              c = 0;
-              nb = 0;
-              nbuf = 0;
-              busy = true;
-            } else {
-              drained = true;
-            }
-          }
-          const unsigned bm = __ballot_sync(0xffffffffu, busy);
-          if (bm == 0u) break;
-          // a busy lane without its next draw buffered: every lane computes
-          // one draw (Philox, uniforms, logarithm) for the busy lanes, the
-          // draws c .. c + 32 / k - 1 of each, so that in the list's tail one
-          // logarithm sequence of the warp serves several rounds
-          if (__any_sync(0xffffffffu, busy && (nbuf == 0 || c - cb >= (uint32_t)nbuf))) {
-            const int k = __popc(bm);
-            const int per = 32 / k;
-            const int ro = lane % k, jo = lane / k;
-            // the busy lane of rank ro (the ro-th set bit of bm, by halving)
-            uint32_t x = bm;
-            int n = ro, owner = 0;
-#pragma unroll
-            for (int sft = 16; sft > 0; sft >>= 1) {
-              const int cnt = __popc(x & ((1u << sft) - 1u));
-              if (n >= cnt) {
-                n -= cnt;
-                x >>= sft;
-                owner += sft;
-              }
-            }
-            const uint32_t oc = __shfl_sync(0xffffffffu, c, owner);
-            const uint32_t on = (uint32_t)__shfl_sync(0xffffffffu, node, owner);
-            const uint32_t ot = __shfl_sync(0xffffffffu, tag, owner);
-            if (jo < per) {
-              const U4 xr = philox10(U4{oc + (uint32_t)jo, on, (uint32_t)Td, ot}, k0, k1);
-              bufE = -log_pos(u01_open(xr.x, xr.y));
-              bufR = u01_open(xr.z, xr.w);
-            }
-            kref = k;
-            cb = c;
-            nbuf = per;
-            rank = __popc(bm & ((1u << lane) - 1u));
-          }
-          const int src = (rank + (int)(c - cb) * kref) & 31;
-          const double E = __shfl_sync(0xffffffffu, bufE, src);
-          const double R2 = __shfl_sync(0xffffffffu, bufR, src);
-          if (!busy) continue;
-          // one draw: ssa_step's operations and order, with the draw's
-          // random numbers from the buffer and lambda and the inversion's
-          // running sums from the kept prefix sums
-          int r;
-          {
-            const double lam = P[T - 1];
-            if (!gt0(lam)) {
-              r = SSA_DONE;
-            } else if (c >= SG_MAX_DRAWS) {
-              r = SG_ERR_STEP_LIMIT;
-            } else if (nb == a.heavy_after) {
-              r = SSA_HEAVY;
-            } else {
-              ++c;
-              const double tt = t + E / lam;
-              if (order_key(tt) >= Tkey) {
-                r = SSA_DONE;
-              } else {
-                t = tt;
-                const int n = select_prefix<T>(w, P, lam * R2);
-                const int rc = apply_transition<KIND>(u, w, n, kf, tb);
-                rate_prefix<T>(w, P, __ffs(tb.dep[n]) - 1);
-                ++fired;
-                r = rc ? rc : SSA_STEP_FIRED;
-              }
-            }
-          }
-          if (r == SSA_STEP_FIRED) {
-            ++nb;
-            continue;
-          }
-          if (r == SSA_HEAVY) {
+          for (int q = 0; q < NV; ++q) v[q] = a.v[gid * NV + q];
+          M::prepare(v, tb.gdata, kf);
+          int r = a.fast ? ssa_filter<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1,
+                                            __int_as_float(0x7f800000), tb, fired, drawn)
+                         : ssa_exact<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1,
+                                           a.heavy_after, tb, fired, drawn);
+          if (r == SSA_REDO) {
             const int slot = atomicAdd(&s_nheavy, 1);
             if (slot < kSparseHeavy) {
               HeavySlot<C, NK> &hs = s_heavy[slot];
-              hs.t = t;
 #pragma unroll
               for (int q = 0; q < NK; ++q) hs.kf[q] = kf[q];
-              hs.c = c;
               hs.node = node;
               hs.rep = a.rep0 + rep;
               hs.code = (int32_t)(gid - g0);  // the unit, until the warp reports
 #pragma unroll
               for (int p = 0; p < C; ++p) hs.u[p] = u[p];
-              drawn += c;
-              busy = false;
               continue;
             }
-            // no slot left: this lane goes on with its unit (no hand-off)
-            nb = -(1 << 30);
-            continue;
+            // no slot left: this thread runs the day itself
+            r = ssa_exact<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1, -1, tb, fired,
+                                drawn);
           }
-          // done or an error
-          drawn += c;
           if (r < 0) report(a.err, r, a.rep0 + rep, node, Td, -1);
 #pragma unroll
           for (int p = 0; p < C; ++p) a.u[gid * C + p] = u[p];
-          busy = false;
         }
       }
       // a warp with no SSA work left applies the E1 events of day Td of the
@@ -2476,7 +2135,7 @@ k_days_sparse(const SgTables tb, const DayArgs a) {
         HeavySlot<C, NK> &hs = s_heavy[h];
         const long long gid = g0 + hs.code;  // the unit (ssa_warp sets the code)
         __syncwarp();
-        ssa_warp<KIND>(hs, Tn, (uint32_t)Td, k0, k1, tb, fired, drawn);
+        ssa_warp<KIND>(hs, Tn, (uint32_t)Td, k0, k1, a.fast, tb, fired, drawn);
         if (lane == 0) {
           if (hs.code) report(a.err, hs.code, hs.rep, hs.node, Td, -1);
 #pragma unroll

@@ -19,6 +19,7 @@
 #include <nvrtc.h>
 
 #include <cctype>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -212,6 +213,35 @@ std::string code(const Node *n) {
   }
 }
 
+// The same expression on FP32 intervals that enclose the double operands
+// (sg_filter.cuh).
+std::string code_itv(const Node *n) {
+  char buf[96];
+  switch (n->kind) {
+    case Node::NUM: {
+      const float f = (float)n->num;
+      const float lo = (double)f <= n->num ? f : std::nextafterf(f, -INFINITY);
+      const float hi = (double)f >= n->num ? f : std::nextafterf(f, INFINITY);
+      if (!std::isfinite(lo) || !std::isfinite(hi)) return "itv_nan()";
+      std::snprintf(buf, sizeof buf, "Itv{(float)(%a), (float)(%a)}", (double)lo, (double)hi);
+      return buf;
+    }
+    case Node::COMP:
+      return "itv_count(u[" + std::to_string(n->index) + "])";
+    case Node::GD:
+      return "Itv{g_lo[" + std::to_string(n->index) + "], g_hi[" + std::to_string(n->index) + "]}";
+    case Node::NEG:
+      return "itv_neg(" + code_itv(n->a.get()) + ")";
+    default: {
+      const char *f = n->op == '+'   ? "itv_add"
+                      : n->op == '-' ? "itv_sub"
+                      : n->op == '*' ? "itv_mul"
+                                     : "itv_div";
+      return std::string(f) + "(" + code_itv(n->a.get()) + ", " + code_itv(n->b.get()) + ")";
+    }
+  }
+}
+
 // counts of one side ("@" or terms [k*]name joined by '+'); false on error
 bool side(const std::string &text, const std::vector<std::string> &comps, std::vector<int> &cnt,
           std::string &err) {
@@ -297,6 +327,7 @@ int mparse(const char *const *transitions, int n_trans, const char *const *compa
   out.S.assign((size_t)n_comp * n_trans, 0);
   out.G.assign((size_t)n_trans * n_trans, 0);
   out.rate_code.clear();
+  out.rate_itv_code.clear();
   std::vector<std::vector<char>> rd;
   for (int j = 0; j < n_trans; ++j) {
     if (!transitions[j]) return SG_ERR_ARG;
@@ -333,6 +364,7 @@ int mparse(const char *const *transitions, int n_trans, const char *const *compa
     reads(tree.get(), r);
     rd.push_back(r);
     out.rate_code.push_back(code(tree.get()));
+    out.rate_itv_code.push_back(code_itv(tree.get()));
   }
   // G[k, j] = 1 when propensity k reads a compartment transition j changes
   for (int j = 0; j < n_trans; ++j)
@@ -392,7 +424,8 @@ const Nvrtc &nvrtc() {
 
 std::string generic_source(const ParsedModel &pm) {
   std::string s;
-  s += "#include \"sg_common.h\"\n#include \"sg_device.cuh\"\nnamespace sg {\n";
+  s += "#include \"sg_common.h\"\n#include \"sg_device.cuh\"\n#include \"sg_filter.cuh\"\n"
+       "namespace sg {\n";
   s += "template <> struct ModelTraits<SG_GENERIC> {\n";
   s += "  static constexpr int C = " + std::to_string(pm.C) + ", T = " + std::to_string(pm.T) +
        ", NV = 0, NK = 1;\n";
@@ -403,6 +436,11 @@ std::string generic_source(const ParsedModel &pm) {
   for (int j = 0; j < pm.T; ++j)
     s += "      case " + std::to_string(j) + ": return " + pm.rate_code[j] + ";\n";
   s += "    }\n    return 0.0;\n  }\n";
+  s += "  __device__ static __forceinline__ Itv rate_itv(int j, const int *u, const float *g_lo, "
+       "const float *g_hi) {\n    switch (j) {\n";
+  for (int j = 0; j < pm.T; ++j)
+    s += "      case " + std::to_string(j) + ": return " + pm.rate_itv_code[j] + ";\n";
+  s += "    }\n    return itv_nan();\n  }\n";
   s += "  __device__ static __forceinline__ double rate(int j, const int *u, const double *, "
        "const double *g) {\n    return rate_k(j, u, nullptr, g);\n  }\n};\n}  // namespace sg\n";
   s += "#include \"sg_kernels.cuh\"\n";

@@ -18,7 +18,8 @@ namespace sg {
 struct ParsedModel {
   int C = 0, T = 0;
   std::vector<int> S, G;
-  std::vector<std::string> rate_code;
+  std::vector<std::string> rate_code;      // in FP64
+  std::vector<std::string> rate_itv_code;  // on FP32 intervals
 };
 
 // The engine's kernels compiled for one parsed model.
