@@ -615,7 +615,8 @@ extern "C" int sg_model_create_parsed(const char *const *transitions, int32_t n_
   *out = nullptr;
   ParsedModel pm;
   std::string text;
-  int rc = mparse(transitions, n_trans, compartments, n_comp, gdata_names, n_gdata, pm, text);
+  int rc = mparse(transitions, n_trans, compartments, n_comp, gdata_names, gdata, n_gdata, pm,
+                  text);
   if (rc) {
     put_msg(msg, msg_len, text);
     return rc;
@@ -825,8 +826,18 @@ static void launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, si
 // otherwise.
 static int32_t default_npb(long long units) {
   int32_t npb = kDayBlock;
-  while (npb > 16 && (units + npb - 1) / npb < 2 * 152) npb >>= 1;
+  while (npb > 4 && (units + npb - 1) / npb < 2 * 152) npb >>= 1;
   return npb;
+}
+
+// Which days go to a whole warp: those expecting kWarpRate transitions or more
+// in a block with at most kWarpMax of them (a warp is a few times faster than
+// a thread on one long day and ten times slower on 32 of them), or as tuned.
+constexpr float kWarpRate = 16.0f;
+constexpr int kWarpMax = 8;
+static void set_warp_rule(DayArgs &da, int32_t heavy_after) {
+  da.warp_rate = heavy_after >= 0 ? (float)std::max(1, heavy_after) : kWarpRate;
+  da.warp_max = heavy_after >= 0 ? 0x7fffffff : kWarpMax;
 }
 
 template <int KIND>
@@ -1516,7 +1527,7 @@ extern "C" int sg_run(sg_model *m, const int32_t *tspan, int32_t n_tspan, uint64
   da.rep0 = m->rep0;
   da.heavy_after = m->heavy_after >= 0 ? m->heavy_after : 2;
   da.fast = filter_applies(tb) ? 1 : 0;
-  da.warp_rate = m->heavy_after >= 0 ? (float)std::max(1, m->heavy_after) : INFINITY;
+  set_warp_rule(da, m->heavy_after);
   da.npb = m->npb > 0 ? m->npb : default_npb((long long)Nn * n_rep);
   // the sparse-activity schedule (nodes_per_block > kDayBlock) is for the
   // direct method on the built-in kinds with the day / E2 kernel pair;
@@ -1990,7 +2001,7 @@ extern "C" int sg_run_noalloc(const sg_desc *d, const double *d_ldata, const int
       da.slots = 1;
       da.heavy_after = 2;
       da.fast = filter_applies(tb) ? 1 : 0;
-      da.warp_rate = INFINITY;
+      set_warp_rule(da, -1);
       da.npb = default_npb((long long)Nn * n_rep);
       da.emu = nullptr;
       da.T_begin = t0 + 1;

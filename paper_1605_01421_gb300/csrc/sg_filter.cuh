@@ -73,9 +73,6 @@ __device__ __forceinline__ Itv itv_nonneg(double x) {
   return Itv{__uint_as_float(lo), __uint_as_float(lo + 1u)};
 }
 
-__device__ __forceinline__ Itv itv_count(int n) {
-  return Itv{__int2float_rd(n), __int2float_ru(n)};
-}
 __device__ __forceinline__ Itv itv_neg(Itv a) { return Itv{-a.hi, -a.lo}; }
 __device__ __forceinline__ Itv itv_add(Itv a, Itv b) {
   return Itv{__fadd_rd(a.lo, b.lo), __fadd_ru(a.hi, b.hi)};
@@ -83,13 +80,15 @@ __device__ __forceinline__ Itv itv_add(Itv a, Itv b) {
 __device__ __forceinline__ Itv itv_sub(Itv a, Itv b) {
   return Itv{__fsub_rd(a.lo, b.hi), __fsub_ru(a.hi, b.lo)};
 }
+// a * b, both >= 0
+__device__ __forceinline__ Itv itv_mul_pos(Itv a, Itv b) {
+  return Itv{__fmul_rd(a.lo, b.lo), __fmul_ru(a.hi, b.hi)};
+}
 // a * b for an exact b >= 0
 __device__ __forceinline__ Itv itv_scale(Itv a, float b) {
   return Itv{__fmul_rd(a.lo, b), __fmul_ru(a.hi, b)};
 }
 __device__ __forceinline__ Itv itv_mul(Itv a, Itv b) {
-  if (a.lo >= 0.0f && b.lo >= 0.0f)
-    return Itv{__fmul_rd(a.lo, b.lo), __fmul_ru(a.hi, b.hi)};
   if (!(fabsf(a.lo) < kItvMax && fabsf(a.hi) < kItvMax && fabsf(b.lo) < kItvMax &&
         fabsf(b.hi) < kItvMax))
     return itv_nan();  // fminf / fmaxf would drop a NaN product
@@ -99,13 +98,15 @@ __device__ __forceinline__ Itv itv_mul(Itv a, Itv b) {
                          fmaxf(__fmul_ru(a.hi, b.lo), __fmul_ru(a.hi, b.hi)));
   return Itv{lo, hi};
 }
+// 1 / b for b in [kItvMin, kItvMax] or its negative, else NaN
+__device__ __forceinline__ Itv itv_rcp_pos(Itv b) {
+  const Itv r{rcp_lo(b.hi), rcp_hi(b.lo)};
+  return b.lo >= kItvMin && b.hi <= kItvMax ? r : itv_nan();
+}
+__device__ __forceinline__ Itv itv_div_pos(Itv a, Itv b) { return itv_mul_pos(a, itv_rcp_pos(b)); }
 __device__ __forceinline__ Itv itv_div(Itv a, Itv b) {
-  if (b.hi < 0.0f) {
-    a = itv_neg(a);
-    b = itv_neg(b);
-  }
-  if (!(b.lo >= kItvMin && b.hi <= kItvMax)) return itv_nan();
-  return itv_mul(a, Itv{rcp_lo(b.hi), rcp_hi(b.lo)});
+  if (b.hi < 0.0f) return itv_mul(itv_neg(a), itv_rcp_pos(itv_neg(b)));
+  return itv_mul(a, itv_rcp_pos(b));
 }
 
 // The waiting-time numerator E = -log r1 of the draw with Philox words (w0,
@@ -134,118 +135,130 @@ __device__ __forceinline__ Itv itv_r2(uint32_t w3) {
 // The kind's rates as intervals.  load() takes the counts and the day's rate
 // factors (ModelTraits::prepare) and tells whether the intervals apply;
 // sums() gives the running sums of the rates in index order; fire(n) moves
-// the counts by transition n of the kind's own S (the host only sets
+// the counts x by transition n of the kind's own S (the host only sets
 // DayArgs::fast when the model's S and G are the kind's).  Counts of the
 // built-in kinds are kept as FP32: their transitions keep every node's total,
 // so with each count below 2^20 at the start they stay exact.
-template <int KIND> struct Filter;
+//
+// The general form is that of models from transition strings: sums and
+// moves are generated (ModelTraits::sums_itv, move), the parameters' values
+// in them; counts outside 0 .. 2^23 settle nothing.
+template <int KIND> struct Filter {
+  using M = ModelTraits<KIND>;
+  float x[M::C];
+  __device__ __forceinline__ bool load(const int *u, const double *, const SgTables &) {
+    bool in = true;
+#pragma unroll
+    for (int p = 0; p < M::C; ++p) {
+      x[p] = (float)u[p];
+      in = in && (uint32_t)u[p] < (1u << 23);
+    }
+    return in;
+  }
+  __device__ __forceinline__ bool sums(Itv *P, const SgTables &) const {
+    bool good = M::sums_itv(x, P);
+#pragma unroll
+    for (int p = 0; p < M::C; ++p) good = good && x[p] >= 0.0f && x[p] <= 0x1.0p23f;
+    return good;
+  }
+  __device__ __forceinline__ void fire(int n, const SgTables &) { M::move(n, x); }
+};
 
 __device__ __forceinline__ bool small_counts(const int *u, int n) {
   int all = 0;
+#pragma unroll
   for (int p = 0; p < n; ++p) all |= u[p];
   return (uint32_t)all < (1u << 20);
 }
 
 template <> struct Filter<SG_SIR> {
-  float s, i, r;
+  float x[3];
   Itv inv, g0, g1;
   __device__ __forceinline__ bool load(const int *u, const double *, const SgTables &tb) {
-    s = (float)u[0];
-    i = (float)u[1];
-    r = (float)u[2];
-    const float n = s + i + r;  // exact
-    inv = Itv{rcp_lo(fmaxf(n, 1.0f)), rcp_hi(fmaxf(n, 1.0f))};
+#pragma unroll
+    for (int p = 0; p < 3; ++p) x[p] = (float)u[p];
+    const float n = fmaxf(x[0] + x[1] + x[2], 1.0f);  // exact; rates are 0 in an empty node
+    inv = Itv{rcp_lo(n), rcp_hi(n)};
     g0 = Itv{tb.g_lo[0], tb.g_hi[0]};
     g1 = Itv{tb.g_lo[1], tb.g_hi[1]};
     return small_counts(u, 3);
   }
   __device__ __forceinline__ bool sums(Itv *P, const SgTables &) const {
-    P[0] = itv_scale(itv_scale(g0, s), i);
-    P[0] = Itv{__fmul_rd(P[0].lo, inv.lo), __fmul_ru(P[0].hi, inv.hi)};
-    P[1] = itv_add(P[0], itv_scale(g1, i));
+    const Itv w = itv_scale(itv_scale(g0, x[0]), x[1]);
+    P[0] = Itv{__fmul_rd(w.lo, inv.lo), __fmul_ru(w.hi, inv.hi)};
+    P[1] = itv_add(P[0], itv_scale(g1, x[1]));
     return true;
   }
   __device__ __forceinline__ void fire(int n, const SgTables &) {
-    s -= n == 0 ? 1.0f : 0.0f;
-    i += n == 0 ? 1.0f : -1.0f;
-    r += n == 0 ? 0.0f : 1.0f;
-  }
-  __device__ __forceinline__ void store(int *u) const {
-    u[0] = (int)s;
-    u[1] = (int)i;
-    u[2] = (int)r;
+    x[0] -= n == 0 ? 1.0f : 0.0f;
+    x[1] += n == 0 ? 1.0f : -1.0f;
+    x[2] += n == 0 ? 0.0f : 1.0f;
   }
 };
 
-template <> struct Filter<SG_SIS> {
-  float s, i;
-  __device__ __forceinline__ bool load(const int *u, const double *, const SgTables &) {
-    s = (float)u[0];
-    i = (float)u[1];
-    return small_counts(u, 2);
-  }
-  __device__ __forceinline__ bool sums(Itv *P, const SgTables &tb) const {
-    P[0] = itv_scale(itv_scale(Itv{tb.g_lo[0], tb.g_hi[0]}, s), i);
-    P[1] = itv_add(P[0], itv_scale(Itv{tb.g_lo[1], tb.g_hi[1]}, i));
-    return true;
-  }
+// SIS, SISe: S -> I and back.
+struct FilterSI {
+  float x[2];
+  Itv g0, g1;
   __device__ __forceinline__ void fire(int n, const SgTables &) {
     const float d = n == 0 ? 1.0f : -1.0f;
-    s -= d;
-    i += d;
-  }
-  __device__ __forceinline__ void store(int *u) const {
-    u[0] = (int)s;
-    u[1] = (int)i;
+    x[0] -= d;
+    x[1] += d;
   }
 };
 
-template <> struct Filter<SG_SISE> {
-  float s, i;
-  Itv k;
-  __device__ __forceinline__ bool load(const int *u, const double *kf, const SgTables &) {
-    s = (float)u[0];
-    i = (float)u[1];
-    k = itv_nonneg(kf[0]);
+template <> struct Filter<SG_SIS> : FilterSI {
+  __device__ __forceinline__ bool load(const int *u, const double *, const SgTables &tb) {
+    x[0] = (float)u[0];
+    x[1] = (float)u[1];
+    g0 = Itv{tb.g_lo[0], tb.g_hi[0]};
+    g1 = Itv{tb.g_lo[1], tb.g_hi[1]};
     return small_counts(u, 2);
   }
-  __device__ __forceinline__ bool sums(Itv *P, const SgTables &tb) const {
-    P[0] = itv_scale(k, s);
-    P[1] = itv_add(P[0], itv_scale(Itv{tb.g_lo[1], tb.g_hi[1]}, i));
+  __device__ __forceinline__ bool sums(Itv *P, const SgTables &) const {
+    P[0] = itv_scale(itv_scale(g0, x[0]), x[1]);
+    P[1] = itv_add(P[0], itv_scale(g1, x[1]));
     return true;
   }
-  __device__ __forceinline__ void fire(int n, const SgTables &) {
-    const float d = n == 0 ? 1.0f : -1.0f;
-    s -= d;
-    i += d;
+};
+
+template <> struct Filter<SG_SISE> : FilterSI {
+  // g0: upsilon phi of the day
+  __device__ __forceinline__ bool load(const int *u, const double *kf, const SgTables &tb) {
+    x[0] = (float)u[0];
+    x[1] = (float)u[1];
+    g0 = itv_nonneg(kf[0]);
+    g1 = Itv{tb.g_lo[1], tb.g_hi[1]};
+    return small_counts(u, 2);
   }
-  __device__ __forceinline__ void store(int *u) const {
-    u[0] = (int)s;
-    u[1] = (int)i;
+  __device__ __forceinline__ bool sums(Itv *P, const SgTables &) const {
+    P[0] = itv_scale(g0, x[0]);
+    P[1] = itv_add(P[0], itv_scale(g1, x[1]));
+    return true;
   }
 };
 
 template <> struct Filter<SG_SISE_SP> : Filter<SG_SISE> {};
 
 template <> struct Filter<SG_SISE3> {
-  float s[3], i[3];
-  Itv k[3];
-  __device__ __forceinline__ bool load(const int *u, const double *kf, const SgTables &) {
+  float x[6];
+  Itv k[3], g[3];
+  __device__ __forceinline__ bool load(const int *u, const double *kf, const SgTables &tb) {
+#pragma unroll
+    for (int p = 0; p < 6; ++p) x[p] = (float)u[p];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      s[a] = (float)u[2 * a];
-      i[a] = (float)u[2 * a + 1];
       k[a] = itv_nonneg(kf[a]);
+      g[a] = Itv{tb.g_lo[3 + a], tb.g_hi[3 + a]};
     }
     return small_counts(u, 6);
   }
-  __device__ __forceinline__ bool sums(Itv *P, const SgTables &tb) const {
+  __device__ __forceinline__ bool sums(Itv *P, const SgTables &) const {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const Itv w = itv_scale(k[a], s[a]);
+      const Itv w = itv_scale(k[a], x[2 * a]);
       P[2 * a] = a == 0 ? w : itv_add(P[2 * a - 1], w);
-      P[2 * a + 1] =
-          itv_add(P[2 * a], itv_scale(Itv{tb.g_lo[3 + a], tb.g_hi[3 + a]}, i[a]));
+      P[2 * a + 1] = itv_add(P[2 * a], itv_scale(g[a], x[2 * a + 1]));
     }
     return true;
   }
@@ -253,51 +266,10 @@ template <> struct Filter<SG_SISE3> {
     const float d = (n & 1) ? -1.0f : 1.0f;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const float x = (n >> 1) == a ? d : 0.0f;
-      s[a] -= x;
-      i[a] += x;
+      const float y = (n >> 1) == a ? d : 0.0f;
+      x[2 * a] -= y;
+      x[2 * a + 1] += y;
     }
-  }
-  __device__ __forceinline__ void store(int *u) const {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      u[2 * a] = (int)s[a];
-      u[2 * a + 1] = (int)i[a];
-    }
-  }
-};
-
-// Models from transition strings: the generated propensities on intervals
-// (ModelTraits::rate_itv), counts as integers, S from the tables.
-template <> struct Filter<SG_GENERIC> {
-  int u[SG_MAX_COMP];
-  template <int KIND = SG_GENERIC>
-  __device__ __forceinline__ bool load(const int *u0, const double *, const SgTables &) {
-#pragma unroll
-    for (int p = 0; p < ModelTraits<KIND>::C; ++p) u[p] = u0[p];
-    return true;
-  }
-  template <int KIND = SG_GENERIC>
-  __device__ __forceinline__ bool sums(Itv *P, const SgTables &tb) const {
-    using M = ModelTraits<KIND>;
-    bool nonneg = true;
-#pragma unroll
-    for (int j = 0; j < M::T; ++j) {
-      const Itv w = M::rate_itv(j, u, tb.g_lo, tb.g_hi);
-      nonneg = nonneg && w.lo >= 0.0f;
-      P[j] = j == 0 ? w : itv_add(P[j - 1], w);
-    }
-    return nonneg;
-  }
-  template <int KIND = SG_GENERIC>
-  __device__ __forceinline__ void fire(int n, const SgTables &tb) {
-#pragma unroll
-    for (int p = 0; p < ModelTraits<KIND>::C; ++p) u[p] += tb.S[n][p];
-  }
-  template <int KIND = SG_GENERIC>
-  __device__ __forceinline__ void store(int *out) const {
-#pragma unroll
-    for (int p = 0; p < ModelTraits<KIND>::C; ++p) out[p] = u[p];
   }
 };
 

@@ -171,7 +171,8 @@ struct DayArgs {
   // 1: the model's S and G are its kind's own and its parameters finite and
   // not negative, so the intervals of sg_filter.cuh apply
   int32_t fast;
-  float warp_rate;         // expected transitions from which a unit's day goes to a warp
+  float warp_rate;         // expected transitions from which a unit's day goes to a warp,
+  int32_t warp_max;        // if the block has at most this many such units
   int32_t npb;             // nodes per block (<= kDayBlock); the other
                            // threads of the block only serve heavy nodes
   const int32_t *emu;      // [R][Nn][4]: emulated increments of I_1..I_3 and
@@ -554,12 +555,38 @@ __device__ __forceinline__ int select_exact(const int *u, const double *kf, uint
   return select_prefix<M::T>(w, P, P[M::T - 1] * u01_open(w2, w3));
 }
 
-// Time within the day in units of 2^-31 of it, rounded outward.  FP64's own
-// rounding of t + tau moves the time by at most half an ulp at |T| + 1 per
-// transition: time_slack(T) units.
+// Time since the day's start, an interval [lo, hi] in units of 2^-31 of the
+// day, its ends rounded outward and each waiting time cut at one day (so the
+// sums stay below 2^32).  FP64's own rounding of t + tau moves the time by at
+// most half an ulp at |T| + 1 per transition, (|T| + 1) 2^-22 units; drift
+// is that in 2^-6 units, rounded up, and d the number of transitions
+// (at most kFilterDraws, so d * drift < 2^32).
 constexpr uint32_t kDayUnits = 1u << 31;
-__device__ __forceinline__ uint32_t time_slack(uint32_t Td) {
-  return ((uint32_t)abs((int)Td) >> 22) + 1u;
+constexpr uint32_t kFilterDraws = 1u << 16;  // longer days take exact times
+struct DayTime {
+  uint32_t lo = 0, hi = 0, d = 0, drift;
+  __device__ __forceinline__ explicit DayTime(uint32_t Td)
+      : drift((((uint32_t)abs((int)Td) + 1u) >> 16) + 1u) {}
+  __device__ __forceinline__ void add(uint32_t t_lo, uint32_t t_hi) {
+    lo += t_lo;
+    hi += t_hi;
+    ++d;
+  }
+  // t + tau >= Tn certainly
+  __device__ __forceinline__ bool after(uint32_t t_lo) const {
+    return lo + t_lo >= kDayUnits + ((d * drift + 63u) >> 6);
+  }
+  // t + tau < Tn certainly for each of the next n draws, which take at most
+  // t_hi together
+  __device__ __forceinline__ bool before(uint32_t t_hi, uint32_t n) const {
+    return hi + t_hi < kDayUnits - (((d + n) * drift + 63u) >> 6);
+  }
+};
+__device__ __forceinline__ uint32_t day_units_lo(float t) {
+  return __float2uint_rd(fminf(t, 1.0f) * 0x1.0p31f);
+}
+__device__ __forceinline__ uint32_t day_units_hi(float t) {
+  return __float2uint_ru(fminf(t, 1.0f) * 0x1.0p31f);
 }
 
 // Direct SSA of one unit's whole day in its thread, decided from intervals
@@ -567,8 +594,6 @@ __device__ __forceinline__ uint32_t time_slack(uint32_t Td) {
 // Returns SSA_DONE with the counts after the day in u, or SSA_REDO (counts
 // unchanged) where an interval does not settle the time of
 // an event or applies no more: the day must then run with exact times.
-// `warp_rate`: with an expected number of transitions (lambda at the day's
-// start) of at least this the thread leaves the unit to a warp (SSA_REDO).
 //
 // Cost: a draw is ~150 instructions, none of them FP64 (the FP64 form of it
 // is 55 FP64 instructions of ~76 issue cycles each).  The random numbers of
@@ -576,50 +601,44 @@ __device__ __forceinline__ uint32_t time_slack(uint32_t Td) {
 // beside it.  Bound by issue where every lane has a unit (100,000 endemic
 // SISe3 herds x 20 days, 130 M draws: 2.9 ms, in FP64 43.0 ms), elsewhere by
 // the latency of the longest unit (100 SIR nodes x 99 days: 0.23 ms, 1.33 ms).
-constexpr uint32_t kFilterDraws = 1u << 16;  // longer days take exact times
 template <int KIND>
 __device__ __forceinline__ int ssa_filter(int *u, const double *kf, uint32_t node, uint32_t Td,
                                           uint32_t tag, uint32_t k0, uint32_t k1,
-                                          float warp_rate, const SgTables &tb,
-                                          unsigned long long &fired,
+                                          const SgTables &tb, unsigned long long &fired,
                                           unsigned long long &drawn) {
   using M = ModelTraits<KIND>;
   constexpr int T = M::T;
   Filter<KIND> F;
   if (!F.load(u, kf, tb)) return SSA_REDO;
-  const uint32_t slack = time_slack(Td);
-  uint32_t s_lo = 0, s_hi = 0;  // time since the day's start
-  uint32_t d = 0;
+  DayTime t(Td);
   U4 x = philox10(U4{0u, node, Td, tag}, k0, k1);
   Itv E = itv_neglog(x.x, x.y);
-  for (;; ++d) {
-    const U4 xn = philox10(U4{d + 1u, node, Td, tag}, k0, k1);
+  for (;;) {
+    const U4 xn = philox10(U4{t.d + 1u, node, Td, tag}, k0, k1);
     const Itv En = itv_neglog(xn.x, xn.y);
     Itv P[T];
     const bool good = F.sums(P, tb);
     const float l_lo = P[T - 1].lo, l_hi = P[T - 1].hi;
     if (good && l_hi == 0.0f) {  // nothing can fire: jump to Tn
-      drawn += d;
+      drawn += t.d;
       break;
     }
-    if (!(good && l_lo >= kItvMin && l_hi <= kItvMax) || d >= kFilterDraws ||
-        (d == 0 && l_lo >= warp_rate))
+    if (!(good && l_lo >= kItvMin && l_hi <= kItvMax) || t.d >= kFilterDraws)
       return SSA_REDO;
     // tau = E / lambda
-    const float t_lo = __fmul_rd(E.lo, rcp_lo(l_hi)), t_hi = __fmul_ru(E.hi, rcp_hi(l_lo));
-    const uint32_t n_lo = s_lo + __float2uint_rd(fminf(t_lo, 1.0f) * 0x1.0p31f);
-    const uint32_t n_hi = s_hi + __float2uint_ru(fminf(t_hi, 1.5f) * 0x1.0p31f) + slack;
-    if (n_lo >= kDayUnits) {  // at or after Tn: the draw is discarded
-      drawn += d + 1u;
+    const uint32_t t_lo = day_units_lo(__fmul_rd(E.lo, rcp_lo(l_hi)));
+    const uint32_t t_hi = day_units_hi(__fmul_ru(E.hi, rcp_hi(l_lo)));
+    if (t.after(t_lo)) {  // the draw is discarded
+      drawn += t.d + 1u;
       break;
     }
-    if (n_hi >= kDayUnits) return SSA_REDO;
-    s_lo = n_lo > slack ? n_lo - slack : 0u;
-    s_hi = n_hi;
+    if (!t.before(t_hi, 1)) return SSA_REDO;
+    t.add(t_lo, t_hi);
     int n = itv_select<T>(P, itv_r2(x.w));
     if (n < 0) {
       int v[M::C];
-      F.store(v);
+#pragma unroll
+      for (int p = 0; p < M::C; ++p) v[p] = (int)F.x[p];
       n = select_exact<KIND>(v, kf, x.z, x.w, tb);
       if (n < 0) return SSA_REDO;
     }
@@ -627,12 +646,169 @@ __device__ __forceinline__ int ssa_filter(int *u, const double *kf, uint32_t nod
     x = xn;
     E = En;
   }
-  F.store(u);
-  fired += d;  // every draw but the one that passed Tn
+#pragma unroll
+  for (int p = 0; p < M::C; ++p) u[p] = (int)F.x[p];
+  fired += t.d;  // every draw but the one that passed Tn
   return SSA_DONE;
 }
 
-// Direct SSA of one unit by a whole warp, with exact times.
+// Direct SSA of one unit's day by a whole warp, decided from intervals.  The
+// draws depend only on (seed, replicate, node, day, draw index), so lane l
+// holds the random numbers of draw c0 + l.  The states that the next J draws
+// can reach are the counts plus a multiset of at most J - 1 transitions; each
+// lane evaluates one of them at its draw (running sums, waiting time,
+// transition), and the walk then follows the fired transitions through the
+// lanes.  One or two transitions: J = 8, 7 and lane j (j + 1) / 2 + b (b
+// times the second one after j); three to six: J = 3, lanes in order of the
+// root, single transitions and sorted pairs; more: J = 2.
+//
+// Latency bound: a round is one evaluation and J dependent shuffles.  At ten
+// times a thread's instructions it pays for the few units of a block whose
+// day is long (1,000 predator-prey nodes x 30 days, 2,600 draws a node-day:
+// 20 ms, by threads 115 ms; 37,000 SISe3 herds x 365 days: 15 ms, 19 ms).
+template <int T>
+struct Window {
+  static constexpr int J = T == 1 ? 8 : T == 2 ? 7 : T <= 6 ? 3 : 2;
+};
+template <int KIND>
+__device__ __forceinline__ int ssa_window(int *u, const double *kf, uint32_t node, uint32_t Td,
+                                          uint32_t tag, uint32_t k0, uint32_t k1,
+                                          const SgTables &tb, unsigned long long &fired,
+                                          unsigned long long &drawn) {
+  using M = ModelTraits<KIND>;
+  constexpr int C = M::C, T = M::T, J = Window<T>::J;
+  constexpr unsigned full = 0xffffffffu;
+  constexpr int kNone = T, kOpen = T + 1, kBad = T + 2;  // no transition; not settled; no interval
+  const int lane = threadIdx.x & 31;
+  Filter<KIND> F;
+  if (!F.load(u, kf, tb)) return SSA_REDO;
+  // this lane's multiset: its size and what it adds to the counts
+  int depth = 0;
+  float add[C];
+  {
+    int m0 = -1, m1 = -1, n0 = 0, n1 = 0;  // n0 times m0 and n1 times m1
+    if (T <= 2) {
+      int l = lane < (T == 1 ? J : J * (J + 1) / 2) ? lane : 0;
+      if (T == 1) {
+        depth = n0 = l;
+      } else {
+        while (l > depth) l -= ++depth;
+        n1 = l;
+        n0 = depth - l;
+      }
+      m0 = 0;
+      m1 = T - 1;
+    } else if (lane >= 1 && lane <= T) {
+      depth = n0 = 1;
+      m0 = lane - 1;
+    } else if (J == 3 && lane > T && lane < 1 + T + T * (T + 1) / 2) {
+      depth = 2;
+      n0 = n1 = 1;
+      int l = lane - 1 - T;
+      m0 = 0;
+      while (l >= T - m0) l -= T - m0++;
+      m1 = m0 + l;
+    }
+#pragma unroll
+    for (int p = 0; p < C; ++p) {
+      int y = 0;
+      if (m0 >= 0 && n0) y += n0 * tb.S[m0][p];
+      if (m1 >= 0 && n1) y += n1 * tb.S[m1][p];
+      add[p] = (float)y;
+    }
+  }
+  DayTime t(Td);
+  uint32_t c0 = 0, w2 = 0, w3 = 0;
+  float e_lo = 0.0f, e_hi = 0.0f;
+  bool have = false;
+  for (;;) {
+    if (!have || t.d + (uint32_t)J - c0 > 32u) {
+      if (t.d >= kFilterDraws) return SSA_REDO;
+      c0 = t.d;
+      const U4 x = philox10(U4{c0 + (uint32_t)lane, node, Td, tag}, k0, k1);
+      const Itv E = itv_neglog(x.x, x.y);
+      e_lo = E.lo;
+      e_hi = E.hi;
+      w2 = x.z;
+      w3 = x.w;
+      have = true;
+    }
+    Filter<KIND> G = F;
+#pragma unroll
+    for (int p = 0; p < C; ++p) G.x[p] += add[p];
+    const int src = (int)(t.d - c0) + depth;
+    const float El = __shfl_sync(full, e_lo, src), Eh = __shfl_sync(full, e_hi, src);
+    const uint32_t r = __shfl_sync(full, w3, src);
+    Itv P[T];
+    const bool good = G.sums(P, tb);
+    const float l_lo = P[T - 1].lo, l_hi = P[T - 1].hi;
+    // the waiting time
+    const uint32_t t_lo = day_units_lo(__fmul_rd(El, rcp_lo(l_hi)));
+    const uint32_t t_hi = day_units_hi(__fmul_ru(Eh, rcp_hi(l_lo)));
+    int n = itv_select<T>(P, itv_r2(r));
+    if (n < 0) n = kOpen;
+    if (!(good && l_lo >= kItvMin && l_hi <= kItvMax)) n = good && l_hi == 0.0f ? kNone : kBad;
+    // the lanes of the states on the way, and what their draws add up to
+    int m[J], L = 0, b = 0;
+    uint32_t a_lo[J], a_hi[J], sum_hi = 0;
+    bool all = true;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      m[j] = __shfl_sync(full, n, L);
+      a_lo[j] = __shfl_sync(full, t_lo, L);
+      a_hi[j] = __shfl_sync(full, t_hi, L);
+      all = all && m[j] < kNone;
+      if (T <= 2) {
+        b += T == 2 ? m[j] : 0;
+        L = T == 1 ? j + 1 : ((j + 1) * (j + 2) / 2 + b) & 31;
+      } else if (j == 0) {
+        L = (1 + m[0]) & 31;
+      } else if (j == 1) {
+        const int lo = min(m[0], m[1]), hi = max(m[0], m[1]);
+        L = (1 + T + lo * T - lo * (lo - 1) / 2 + (hi - lo)) & 31;
+      }
+      sum_hi = min(sum_hi + a_hi[j], kDayUnits - 1u);
+    }
+    if (all && t.before(sum_hi, J)) {  // every one of them falls into the day
+#pragma unroll
+      for (int j = 0; j < J; ++j) {
+        t.add(a_lo[j], a_hi[j]);
+        F.fire(m[j], tb);
+      }
+      continue;
+    }
+    // otherwise one draw at a time; after a draw that the intervals do not
+    // settle, a new round
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      if (m[j] == kBad) return SSA_REDO;
+      if (m[j] == kNone || t.after(a_lo[j])) {
+        drawn += m[j] == kNone ? t.d : t.d + 1u;
+        fired += t.d;
+#pragma unroll
+        for (int p = 0; p < C; ++p) u[p] = (int)F.x[p];
+        return SSA_DONE;
+      }
+      if (!t.before(a_hi[j], 1)) return SSA_REDO;
+      const bool open = m[j] == kOpen;
+      if (open) {
+        int v[C];
+#pragma unroll
+        for (int p = 0; p < C; ++p) v[p] = (int)F.x[p];
+        const uint32_t x2 = __shfl_sync(full, w2, (int)(t.d - c0));
+        const uint32_t x3 = __shfl_sync(full, w3, (int)(t.d - c0));
+        m[j] = select_exact<KIND>(v, kf, x2, x3, tb);
+        if (m[j] < 0) return SSA_REDO;
+      }
+      t.add(a_lo[j], a_hi[j]);
+      F.fire(m[j], tb);
+      if (open) break;
+    }
+  }
+}
+
+// Direct SSA of one unit by a whole warp: from intervals (ssa_window), and
+// where they leave an event's time open, with exact times.
 //
 // With the kind's own tables (`fast`): the transitions of up to 32 draws are
 // walked first, selected from intervals (they depend on the draws' r2 and
@@ -646,7 +822,7 @@ __device__ __forceinline__ int ssa_filter(int *u, const double *kf, uint32_t nod
 // Otherwise (a caller's own S or G): draw by draw, the rates kept as G says;
 // the lanes only compute 32 draws' random numbers at once.
 template <int KIND>
-__device__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK> &hs, double Tn,
+__device__ __noinline__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK> &hs, double Tn,
                          uint32_t Td, uint32_t k0, uint32_t k1, bool fast, const SgTables &tb,
                          unsigned long long &fired, unsigned long long &drawn) {
   using M = ModelTraits<KIND>;
@@ -664,8 +840,20 @@ __device__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK> 
   const uint32_t node = (uint32_t)hs.node;
   const uint32_t tag = (SG_STREAM_SSA << 24) | (uint32_t)hs.rep;
   int code = 0;
-  unsigned long long f = 0;
+  unsigned long long f = 0, wf = 0, wd = 0;
   const long long Tkey = order_key(Tn);
+  if (fast && ssa_window<KIND>(u, kf, node, Td, tag, k0, k1, tb, wf, wd) == SSA_DONE) {
+    __syncwarp();
+    if (lane == 0) {
+#pragma unroll
+      for (int p = 0; p < C; ++p) hs.u[p] = u[p];
+      hs.code = 0;
+      fired += wf;
+      drawn += wd;
+    }
+    __syncwarp();
+    return;
+  }
   Filter<KIND> F;
   if (fast && F.load(u, kf, tb)) {
     bool done = false;
@@ -686,7 +874,8 @@ __device__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK> 
         const uint32_t w2 = __shfl_sync(full, x.z, walked), w3 = __shfl_sync(full, x.w, walked);
         const float e = __shfl_sync(full, e_lo, walked);
         int v[C];
-        F.store(v);
+#pragma unroll
+        for (int p = 0; p < C; ++p) v[p] = (int)F.x[p];
         if (lane == walked) {
 #pragma unroll
           for (int p = 0; p < C; ++p) us[p] = v[p];
@@ -750,10 +939,12 @@ __device__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK> 
           const int n = select_exact<KIND>(u, kf, w2, w3, tb);
           F.load(u, kf, tb);
           F.fire(n, tb);
-          F.store(u);
+#pragma unroll
+          for (int p = 0; p < C; ++p) u[p] = (int)F.x[p];
         }
       } else {
-        F.store(u);
+#pragma unroll
+        for (int p = 0; p < C; ++p) u[p] = (int)F.x[p];
       }
     }
   } else {
@@ -1231,7 +1422,7 @@ __device__ __forceinline__ int finish_step(int Tf, const int *u, double *v, cons
 // (unless a kernel boundary follows) the post time step and recording.
 template <int KIND, bool AEM>
 __global__ void __launch_bounds__(kDayBlock)
-k_days(const SgTables tb, const DayArgs a) {
+k_days(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
   using M = ModelTraits<KIND>;
   constexpr int C = M::C, T = M::T, NV = M::NV, NK = M::NK;
   __shared__ HeavySlot<C, NK> s_heavy[AEM ? 1 : kDayBlock];
@@ -1383,15 +1574,11 @@ k_days(const SgTables tb, const DayArgs a) {
       }
       if (code) bad_day = Td;
     }
-    if (!AEM && live && code == 0 && !emulated) {
+    if constexpr (!AEM) {
+      const bool ssa = live && code == 0 && !emulated;
       double kf[NK];
-      M::prepare(v, tb.gdata, kf);
-      const int r = a.fast ? ssa_filter<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, a.k0,
-                                              a.k1, a.warp_rate, tb, fired, drawn)
-                           : ssa_exact<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, a.k0,
-                                             a.k1, a.heavy_after, tb, fired, drawn);
-      if (r == SSA_REDO) {
-        my = atomicAdd(&s_nheavy, 1);
+      if (ssa) M::prepare(v, tb.gdata, kf);
+      auto to_slot = [&]() {
         HeavySlot<C, NK> &hs = s_heavy[my];
 #pragma unroll
         for (int i = 0; i < NK; ++i) hs.kf[i] = kf[i];
@@ -1400,16 +1587,40 @@ k_days(const SgTables tb, const DayArgs a) {
         hs.code = 0;
 #pragma unroll
         for (int p = 0; p < C; ++p) hs.u[p] = u[p];
-      } else if (r < 0) {
-        code = r;
+      };
+      if (a.fast && ssa) {
+        // a long day goes to a warp if the block has few of them
+        Filter<KIND> F;
+        Itv L[T];
+        if (F.load(u, kf, tb) && F.sums(L, tb) && L[T - 1].lo >= a.warp_rate) {
+          my = atomicAdd(&s_nheavy, 1);
+          to_slot();
+        }
       }
-      if (code) bad_day = Td;
+      __syncthreads();
+      const bool own = s_nheavy > a.warp_max;
+      __syncthreads();
+      if (ssa && (my < 0 || own)) {
+        const int r = a.fast ? ssa_filter<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, a.k0,
+                                                a.k1, tb, fired, drawn)
+                             : ssa_exact<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, a.k0,
+                                               a.k1, a.heavy_after, tb, fired, drawn);
+        if (r == SSA_REDO) {
+          if (my < 0) my = atomicAdd(&s_nheavy, 1);
+          to_slot();
+        } else {
+          if (my >= 0) s_heavy[my].rep = -1;  // done
+          my = -1;
+          if (r < 0) code = r;
+        }
+      }
+      if (ssa && code) bad_day = Td;
     }
     __syncthreads();
     if constexpr (!AEM) {
       const int nh = s_nheavy;
       for (int h = warp; h < nh; h += nwarps)
-        ssa_warp<KIND>(s_heavy[h], Tn, (uint32_t)Td, a.k0, a.k1, a.fast, tb, fired, drawn);
+        if (s_heavy[h].rep >= 0) ssa_warp<KIND>(s_heavy[h], Tn, (uint32_t)Td, a.k0, a.k1, a.fast, tb, fired, drawn);
     } else {
       const int nh = min(s_nheavy, kAemSlots);
       for (int h = warp; h < nh; h += nwarps)
@@ -1853,7 +2064,7 @@ struct UnitPos {
 
 template <int KIND>
 __global__ void __launch_bounds__(kSparseBlock)
-k_days_sparse(const SgTables tb, const DayArgs a) {
+k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
   using M = ModelTraits<KIND>;
   constexpr int C = M::C, T = M::T, NV = M::NV, NK = M::NK;
   // lists of units of the current chunk (indices relative to the chunk)
@@ -2063,8 +2274,13 @@ k_days_sparse(const SgTables tb, const DayArgs a) {
       const int n_long = s_nact;
       const int na = n_long + s_nshort;
       const int n_direct = min(s_nheavy, kSparseHeavy);
-      const int list_warps = min(nwarps, (na + 31) >> 5);
-      if (warp >= list_warps) {
+      // long days go to warps if there are few of them, else to the list's
+      // front
+      const bool own = n_direct > a.warp_max;
+      const int na_all = own ? na + n_direct : na;
+      const int list_warps =
+          min((na_all + 31) >> 5, own ? nwarps : nwarps - min(n_direct, nwarps / 2));
+      if (warp >= list_warps && !own) {
         for (int h = warp - list_warps; h < n_direct; h += nwarps - list_warps) {
           HeavySlot<C, NK> &hs = s_heavy[h];
           const long long gid = g0 + hs.code;
@@ -2079,9 +2295,16 @@ k_days_sparse(const SgTables tb, const DayArgs a) {
         }
       } else {
         for (;;) {
-          const int li = atomicAdd(&s_next, 1);
-          if (li >= na) break;
-          const long long gid = g0 + c0 + s_act[li < n_long ? li : kSparseChunk - 1 - (li - n_long)];
+          int li = atomicAdd(&s_next, 1);
+          if (li >= na_all) break;
+          int slot = -1;
+          if (own) {
+            if (li < n_direct) slot = li;
+            li -= n_direct;
+          }
+          const long long gid =
+              slot >= 0 ? g0 + s_heavy[slot].code
+                        : g0 + c0 + s_act[li < n_long ? li : kSparseChunk - 1 - (li - n_long)];
           const int rep = (int)(gid / Nn);
           const int node = (int)(gid - (long long)rep * Nn);
           const uint32_t tag = (SG_STREAM_SSA << 24) | (uint32_t)(a.rep0 + rep);
@@ -2094,11 +2317,11 @@ k_days_sparse(const SgTables tb, const DayArgs a) {
           for (int q = 0; q < NV; ++q) v[q] = a.v[gid * NV + q];
           M::prepare(v, tb.gdata, kf);
           int r = a.fast ? ssa_filter<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1,
-                                            __int_as_float(0x7f800000), tb, fired, drawn)
+                                            tb, fired, drawn)
                          : ssa_exact<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1,
                                            a.heavy_after, tb, fired, drawn);
           if (r == SSA_REDO) {
-            const int slot = atomicAdd(&s_nheavy, 1);
+            if (slot < 0) slot = atomicAdd(&s_nheavy, 1);
             if (slot < kSparseHeavy) {
               HeavySlot<C, NK> &hs = s_heavy[slot];
 #pragma unroll
@@ -2114,6 +2337,7 @@ k_days_sparse(const SgTables tb, const DayArgs a) {
             r = ssa_exact<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1, -1, tb, fired,
                                 drawn);
           }
+          if (slot >= 0 && slot < kSparseHeavy) s_heavy[slot].rep = -1;  // done
           if (r < 0) report(a.err, r, a.rep0 + rep, node, Td, -1);
 #pragma unroll
           for (int p = 0; p < C; ++p) a.u[gid * C + p] = u[p];
@@ -2129,10 +2353,11 @@ k_days_sparse(const SgTables tb, const DayArgs a) {
       __syncthreads();
       // the warp slots not run yet: all of them when every warp had list
       // units, else those the thread list handed over
-      const int h0 = list_warps < nwarps ? n_direct : 0;
+      const int h0 = list_warps < nwarps && !own ? n_direct : 0;
       const int nh = min(s_nheavy, kSparseHeavy);
       for (int h = h0 + warp; h < nh; h += nwarps) {
         HeavySlot<C, NK> &hs = s_heavy[h];
+        if (hs.rep < 0) continue;
         const long long gid = g0 + hs.code;  // the unit (ssa_warp sets the code)
         __syncwarp();
         ssa_warp<KIND>(hs, Tn, (uint32_t)Td, k0, k1, a.fast, tb, fired, drawn);

@@ -196,50 +196,96 @@ void reads(const Node *n, std::vector<char> &acc) {
   reads(n->b.get(), acc);
 }
 
-std::string code(const Node *n) {
+std::string lit(double x) {
   char buf[64];
+  std::snprintf(buf, sizeof buf, "(%a)", x);
+  return buf;
+}
+
+// The FP64 expression over u; global data as literals (the model's own, so
+// that constant parts fold: each is the same IEEE operation at compile time).
+std::string code(const Node *n, const double *gd) {
   switch (n->kind) {
     case Node::NUM:
-      std::snprintf(buf, sizeof buf, "(%a)", n->num);
-      return buf;
+      return lit(n->num);
     case Node::COMP:
       return "i2d(u[" + std::to_string(n->index) + "])";
     case Node::GD:
-      return "g[" + std::to_string(n->index) + "]";
+      return std::isfinite(gd[n->index]) ? lit(gd[n->index])
+                                         : "g[" + std::to_string(n->index) + "]";
     case Node::NEG:
-      return "(-" + code(n->a.get()) + ")";
+      return "(-" + code(n->a.get(), gd) + ")";
     default:
-      return "(" + code(n->a.get()) + " " + n->op + " " + code(n->b.get()) + ")";
+      return "(" + code(n->a.get(), gd) + " " + n->op + " " + code(n->b.get(), gd) + ")";
   }
 }
 
-// The same expression on FP32 intervals that enclose the double operands
-// (sg_filter.cuh).
-std::string code_itv(const Node *n) {
-  char buf[96];
-  switch (n->kind) {
-    case Node::NUM: {
-      const float f = (float)n->num;
-      const float lo = (double)f <= n->num ? f : std::nextafterf(f, -INFINITY);
-      const float hi = (double)f >= n->num ? f : std::nextafterf(f, INFINITY);
-      if (!std::isfinite(lo) || !std::isfinite(hi)) return "itv_nan()";
-      std::snprintf(buf, sizeof buf, "Itv{(float)(%a), (float)(%a)}", (double)lo, (double)hi);
-      return buf;
-    }
-    case Node::COMP:
-      return "itv_count(u[" + std::to_string(n->index) + "])";
-    case Node::GD:
-      return "Itv{g_lo[" + std::to_string(n->index) + "], g_hi[" + std::to_string(n->index) + "]}";
-    case Node::NEG:
-      return "itv_neg(" + code_itv(n->a.get()) + ")";
-    default: {
-      const char *f = n->op == '+'   ? "itv_add"
-                      : n->op == '-' ? "itv_sub"
-                      : n->op == '*' ? "itv_mul"
-                                     : "itv_div";
-      return std::string(f) + "(" + code_itv(n->a.get()) + ", " + code_itv(n->b.get()) + ")";
-    }
+// The same expression on FP32 intervals that enclose its FP64 value
+// (sg_filter.cuh).  Subexpressions of constants are evaluated here in FP64
+// (with the very operations of the propensity) and become constant
+// intervals; counts x[] are exact and not negative, and products of factors
+// known not to be negative take the two-instruction form.
+struct ItvCode {
+  std::string text;
+  bool constant = false, count = false, nonneg = false;
+  double value = 0.0;  // of a constant
+};
+
+ItvCode code_itv(const Node *n, const double *gd) {
+  auto constant = [](double x) {
+    ItvCode r;
+    r.constant = true;
+    r.value = x;
+    r.nonneg = x >= 0.0;
+    const float f = (float)x;
+    const float lo = (double)f <= x ? f : std::nextafterf(f, -INFINITY);
+    const float hi = (double)f >= x ? f : std::nextafterf(f, INFINITY);
+    if (std::isfinite(lo) && std::isfinite(hi))
+      r.text = "Itv{(float)" + lit(lo) + ", (float)" + lit(hi) + "}";
+    else
+      r.text = "itv_nan()";
+    return r;
+  };
+  if (n->kind == Node::NUM) return constant(n->num);
+  if (n->kind == Node::GD) return constant(gd[n->index]);
+  ItvCode r;
+  if (n->kind == Node::COMP) {
+    r.text = "x[" + std::to_string(n->index) + "]";
+    r.count = r.nonneg = true;
+    return r;
   }
+  auto itv = [](const ItvCode &c) { return c.count ? "Itv{" + c.text + ", " + c.text + "}" : c.text; };
+  const ItvCode a = code_itv(n->a.get(), gd);
+  if (n->kind == Node::NEG) {
+    if (a.constant) return constant(-a.value);
+    r.text = "itv_neg(" + itv(a) + ")";
+    return r;
+  }
+  const ItvCode b = code_itv(n->b.get(), gd);
+  if (a.constant && b.constant) {
+    const volatile double x = a.value, y = b.value;
+    return constant(n->op == '+' ? x + y : n->op == '-' ? x - y : n->op == '*' ? x * y : x / y);
+  }
+  const bool pos = a.nonneg && b.nonneg;
+  switch (n->op) {
+    case '+':
+      r.text = "itv_add(" + itv(a) + ", " + itv(b) + ")";
+      r.nonneg = pos;
+      break;
+    case '-':
+      r.text = "itv_sub(" + itv(a) + ", " + itv(b) + ")";
+      break;
+    case '*':
+      r.text = b.count   ? "itv_scale(" + itv(a) + ", " + b.text + ")"
+               : a.count ? "itv_scale(" + itv(b) + ", " + a.text + ")"
+                         : (pos ? "itv_mul_pos(" : "itv_mul(") + itv(a) + ", " + itv(b) + ")";
+      r.nonneg = pos;
+      break;
+    default:
+      r.text = (pos ? "itv_div_pos(" : "itv_div(") + itv(a) + ", " + itv(b) + ")";
+      r.nonneg = pos;
+  }
+  return r;
 }
 
 // counts of one side ("@" or terms [k*]name joined by '+'); false on error
@@ -294,11 +340,11 @@ bool side(const std::string &text, const std::vector<std::string> &comps, std::v
 }  // namespace
 
 int mparse(const char *const *transitions, int n_trans, const char *const *compartments,
-           int n_comp, const char *const *gdata_names, int n_gdata, ParsedModel &out,
-           std::string &err) {
+           int n_comp, const char *const *gdata_names, const double *gdata, int n_gdata,
+           ParsedModel &out, std::string &err) {
   if (n_trans < 1 || n_trans > SG_MAX_TRANS || n_comp < 1 || n_comp > SG_MAX_COMP ||
       n_gdata < 0 || n_gdata > SG_MAX_GDATA || !transitions || !compartments ||
-      (n_gdata > 0 && !gdata_names)) {
+      (n_gdata > 0 && (!gdata_names || !gdata))) {
     err = "sizes out of range";
     return SG_ERR_ARG;
   }
@@ -363,8 +409,9 @@ int mparse(const char *const *transitions, int n_trans, const char *const *compa
     std::vector<char> r(n_comp, 0);
     reads(tree.get(), r);
     rd.push_back(r);
-    out.rate_code.push_back(code(tree.get()));
-    out.rate_itv_code.push_back(code_itv(tree.get()));
+    out.rate_code.push_back(code(tree.get(), gdata));
+    const ItvCode c = code_itv(tree.get(), gdata);
+    out.rate_itv_code.push_back(c.count ? "Itv{" + c.text + ", " + c.text + "}" : c.text);
   }
   // G[k, j] = 1 when propensity k reads a compartment transition j changes
   for (int j = 0; j < n_trans; ++j)
@@ -436,11 +483,24 @@ std::string generic_source(const ParsedModel &pm) {
   for (int j = 0; j < pm.T; ++j)
     s += "      case " + std::to_string(j) + ": return " + pm.rate_code[j] + ";\n";
   s += "    }\n    return 0.0;\n  }\n";
-  s += "  __device__ static __forceinline__ Itv rate_itv(int j, const int *u, const float *g_lo, "
-       "const float *g_hi) {\n    switch (j) {\n";
-  for (int j = 0; j < pm.T; ++j)
-    s += "      case " + std::to_string(j) + ": return " + pm.rate_itv_code[j] + ";\n";
-  s += "    }\n    return itv_nan();\n  }\n";
+  // running sums of the propensities' intervals (false: one may be negative)
+  s += "  __device__ static __forceinline__ bool sums_itv(const float *x, Itv *P) {\n"
+       "    bool good = true;\n";
+  for (int j = 0; j < pm.T; ++j) {
+    const std::string k = std::to_string(j);
+    s += "    { const Itv w = " + pm.rate_itv_code[j] + "; good = good && w.lo >= 0.0f; P[" + k +
+         "] = " + (j ? "itv_add(P[" + std::to_string(j - 1) + "], w)" : "w") + "; }\n";
+  }
+  s += "    return good;\n  }\n";
+  s += "  __device__ static __forceinline__ void move(int n, float *x) {\n";
+  for (int p = 0; p < pm.C; ++p) {
+    std::string d = "0.0f";
+    for (int j = 0; j < pm.T; ++j)
+      if (const int v = pm.S[(size_t)j * pm.C + p])
+        d = "(n == " + std::to_string(j) + " ? " + std::to_string(v) + ".0f : " + d + ")";
+    s += "    x[" + std::to_string(p) + "] += " + d + ";\n";
+  }
+  s += "  }\n";
   s += "  __device__ static __forceinline__ double rate(int j, const int *u, const double *, "
        "const double *g) {\n    return rate_k(j, u, nullptr, g);\n  }\n};\n}  // namespace sg\n";
   s += "#include \"sg_kernels.cuh\"\n";

@@ -32,8 +32,8 @@ struct JitKernels {
 
 // Returns SG_OK, SG_ERR_ARG or SG_ERR_PARSE (message in err).
 int mparse(const char *const *transitions, int n_trans, const char *const *compartments,
-           int n_comp, const char *const *gdata_names, int n_gdata, ParsedModel &out,
-           std::string &err);
+           int n_comp, const char *const *gdata_names, const double *gdata, int n_gdata,
+           ParsedModel &out, std::string &err);
 // The CUDA source of ModelTraits<SG_GENERIC> plus the kernel headers.
 std::string generic_source(const ParsedModel &pm);
 // Compiles with NVRTC for sm_103a and loads on the current device.  Returns
