@@ -554,6 +554,16 @@ int sg_absmax_bf16(const void *x, int64_t n, float *out, void *stream);
  * d loss / d logits / B as BF16 (leading dimension ldd; columns 387.. are 0). */
 int sg_mlp_ce_loss(const float *logits, int32_t ldl, const int32_t *targets, int32_t B,
                    void *dlogits, int32_t ldd, double *loss_sum, void *stream);
+/* Mean cross-entropy gradients of the network over B rows (a multiple of 8)
+ * in one call: forward pass, loss, backward pass.  feat: B x 16 BF16;
+ * targets: B x 3 int32; W[l], b[l] (l < 4): BF16 weights (out x in) and FP32
+ * biases; dW[l], db[l]: FP32 gradients (out); *loss_sum (device double): the
+ * summed loss (out).  scratch: at least sg_mlp_gradients_scratch(B) bytes on
+ * the device, 256-byte aligned. */
+int64_t sg_mlp_gradients_scratch(int32_t B);
+int sg_mlp_gradients(const void *feat, const int32_t *targets, int32_t B, const void *const *W,
+                     const float *const *b, float *const *dW, float *const *db,
+                     double *loss_sum, void *scratch, int64_t scratch_bytes, void *stream);
 /* dpre[i] = dpost[i] * GELU'(pre[i]) (tanh form; BF16 out), n elements. */
 int sg_gelu_backward(const float *dpost, const float *pre, int64_t n, void *dpre, void *stream);
 /* dst (cols x rows) = src (rows x cols) transposed, BF16. */

@@ -171,7 +171,8 @@ EXPORTS = ["sg_model_create", "sg_set_events", "sg_run", "sg_run_host",
            "sg_run_noalloc", "sg_set_tuning", "sg_autotune", "sg_set_graphs",
            "sg_gemm_bf16", "sg_mlp_ce_loss", "sg_gelu_backward", "sg_transpose_bf16",
            "sg_colsum_bf16", "sg_adam_step", "sg_emu_features", "sg_emu_targets",
-           "sg_emu_sample", "sg_emulator_set", "sg_set_neighbors", "sg_set_solver",
+           "sg_emu_sample", "sg_mlp_gradients", "sg_mlp_gradients_scratch",
+           "sg_emulator_set", "sg_set_neighbors", "sg_set_solver",
            "sg_set_output", "sg_model_create_parsed", "sg_model_tables",
            "sg_set_fused_events", "sg_set_persistent", "sg_gemm_fp8", "sg_quant_fp8_rows",
            "sg_quant_fp8_bf16", "sg_absmax_bf16", "sg_emulator_set_fp8", "sg_gemm_bf16_to_fp8",
@@ -253,6 +254,11 @@ def lib(path: str | None = None):
         L.sg_gemm_bf16.restype = ctypes.c_int
         f32, f64 = ctypes.c_float, ctypes.c_double
         L.sg_mlp_ce_loss.argtypes = [vp, i32, vp, i32, vp, i32, vp, vp]
+        pp = ctypes.POINTER(vp)
+        L.sg_mlp_gradients.argtypes = [vp, vp, i32, pp, pp, pp, pp, vp, vp, i64, vp]
+        L.sg_mlp_gradients.restype = ctypes.c_int
+        L.sg_mlp_gradients_scratch.argtypes = [i32]
+        L.sg_mlp_gradients_scratch.restype = i64
         L.sg_gelu_backward.argtypes = [vp, vp, i64, vp, vp]
         L.sg_transpose_bf16.argtypes = [vp, i32, i32, vp, vp]
         L.sg_colsum_bf16.argtypes = [vp, i32, i32, vp, vp]

@@ -90,24 +90,33 @@ __device__ __forceinline__ uint4 pack_e4m3_16(const float *y) {
 // same 32 bytes), and the accumulator is scaled by a_scale * b_scale[n].
 // Optional outputs: FP32 before the activation, BF16 after it, FP8 E4M3
 // after it (scaled by c8_inv_scale, saturated to the finite range).
+//
+// Up to NBUF stages are in flight (a stage's copies take longer than its
+// MMAs, and with K = 8,192 rows of a training batch there are 128 of them).
+// A long chain is bound by the copies an SM keeps in flight, ~24 KB a
+// microsecond (more or larger stages changed nothing).
+//
+// Training epilogues: with bwd_pre the value is multiplied by GELU's
+// derivative at bwd_pre (the gradient through an activation), and C16T takes
+// a transposed copy of C16 (32 consecutive rows per store of a warp).
 constexpr int kGemmThreads = 256;
-template <int BN, bool F8>
-__global__ void __launch_bounds__(kGemmThreads) k_gemm_tc(const GemmArgs g) {
+__device__ __forceinline__ float gelu_grad(float x);
+
+template <int BN, bool F8, int NBUF>
+__device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr int kStageK = F8 ? 2 * kBK : kBK;    // elements of K per stage
   constexpr uint32_t kAStage = kBM * kBK * 2;  // 16 KB (128 bytes per row)
   constexpr uint32_t kBStage = BN * kBK * 2;
-  unsigned char *sA[2] = {smem, smem + kAStage};
-  unsigned char *sB[2] = {smem + 2 * kAStage, smem + 2 * kAStage + kBStage};
-  __shared__ __align__(8) uint64_t bar[2];
+  auto sA = [&](int b) { return smem + (uint32_t)b * kAStage; };
+  auto sB = [&](int b) { return smem + NBUF * kAStage + (uint32_t)b * kBStage; };
+  __shared__ __align__(8) uint64_t bar[NBUF];
   __shared__ uint32_t tmem_slot;
   __shared__ int s_fail;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * BN;
   if (tid == 0) {
-    tc::mbar_init(&bar[0], 1);
-    tc::mbar_init(&bar[1], 1);
+    for (int b = 0; b < NBUF; ++b) tc::mbar_init(&bar[b], 1);
     tc::fence_mbar_init();
     s_fail = 0;
   }
@@ -118,51 +127,69 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_tc(const GemmArgs g) {
   const uint32_t tmem = tmem_slot;
   constexpr uint32_t idesc = F8 ? tc::idesc_e4m3_f32(kBM, BN) : tc::idesc_bf16_f32(kBM, BN);
   const int stages = (g.K + kStageK - 1) / kStageK;
-  uint32_t uses[2] = {0, 0};
   bool ok = true;
 
   // Stage loader: every thread issues its 16-byte asynchronous copies
-  // (cp.async) for stage s into buffer s & 1, rows past M / N and columns
-  // past K are zero-filled.
+  // (cp.async) for stage s into buffer s mod NBUF, rows past M / N and
+  // columns past K are zero-filled.  A warp copies 8 rows x 4 chunks: whole
+  // 32-byte sectors of each row, 512 consecutive bytes of shared memory.
+  // Each thread's rows are fixed, so their addresses are formed once.
+  constexpr int kChunk = F8 ? 16 : 8;            // elements per 16-byte chunk
+  constexpr int kWarps = kGemmThreads / 32;
+  constexpr int kNA = kBM / 4 / kWarps, kNB = BN / 4 / kWarps;
+  const int K = g.K, rl = lane & 7, kl = lane >> 3;
+  const char *pa[kNA], *pb[kNB];
+  bool ia[kNA], ib[kNB];
+  const char *Abase = F8 ? (const char *)g.A8 : (const char *)g.A;
+  const char *Bbase = F8 ? (const char *)g.B8 : (const char *)g.Bt;
+  auto row_of = [&](int i) { return ((warp + i * kWarps) >> 1) * 8 + rl; };
+  auto chunk_of = [&](int i) { return ((warp + i * kWarps) & 1) * 4 + kl; };
+#pragma unroll
+  for (int i = 0; i < kNA; ++i) {
+    const int m = m0 + row_of(i);
+    ia[i] = m < g.M;
+    pa[i] = Abase + ((long long)(ia[i] ? m : 0) * g.lda + chunk_of(i) * kChunk) * (F8 ? 1 : 2);
+  }
+#pragma unroll
+  for (int i = 0; i < kNB; ++i) {
+    const int n = n0 + row_of(i);
+    ib[i] = n < g.N;
+    pb[i] = Bbase + ((long long)(ib[i] ? n : 0) * g.ldb + chunk_of(i) * kChunk) * (F8 ? 1 : 2);
+  }
   auto load_stage = [&](int s) {
-    const int b = s & 1, k0 = s * kStageK;
-    constexpr int kChunk = F8 ? 16 : 8;  // elements per 16-byte chunk
-    const uint32_t a0 = tc::smem_u32(sA[b]), b0 = tc::smem_u32(sB[b]);
-    for (int idx = tid; idx < kBM * 8; idx += kGemmThreads) {
-      const int r = idx >> 3, kg = idx & 7;
-      const int m = m0 + r, k = k0 + kg * kChunk;
-      const bool in = m < g.M && k < g.K;
-      const void *src;
-      if constexpr (F8)
-        src = in ? (const void *)(g.A8 + (long long)m * g.lda + k) : (const void *)g.A8;
-      else
-        src = in ? (const void *)(g.A + (long long)m * g.lda + k) : (const void *)g.A;
-      cp_async16(a0 + stage_off(r, kg), src, in ? 16 : 0);
+    const int b = s % NBUF;
+    const uint32_t a0 = tc::smem_u32(sA(b)), b0 = tc::smem_u32(sB(b));
+    const long long off = (long long)s * 128;  // a stage is 128 bytes of a row
+#pragma unroll
+    for (int i = 0; i < kNA; ++i) {
+      const bool in = ia[i] && s * kStageK + chunk_of(i) * kChunk < K;
+      cp_async16(a0 + stage_off(row_of(i), chunk_of(i)), in ? pa[i] + off : Abase, in ? 16 : 0);
     }
-    for (int idx = tid; idx < BN * 8; idx += kGemmThreads) {
-      const int r = idx >> 3, kg = idx & 7;
-      const int n = n0 + r, k = k0 + kg * kChunk;
-      const bool in = n < g.N && k < g.K;
-      const void *src;
-      if constexpr (F8)
-        src = in ? (const void *)(g.B8 + (long long)n * g.ldb + k) : (const void *)g.B8;
-      else
-        src = in ? (const void *)(g.Bt + (long long)n * g.ldb + k) : (const void *)g.Bt;
-      cp_async16(b0 + stage_off(r, kg), src, in ? 16 : 0);
+#pragma unroll
+    for (int i = 0; i < kNB; ++i) {
+      const bool in = ib[i] && s * kStageK + chunk_of(i) * kChunk < K;
+      cp_async16(b0 + stage_off(row_of(i), chunk_of(i)), in ? pb[i] + off : Bbase, in ? 16 : 0);
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
 
-  if (stages > 0) load_stage(0);
-  for (int s = 0; s < stages && ok; ++s) {
-    const int b = s & 1;
+  for (int s = 0; s < NBUF - 1; ++s) {
+    if (s < stages) load_stage(s);
+    commit();  // one group per stage, also where there is none
+  }
+  for (int s = 0; s < stages; ++s) {
+    const int b = s % NBUF;
     // stage s has landed in shared memory
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    asm volatile("cp.async.wait_group %0;" ::"n"(NBUF - 2) : "memory");
     tc::fence_async_smem();
     __syncthreads();
+    if (s_fail) {
+      ok = false;
+      break;
+    }
     if (tid == 0) {
       tc::tc_fence_after();
-      const uint32_t a0 = tc::smem_u32(sA[b]), b0 = tc::smem_u32(sB[b]);
+      const uint32_t a0 = tc::smem_u32(sA(b)), b0 = tc::smem_u32(sB(b));
 #pragma unroll
       for (int kk = 0; kk < kBK / 16; ++kk) {
         // two core matrices along K per MMA: +256 bytes per K step of 16
@@ -175,31 +202,31 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_tc(const GemmArgs g) {
       }
       tc::mma_commit(&bar[b]);
     }
-    ++uses[b];
-    if (s + 1 < stages) {
-      // the other buffer is free once the MMAs of stage s - 1 are done; its
-      // loads then overlap the MMAs of stage s
-      const int nb = (s + 1) & 1;
-      if (uses[nb] > 0 && !tc::mbar_wait(&bar[nb], (uses[nb] - 1) & 1, kWaitLimit)) s_fail = 1;
-      __syncthreads();
-      if (s_fail) {
-        ok = false;
-        break;
-      }
-      load_stage(s + 1);
+    // the buffer of stage s + NBUF - 1 is free once the MMAs of stage s - 1
+    // are done; its loads overlap those of the stages between
+    const int nx = s + NBUF - 1;
+    if (nx < stages) {
+      if (s > 0 &&
+          !tc::mbar_wait(&bar[(s - 1) % NBUF], ((s - 1) / NBUF) & 1, kWaitLimit))
+        s_fail = 1;
+      else
+        load_stage(nx);
     }
+    commit();
   }
   // all MMAs done: the last stage's commit completes after every earlier one
   if (ok && stages > 0) {
-    const int b = (stages - 1) & 1;
-    if (!tc::mbar_wait(&bar[b], (uses[b] - 1) & 1, kWaitLimit)) ok = false;
+    const int l = stages - 1;
+    if (!tc::mbar_wait(&bar[l % NBUF], (l / NBUF) & 1, kWaitLimit)) ok = false;
   }
   if (!ok) {
     if (tid == 0) atomicExch(g.err, SG_ERR_TIMEOUT);
-    // let MMAs still in flight finish (bounded) before the TMEM is freed
-    for (int b = 0; b < 2; ++b)
-      if (uses[b]) tc::mbar_wait(&bar[b], (uses[b] - 1) & 1, kWaitLimit);
-  } else {
+    // copies and MMAs still in flight end (bounded) before the memory is freed
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    for (int l = max(0, stages - NBUF); l < stages; ++l)
+      tc::mbar_wait(&bar[l % NBUF], (l / NBUF) & 1, 1u << 16);
+  }
+  if (ok) {
     // Epilogue.  Warp w reads TMEM lanes 32 (w % 4) .. + 31 (tile rows) and
     // the columns of half w / 4.  FP32 results go out as 16-byte vectors;
     // BF16 results are staged in shared memory (the stage buffers are free
@@ -249,8 +276,32 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_tc(const GemmArgs g) {
       }
       if (g.C16) {
         float y[16];
+        if (g.bwd_pre) {
+          const float *pre = g.bwd_pre + (long long)row * g.N + nb;
+          if (row < g.M && nb + 16 <= g.N && (((uintptr_t)pre) & 15) == 0) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) y[i] = g.act == 1 ? gelu_scaled(v[i], 0.5f) : v[i];
+            for (int i = 0; i < 16; i += 4) {
+              const float4 p4 = __ldg(reinterpret_cast<const float4 *>(pre + i));
+              y[i] = v[i] * gelu_grad(p4.x);
+              y[i + 1] = v[i + 1] * gelu_grad(p4.y);
+              y[i + 2] = v[i + 2] * gelu_grad(p4.z);
+              y[i + 3] = v[i + 3] * gelu_grad(p4.w);
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              y[i] = row < g.M && nb + i < g.N ? v[i] * gelu_grad(pre[i]) : 0.0f;
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) y[i] = g.act == 1 ? gelu_scaled(v[i], 0.5f) : v[i];
+        }
+        if (g.C16T && row < g.M) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (nb + i < g.N)
+              g.C16T[(long long)(nb + i) * g.ldc16t + row] = __float2bfloat16_rn(y[i]);
+        }
         uint32_t packed[8];
 #pragma unroll
         for (int i = 0; i < 16; i += 2) {
@@ -304,6 +355,31 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_tc(const GemmArgs g) {
   if (warp == 0) tc::tmem_dealloc(tmem, BN);
 }
 
+template <int BN, bool F8, int NBUF>
+__global__ void __launch_bounds__(kGemmThreads) k_gemm_tc(const __grid_constant__ GemmArgs g) {
+  gemm_tile<BN, F8, NBUF>(g, blockIdx.x * kBM, blockIdx.y * BN);
+}
+
+// Up to four contractions in one launch, for a training step's weight
+// gradients: (256..392) x (16..256) outputs with K = the batch are a few
+// tiles each, bound by their chain of stages (128 for 8,192 rows), so the
+// chains run side by side: 126 us for the four, 1,260 us one after the other
+// in 128 x 256 tiles.  Bit for bit the result of one at a time (a split K
+// would not be).
+constexpr int kGroupBN = 64, kGroupBuf = 6;
+struct GemmGroup {
+  GemmArgs g[4];
+  int n, first[5];  // tiles of contraction i: first[i] .. first[i + 1] - 1
+};
+__global__ void __launch_bounds__(kGemmThreads)
+k_gemm_group(const __grid_constant__ GemmGroup q) {
+  int i = 0;
+  while (i + 1 < q.n && (int)blockIdx.x >= q.first[i + 1]) ++i;
+  const GemmArgs g = q.g[i];
+  const int t = (int)blockIdx.x - q.first[i], nt = (g.N + kGroupBN - 1) / kGroupBN;
+  gemm_tile<kGroupBN, false, kGroupBuf>(g, (t / nt) * kBM, (t % nt) * kGroupBN);
+}
+
 std::mutex g_err_mu;
 int *g_err_buf[64] = {};
 
@@ -325,19 +401,52 @@ int gemm_err_buf(int **out) {
   return SG_OK;
 }
 
-template <int BN, bool F8>
-void launch_gemm(const GemmArgs &g, cudaStream_t st) {
-  const size_t smem = 2 * ((size_t)kBM * kBK * 2 + (size_t)BN * kBK * 2);
-  static unsigned long long attr_set = 0;
+// Opts a kernel into `smem` bytes of dynamic shared memory, once per device.
+template <typename K>
+void allow_smem(K *kernel, size_t smem, unsigned long long &done) {
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev < 64 && !((attr_set >> dev) & 1ull)) {
-    cudaFuncSetAttribute(k_gemm_tc<BN, F8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    attr_set |= 1ull << dev;
+  if (dev < 64 && !((done >> dev) & 1ull)) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    done |= 1ull << dev;
   }
+}
+
+constexpr size_t gemm_smem(int bn, int nbuf) {
+  return nbuf * ((size_t)kBM * kBK * 2 + (size_t)bn * kBK * 2);
+}
+
+template <int BN, bool F8, int NBUF>
+void launch_gemm(const GemmArgs &g, cudaStream_t st) {
+  static unsigned long long attr_set = 0;
+  allow_smem(k_gemm_tc<BN, F8, NBUF>, gemm_smem(BN, NBUF), attr_set);
   const dim3 grid((unsigned)((g.M + kBM - 1) / kBM), (unsigned)((g.N + BN - 1) / BN));
-  k_gemm_tc<BN, F8><<<grid, kGemmThreads, smem, st>>>(g);
+  k_gemm_tc<BN, F8, NBUF><<<grid, kGemmThreads, gemm_smem(BN, NBUF), st>>>(g);
+}
+
+// The widest tile that still gives every SM one, else the narrowest (8,192 x
+// 256 x 256 in 64 wide tiles: 20-28 us, most SMs idle).
+constexpr int kGemmSms = 152;
+template <bool F8>
+void launch_gemm_tiles(const GemmArgs &g, cudaStream_t st) {
+  const long long mt = (g.M + kBM - 1) / kBM;
+  auto tiles = [&](int bn) { return mt * ((g.N + bn - 1) / bn); };
+  if (g.N > 128 && tiles(256) >= kGemmSms)
+    launch_gemm<256, F8, 2>(g, st);
+  else if (g.N > 64 && tiles(128) >= kGemmSms)
+    launch_gemm<128, F8, 3>(g, st);
+  else
+    launch_gemm<64, F8, 4>(g, st);
+}
+
+void launch_gemm_group(GemmGroup &q, cudaStream_t st) {
+  q.first[0] = 0;
+  for (int i = 0; i < q.n; ++i)
+    q.first[i + 1] = q.first[i] + (q.g[i].M + kBM - 1) / kBM *
+                                      ((q.g[i].N + kGroupBN - 1) / kGroupBN);
+  static unsigned long long attr_set = 0;
+  allow_smem(k_gemm_group, gemm_smem(kGroupBN, kGroupBuf), attr_set);
+  k_gemm_group<<<q.first[q.n], kGemmThreads, gemm_smem(kGroupBN, kGroupBuf), st>>>(q);
 }
 
 }  // namespace
@@ -360,21 +469,10 @@ int gemm_bf16(const GemmArgs &g0, cudaStream_t st) {
     int rc = gemm_err_buf(&g.err);
     if (rc) return rc;
   }
-  if (f8) {
-    if (g.N <= 64)
-      launch_gemm<64, true>(g, st);
-    else if (g.N <= 128)
-      launch_gemm<128, true>(g, st);
-    else
-      launch_gemm<256, true>(g, st);
-  } else {
-    if (g.N <= 64)
-      launch_gemm<64, false>(g, st);
-    else if (g.N <= 128)
-      launch_gemm<128, false>(g, st);
-    else
-      launch_gemm<256, false>(g, st);
-  }
+  if (f8)
+    launch_gemm_tiles<true>(g, st);
+  else
+    launch_gemm_tiles<false>(g, st);
   return SG_OK;
 }
 
@@ -501,36 +599,60 @@ __device__ __forceinline__ float gelu_grad(float x) {
 }
 
 // Cross-entropy over the three 129-way heads, one warp per row: loss and
-// d loss / d logits (scaled by 1 / B, BF16; padding columns get 0).
-__global__ void k_ce_loss(const float *__restrict__ logits, int ldl,
-                          const int32_t *__restrict__ tgt, int B, __nv_bfloat16 *dlog, int ldd,
-                          int ncols_grad, double *loss_sum) {
+// d loss / d logits (scaled by 1 / B, BF16; padding columns get 0).  Each
+// head's logits are read once into registers; the block's losses go out in
+// one atomic (8,192 rows x 392: one atomic per row took most of 24 us).
+__global__ void __launch_bounds__(256)
+k_ce_loss(const float *__restrict__ logits, int ldl, const int32_t *__restrict__ tgt, int B,
+          __nv_bfloat16 *dlog, int ldd, int ncols_grad, double *loss_sum) {
+  __shared__ double s_loss[8];
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= B) return;
-  const float *row = logits + (long long)warp * ldl;
-  __nv_bfloat16 *grow = dlog + (long long)warp * ldd;
-  const float invB = 1.0f / (float)B;
+  constexpr int kPer = (kBins + 31) / 32;
   float loss = 0.0f;
-  for (int h = 0; h < kHeads; ++h) {
-    const float *lg = row + h * kBins;
-    float mx = -INFINITY;
-    for (int c = lane; c < kBins; c += 32) mx = fmaxf(mx, lg[c]);
+  if (warp < B) {
+    const float *row = logits + (long long)warp * ldl;
+    __nv_bfloat16 *grow = dlog + (long long)warp * ldd;
+    const float invB = 1.0f / (float)B;
+    float x[kHeads][kPer];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    float se = 0.0f;
-    for (int c = lane; c < kBins; c += 32) se += expf(lg[c] - mx);
+    for (int h = 0; h < kHeads; ++h)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
-    const float lz = mx + logf(se);
-    const int t = tgt[(long long)warp * kHeads + h];
-    if (lane == 0) loss += lz - lg[t];
-    for (int c = lane; c < kBins; c += 32) {
-      const float p = expf(lg[c] - lz) - (c == t ? 1.0f : 0.0f);
-      grow[h * kBins + c] = __float2bfloat16_rn(p * invB);
+      for (int i = 0; i < kPer; ++i)
+        x[h][i] = lane + 32 * i < kBins ? row[h * kBins + lane + 32 * i] : -INFINITY;
+#pragma unroll
+    for (int h = 0; h < kHeads; ++h) {
+      float mx = -INFINITY;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) mx = fmaxf(mx, x[h][i]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      float se = 0.0f;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i)
+        if (lane + 32 * i < kBins) se += expf(x[h][i] - mx);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
+      const float lz = mx + logf(se);
+      const int t = tgt[(long long)warp * kHeads + h];
+      if (lane == 0) loss += lz - row[h * kBins + t];
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const int c = lane + 32 * i;
+        if (c >= kBins) continue;
+        const float p = expf(x[h][i] - lz) - (c == t ? 1.0f : 0.0f);
+        grow[h * kBins + c] = __float2bfloat16_rn(p * invB);
+      }
     }
+    for (int c = kHeads * kBins + lane; c < ncols_grad; c += 32)
+      grow[c] = __float2bfloat16_rn(0.0f);
   }
-  for (int c = kHeads * kBins + lane; c < ncols_grad; c += 32) grow[c] = __float2bfloat16_rn(0.0f);
-  if (lane == 0) atomicAdd(loss_sum, (double)loss);
+  if (lane == 0) s_loss[threadIdx.x >> 5] = (double)loss;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double sum = 0.0;
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) sum += s_loss[i];
+    atomicAdd(loss_sum, sum);
+  }
 }
 
 __global__ void k_gelu_bwd(const float *__restrict__ dpost, const float *__restrict__ pre,
@@ -1294,6 +1416,217 @@ extern "C" int sg_colsum_bf16(const void *src, int32_t rows, int32_t cols, float
   cudaStream_t st = (cudaStream_t)stream;
   if (cols) k_colsum<<<(cols + 127) / 128, 128, 0, st>>>((const __nv_bfloat16 *)src, rows, cols, out);
   return finish(st);
+}
+
+namespace {
+
+// Up to four transposes in one launch (blockIdx.z picks one), 64 x 64 tiles.
+struct TransposeJobs {
+  const __nv_bfloat16 *src[4];
+  __nv_bfloat16 *dst[4];
+  int rows[4], cols[4];
+};
+__global__ void __launch_bounds__(256) k_transpose_jobs(const TransposeJobs t) {
+  __shared__ __nv_bfloat16 tile[64][66];
+  const int z = blockIdx.z, rows = t.rows[z], cols = t.cols[z];
+  const int r0 = blockIdx.x * 64, c0 = blockIdx.y * 64;
+  if (r0 >= rows || c0 >= cols) return;
+  // every dimension here is a multiple of 8: pairs along both, 4 bytes each
+  const int tx = (threadIdx.x & 31) * 2, ty = threadIdx.x >> 5;
+#pragma unroll
+  for (int i = 0; i < 64; i += 8) {
+    const int r = i + ty;
+    if (r0 + r < rows && c0 + tx < cols) {
+      const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162 *>(
+          t.src[z] + (long long)(r0 + r) * cols + c0 + tx);
+      tile[r][tx] = v.x;
+      tile[r][tx + 1] = v.y;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 64; i += 8) {
+    const int c = i + ty;
+    if (c0 + c < cols && r0 + tx < rows)
+      *reinterpret_cast<__nv_bfloat162 *>(t.dst[z] + (long long)(c0 + c) * rows + r0 + tx) =
+          __halves2bfloat162(tile[tx][c], tile[tx + 1][c]);
+  }
+}
+
+// Sums of the rows (length n) of up to four matrices, one block per row: the
+// bias gradients from the transposed deltas.
+struct RowsumJobs {
+  const __nv_bfloat16 *src[4];
+  float *dst[4];
+  int rows[4];
+};
+__global__ void __launch_bounds__(256) k_rowsum_jobs(const RowsumJobs t, int n) {
+  __shared__ float s_sum[8];
+  int r = blockIdx.x, z = 0;
+  while (z < 3 && r >= t.rows[z]) r -= t.rows[z++];
+  const __nv_bfloat16 *x = t.src[z] + (long long)r * n;
+  float sum = 0.0f;
+  if ((n & 7) == 0) {
+    for (int i = threadIdx.x * 8; i < n; i += 256 * 8) {
+      const uint4 v = *reinterpret_cast<const uint4 *>(x + i);
+      const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float2 f = __bfloat1622float2(h[k]);
+        sum += f.x;
+        sum += f.y;
+      }
+    }
+  } else {
+    for (int i = threadIdx.x; i < n; i += 256) sum += __bfloat162float(x[i]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float v = 0.0f;
+    for (int i = 0; i < 8; ++i) v += s_sum[i];
+    t.dst[z][r] = v;
+  }
+}
+
+constexpr int kLayerOut[4] = {kEmuHidden, kEmuHidden, kEmuHidden, kEmuOut};
+constexpr int kLayerIn[4] = {kEmuIn, kEmuHidden, kEmuHidden, kEmuHidden};
+
+// Scratch of one gradient pass over B rows, every part 256-byte aligned.
+struct GradScratch {
+  float *logits, *pre[3];
+  __nv_bfloat16 *act[3], *in_t[4], *delta[4], *delta_t[4], *w_t[4];
+  size_t bytes;
+  GradScratch(unsigned char *base, size_t B) {
+    size_t off = 0;
+    auto place = [&](size_t n) {
+      unsigned char *p = base + off;
+      off += (n + 255) & ~(size_t)255;
+      return p;
+    };
+    logits = (float *)place(B * kEmuOut * 4);
+    for (int l = 0; l < 3; ++l) {
+      pre[l] = (float *)place(B * kEmuHidden * 4);
+      act[l] = (__nv_bfloat16 *)place(B * kEmuHidden * 2);
+    }
+    for (int l = 0; l < 4; ++l) {
+      in_t[l] = (__nv_bfloat16 *)place(B * kLayerIn[l] * 2);
+      delta[l] = (__nv_bfloat16 *)place(B * kLayerOut[l] * 2);
+      delta_t[l] = (__nv_bfloat16 *)place(B * kLayerOut[l] * 2);
+      w_t[l] = (__nv_bfloat16 *)place((size_t)kLayerOut[l] * kLayerIn[l] * 2);
+    }
+    bytes = off;
+  }
+};
+
+}  // namespace
+
+extern "C" int64_t sg_mlp_gradients_scratch(int32_t B) {
+  return B < 0 ? 0 : (int64_t)GradScratch(nullptr, (size_t)B).bytes;
+}
+
+extern "C" int sg_mlp_gradients(const void *feat, const int32_t *targets, int32_t B,
+                                const void *const *W, const float *const *b, float *const *dW,
+                                float *const *db, double *loss_sum, void *scratch,
+                                int64_t scratch_bytes, void *stream) {
+  // rows of the transposed operands are the batch: a multiple of 8 of them
+  if (B < 8 || B % 8 != 0 || !feat || !targets || !W || !b || !dW || !db || !loss_sum ||
+      !scratch || ((uintptr_t)scratch & 255) != 0 ||
+      scratch_bytes < sg_mlp_gradients_scratch(B))
+    return SG_ERR_ARG;
+  for (int l = 0; l < 4; ++l)
+    if (!W[l] || !b[l] || !dW[l] || !db[l]) return SG_ERR_ARG;
+  cudaStream_t st = (cudaStream_t)stream;
+  const GradScratch s((unsigned char *)scratch, (size_t)B);
+  cudaMemsetAsync(loss_sum, 0, sizeof(double), st);
+  // transposes of the features and of the weights that the backward pass reads
+  TransposeJobs t{};
+  t.src[0] = (const __nv_bfloat16 *)feat;
+  t.dst[0] = s.in_t[0];
+  t.rows[0] = B;
+  t.cols[0] = kEmuIn;
+  for (int l = 1; l < 4; ++l) {
+    t.src[l] = (const __nv_bfloat16 *)W[l];
+    t.dst[l] = s.w_t[l];
+    t.rows[l] = kLayerOut[l];
+    t.cols[l] = kLayerIn[l];
+  }
+  k_transpose_jobs<<<dim3((unsigned)((std::max(B, kEmuOut) + 63) / 64), 4, 4), 256, 0, st>>>(t);
+  GemmGroup q{};
+  int rc = gemm_err_buf(&q.g[0].err);
+  auto shape = [&](const __nv_bfloat16 *A, const __nv_bfloat16 *Bt, int M, int N, int K,
+                   GemmArgs &g) {
+    g.A = A;
+    g.lda = K;
+    g.Bt = Bt;
+    g.ldb = K;
+    g.M = M;
+    g.N = N;
+    g.K = K;
+    g.ldc32 = g.ldc16 = N;
+  };
+  auto gemm = [&](const __nv_bfloat16 *A, const __nv_bfloat16 *Bt, int M, int N, int K,
+                  GemmArgs g) {
+    shape(A, Bt, M, N, K, g);
+    if (!rc) rc = sg::gemm_bf16(g, st);
+  };
+  // forward: pre-activations, activations and their transposes
+  const __nv_bfloat16 *x = (const __nv_bfloat16 *)feat;
+  for (int l = 0; l < 4; ++l) {
+    GemmArgs g{};
+    g.bias = b[l];
+    if (l < 3) {
+      g.act = 1;
+      g.C32 = s.pre[l];
+      g.C16 = s.act[l];
+      g.C16T = s.in_t[l + 1];
+      g.ldc16t = B;
+    } else {
+      g.C32 = s.logits;
+    }
+    gemm(x, (const __nv_bfloat16 *)W[l], B, kLayerOut[l], kLayerIn[l], g);
+    if (l < 3) x = s.act[l];
+  }
+  k_ce_loss<<<(B + 7) / 8, 256, 0, st>>>(s.logits, kEmuOut, targets, B, s.delta[3], kEmuOut,
+                                         kEmuOut, loss_sum);
+  TransposeJobs d{};
+  d.src[0] = s.delta[3];
+  d.dst[0] = s.delta_t[3];
+  d.rows[0] = B;
+  d.cols[0] = kEmuOut;
+  k_transpose_jobs<<<dim3((B + 63) / 64, (kEmuOut + 63) / 64, 1), 256, 0, st>>>(d);
+  for (int l = 3; l > 0; --l) {
+    GemmArgs h{};
+    h.C16 = s.delta[l - 1];
+    h.C16T = s.delta_t[l - 1];
+    h.ldc16t = B;
+    h.bwd_pre = s.pre[l - 1];
+    gemm(s.delta[l], s.w_t[l], B, kLayerIn[l], kLayerOut[l], h);
+  }
+  q.n = 4;
+  for (int l = 0; l < 4; ++l) {
+    q.g[l].err = q.g[0].err;
+    q.g[l].C32 = dW[l];
+    shape(s.delta_t[l], s.in_t[l], kLayerOut[l], kLayerIn[l], B, q.g[l]);
+  }
+  if (!rc) launch_gemm_group(q, st);
+  RowsumJobs r{};
+  int rows = 0;
+  for (int l = 0; l < 4; ++l) {
+    r.src[l] = s.delta_t[l];
+    r.dst[l] = db[l];
+    r.rows[l] = kLayerOut[l];
+    rows += kLayerOut[l];
+  }
+  k_rowsum_jobs<<<rows, 256, 0, st>>>(r, B);
+  if (rc) {
+    cudaStreamSynchronize(st);
+    cudaGetLastError();
+    return rc;
+  }
+  return sg::gemm_check(st);
 }
 
 extern "C" int sg_quant_fp8_rows(const float *W, int32_t rows, int32_t cols, void *W8,

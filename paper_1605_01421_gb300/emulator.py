@@ -118,33 +118,23 @@ class Emulator:
     # -- backward ------------------------------------------------------------
     def gradients(self, feat16, targets):
         """Mean cross-entropy and its gradients (dW per layer FP32 out x in,
-        db per layer), all on the GPU."""
+        db per layer), all on the GPU (a multiple of 8 rows)."""
         torch = self.torch
         L = binding.lib()
         B = feat16.shape[0]
-        logits, acts, pres = self.forward(feat16, keep=True)
-        dlog = torch.empty((B, NOUT), dtype=torch.bfloat16, device=self.device)
-        loss = torch.zeros(1, dtype=torch.float64, device=self.device)
-        _check(L.sg_mlp_ce_loss(_p(logits), NOUT, _p(targets), B, _p(dlog), NOUT, _p(loss),
-                                _s()))
-        dW, db = [None] * 4, [None] * 4
-        delta = dlog
-        for li in (3, 2, 1, 0):
-            o, i = DIMS[li]
-            dT = torch.empty((o, B), dtype=torch.bfloat16, device=self.device)
-            aT = torch.empty((i, B), dtype=torch.bfloat16, device=self.device)
-            _check(L.sg_transpose_bf16(_p(delta), B, o, _p(dT), _s()))
-            _check(L.sg_transpose_bf16(_p(acts[li]), B, i, _p(aT), _s()))
-            dW[li], _ = binding.gemm_bf16(dT, aT, out32=True)
-            db[li] = torch.empty(o, dtype=torch.float32, device=self.device)
-            _check(L.sg_colsum_bf16(_p(delta), B, o, _p(db[li]), _s()))
-            if li > 0:
-                WT = torch.empty((i, o), dtype=torch.bfloat16, device=self.device)
-                _check(L.sg_transpose_bf16(_p(self.W16[li]), o, i, _p(WT), _s()))
-                dpost, _ = binding.gemm_bf16(delta, WT, out32=True)
-                nxt = torch.empty((B, i), dtype=torch.bfloat16, device=self.device)
-                _check(L.sg_gelu_backward(_p(dpost), _p(pres[li - 1]), B * i, _p(nxt), _s()))
-                delta = nxt
+        dW = [torch.empty((o, i), dtype=torch.float32, device=self.device) for o, i in DIMS]
+        db = [torch.empty(o, dtype=torch.float32, device=self.device) for o, _ in DIMS]
+        loss = torch.empty(1, dtype=torch.float64, device=self.device)
+        nb = int(L.sg_mlp_gradients_scratch(B))
+        scratch = torch.empty(nb, dtype=torch.uint8, device=self.device)
+
+        def ptrs(ts):
+            return (ctypes.c_void_p * 4)(*[t.data_ptr() for t in ts])
+
+        _check(L.sg_mlp_gradients(
+            binding._dev_ptr(feat16, torch.bfloat16, (B, NIN), "feat16"),
+            _p(targets), B, ptrs(self.W16), ptrs(self.b32), ptrs(dW), ptrs(db), _p(loss),
+            _p(scratch), nb, _s()))
         return float(loss.item()) / B, dW, db
 
     def adam(self, dW, db, lr, b1=0.9, b2=0.999, eps=1e-8):
