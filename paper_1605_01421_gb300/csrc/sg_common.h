@@ -27,18 +27,25 @@ struct SgTables {
   float g_lo[SG_MAX_GDATA], g_hi[SG_MAX_GDATA];  // FP32 neighbours: g_lo <= gdata <= g_hi
 };
 
-// Scheduled events in planned order, structure of arrays on the device.
-struct SgEventsDev {
-  const int8_t *type;
-  const uint8_t *select;
-  const int8_t *shift;     // -1 = no shift
-  const int32_t *node;
-  const int32_t *dest;
-  const int32_t *n;
-  const double *proportion;
-  const int64_t *index;    // position in the caller's list (random stream key)
-  const int32_t *rep;      // replicate of a replicate-specific event, or -1
+// A scheduled event in planned order, one 32-byte sector (two 16-byte loads;
+// as eight arrays each event touched eight sectors).  An E1 event (exit,
+// enter, internal transfer) is found through its node's list, so its node
+// and dest fields hold what the walk along that list needs instead.
+struct SgEvent {
+  union {
+    int32_t node;
+    int32_t next;  // E1: day index of the node's next E1 event, or SG_NO_DAY
+  };
+  int32_t dest;    // E1: unused
+  int32_t n;
+  int8_t type;
+  uint8_t select;
+  int8_t shift;    // -1 = no shift
+  uint8_t pad;
+  double proportion;
+  int64_t index;   // position in the caller's list (random stream key)
 };
+#define SG_NO_DAY 0x7fffffff
 
 // Error word written by kernels: the first error wins (atomicCAS on code).
 struct SgDevError {

@@ -82,6 +82,11 @@ __device__ __forceinline__ long long order_key(double x) {
 // x > 0 for a value that is not NaN (negative zero is not > 0).
 __device__ __forceinline__ bool gt0(double x) { return __double_as_longlong(x) > 0; }
 
+// isfinite, from the bits.
+__device__ __forceinline__ bool finite_bits(double x) {
+  return (__double_as_longlong(x) & 0x7ff0000000000000LL) != 0x7ff0000000000000LL;
+}
+
 // a <= b for two values that are not NaN and not negative.
 __device__ __forceinline__ bool le_nonneg(double a, double b) {
   return __double_as_longlong(a) <= __double_as_longlong(b);
@@ -111,7 +116,8 @@ __device__ __forceinline__ double log_pos(double x) {
   k += (int)(bits >> 52) - 1023;
   double m = __longlong_as_double((bits & 0x000fffffffffffffLL) |
                                   0x3ff0000000000000LL);
-  if (m > 0x1.6a09e667f3bcdp+0) {  // sqrt(2) rounded to nearest
+  // m > sqrt(2) rounded to nearest (both positive: compared as integers)
+  if (__double_as_longlong(m) > 0x3ff6a09e667f3bcdLL) {
     m = m * 0.5;
     k = k + 1;
   }
@@ -346,7 +352,7 @@ __device__ __forceinline__ bool bad_rate(double w) {
 
 // Season ends as integers: for an integer day d, d <= e exactly when
 // d <= floor(e) (any finite e); NaN ends never hold.
-__device__ __forceinline__ int season_end_int(double e) {
+__host__ __device__ __forceinline__ int season_end_int(double e) {
   if (e >= 2147483647.0) return 0x7fffffff;
   if (!(e >= -2147483648.0)) return (int)0x80000000;
   return (int)floor(e);
@@ -387,7 +393,7 @@ __device__ __forceinline__ int post_step(double *v, const int *u, const int *end
   const double beta = season_decay(t, ends, pg + 1);
   const double nv = phi + (shed - beta * phi);
   v[0] = nv;
-  if (!isfinite(nv)) return SG_ERR_PTS;
+  if (!finite_bits(nv)) return SG_ERR_PTS;
   return __double_as_longlong(nv) != __double_as_longlong(phi) ? 1 : 0;
 }
 

@@ -35,18 +35,27 @@ using namespace sg;
 namespace {
 
 // SISe_sp post time step of every node for unit time T from the same old
-// values (Sec. 4.2 with the coupling term), one thread per (replicate, node):
+// values (Sec. 4.2 with the coupling term):
 //   phi' = phi + ((alpha I / N + sum_k ((phi_k N_k - phi N) / N) (D / d_k))
 //                 - beta(T) phi),
 // neighbours in list order, both terms 0 in an empty node; then recording.
+//
+// Eight lanes per (replicate, node): each forms one neighbour's term at a
+// time (13 FP64 operations, whatever the number of active lanes), and the
+// terms are added in list order.  D / d_k does not change from day to day
+// and is kept with the neighbour list.  (One thread per node with the
+// division in it: a chain of ~800 cycles per neighbour on 13 of 152 SMs;
+// 1,600 farms x 365 days 26.8 ms with the day's other kernels.)
+constexpr int kPtsLanes = 8;
 struct PtsSpArgs {
   const int *u;
   const double *v_old;
   double *v_new;
   const double *ldata;
+  const int4 *ends;
   const int64_t *nb_ptr;
   const int32_t *nb_idx;
-  const double *nb_dist;
+  const double *nb_rate;  // D / d_k
   int32_t *U;
   double *V;
   const int32_t *rec;
@@ -56,66 +65,72 @@ struct PtsSpArgs {
   OutDev out;
 };
 
-// The coupled post time step of one (replicate, node) and its recording at
-// slot m; the node's counts are returned in uu.
-__device__ __forceinline__ void pts_sp_node(const SgTables &tb, const PtsSpArgs &a, long long gid,
-                                          int m, int *uu) {
+__global__ void __launch_bounds__(128) k_pts_sp(const __grid_constant__ SgTables tb,
+                                                const __grid_constant__ PtsSpArgs a) {
+  pdl_trigger();
+  pdl_wait();
+  constexpr unsigned full = 0xffffffffu;
   const int Nn = tb.n_nodes;
-  const int rep = (int)(gid / Nn), node = (int)(gid - (long long)rep * Nn);
+  const int lane = threadIdx.x & 31, sub = lane & (kPtsLanes - 1);
+  const long long gid =
+      ((long long)blockIdx.x * blockDim.x + threadIdx.x) / kPtsLanes;
+  const bool in_range = gid < (long long)Nn * a.n_rep;
+  const int m = a.rec[a.T - a.t0];
+  const int rep = in_range ? (int)(gid / Nn) : 0;
+  const int node = in_range ? (int)(gid - (long long)rep * Nn) : 0;
   const int *ur = a.u + (long long)rep * Nn * 2;
   const double *vr = a.v_old + (long long)rep * Nn;
   const double *g = tb.gdata;
-  const int S = ur[node * 2], I = ur[node * 2 + 1];
-  const double Ni = i2d(S) + i2d(I);
-  const double phi = vr[node];
-  double shed = 0.0, coupling = 0.0;
-  if (gt0(Ni)) {
-    shed = (g[2] * i2d(I)) / Ni;
-    if (a.nb_ptr) {
-      const double DN = g[7];
-      for (long long k = a.nb_ptr[node]; k < a.nb_ptr[node + 1]; ++k) {
-        const int j = a.nb_idx[k];
-        const double Nk = i2d(ur[j * 2]) + i2d(ur[j * 2 + 1]);
-        const double term = ((vr[j] * Nk - phi * Ni) / Ni) * (DN / a.nb_dist[k]);
-        coupling = coupling + term;
-      }
-    }
-  }
-  int ends[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) ends[i] = season_end_int(a.ldata[(long long)node * tb.n_ldata + i]);
-  const double beta = season_decay(a.T, ends, g + 3);
-  const double nv = phi + ((shed + coupling) - beta * phi);
-  a.v_new[gid] = nv;
-  if (!isfinite(nv)) report(a.err, SG_ERR_PTS, a.rep0 + rep, node, a.T, -1);
-  uu[0] = S;
-  uu[1] = I;
-  if (m >= 0) {
-    const long long base = ((long long)rep * a.M + m) * Nn + node;
-    if (a.U) {
-      a.U[base * 2] = S;
-      a.U[base * 2 + 1] = I;
-    }
-    if (a.V) a.V[base] = nv;
-    record_sparse<2, 1>(a.out, m, rep, node, uu, &nv);
-  }
-}
-
-__global__ void __launch_bounds__(128) k_pts_sp(const SgTables tb, const PtsSpArgs a) {
-  pdl_trigger();
-  pdl_wait();
-  const int Nn = tb.n_nodes;
-  const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool in_range = gid < (long long)Nn * a.n_rep;
-  const int m = a.rec[a.T - a.t0];
   int uu[2] = {0, 0};
-  if (in_range) pts_sp_node(tb, a, gid, m, uu);
-  if (m >= 0 && a.out.prev) {
-    const int rep = in_range ? (int)(gid / Nn) : 0;
-    prevalence_add<2>(a.out, in_range ? (long long)rep * a.M + m : -1, in_range, uu);
+  double phi = 0.0;
+  long long k = 0, end = 0;
+  if (in_range) {
+    uu[0] = ur[node * 2];
+    uu[1] = ur[node * 2 + 1];
+    phi = vr[node];
+    if (a.nb_ptr) {
+      k = a.nb_ptr[node];
+      end = a.nb_ptr[node + 1];
+    }
+  }
+  const double Ni = l2d((long long)uu[0] + uu[1]);
+  if (!gt0(Ni)) end = k;
+  const double own = phi * Ni;
+  double coupling = 0.0;
+  while (__any_sync(full, k < end)) {
+    double term = 0.0;
+    if (k + sub < end) {
+      const int j = a.nb_idx[k + sub];
+      const double Nk = l2d((long long)ur[j * 2] + ur[j * 2 + 1]);
+      term = ((vr[j] * Nk - own) / Ni) * a.nb_rate[k + sub];
+    }
+#pragma unroll
+    for (int q = 0; q < kPtsLanes; ++q) {
+      const double x = __shfl_sync(full, term, (lane & ~(kPtsLanes - 1)) + q);
+      if (k + q < end) coupling = coupling + x;
+    }
+    k += kPtsLanes;
+  }
+  if (in_range && sub == 0) {
+    const double shed = gt0(Ni) ? (g[2] * i2d(uu[1])) / Ni : 0.0;
+    int ends[4];
+    load_ends(a.ends, a.ldata, tb, node, ends);
+    const double beta = season_decay(a.T, ends, g + 3);
+    const double nv = phi + ((shed + coupling) - beta * phi);
+    a.v_new[gid] = nv;
+    if (!finite_bits(nv)) report(a.err, SG_ERR_PTS, a.rep0 + rep, node, a.T, -1);
+    if (m >= 0) {
+      const long long base = ((long long)rep * a.M + m) * Nn + node;
+      if (a.U) {
+        a.U[base * 2] = uu[0];
+        a.U[base * 2 + 1] = uu[1];
+      }
+      if (a.V) a.V[base] = nv;
+      record_sparse<2, 1>(a.out, m, rep, node, uu, &nv);
+      if (a.out.prev) prevalence_add_unit<2>(a.out, (long long)rep * a.M + m, uu);
+    }
   }
 }
-
 
 // Channels of the all events method before the first day: rate 0, asleep
 // (firing time +inf), no draws taken.
@@ -353,6 +368,7 @@ struct GraphKey {
 struct sg_model {
   SgTables tb;
   DevBuf<double> ldata;
+  DevBuf<int4> ends;  // the nodes' season ends (models with phi)
   EventTable ev;
   // planned events for the cached window
   bool plan_ok = false;
@@ -361,11 +377,9 @@ struct sg_model {
   // one host staging buffer (ev_stage)
   DevBuf<unsigned char> ev_arena;
   std::vector<unsigned char> ev_stage;
-  int8_t *e_type = nullptr, *e_shift = nullptr;
-  uint8_t *e_select = nullptr;
-  int32_t *e_node = nullptr, *e_dest = nullptr, *e_n = nullptr, *e1_day = nullptr;
-  double *e_prop = nullptr;
-  int64_t *e_index = nullptr, *wave_ev = nullptr, *wave_off = nullptr, *e1_node_off = nullptr;
+  SgEvent *e_rec = nullptr;
+  int32_t *e1_day = nullptr;
+  int64_t *wave_ev = nullptr, *wave_off = nullptr, *e1_node_off = nullptr;
   int32_t heavy_after = -1;  // draws a thread takes before its warp takes
   int32_t npb = -1;          // nodes per block; -1 = chosen from the size
   // sg_set_replicate_range: the runs cover global replicates rep0 .. rep0 +
@@ -373,7 +387,7 @@ struct sg_model {
   int32_t rep0 = 0, rep_total = 0;
   // working memory
   DevBuf<int32_t> e1_cur;
-  DevBuf<int32_t> e1_next;  // sparse schedule: day of each unit's next E1 event
+  DevBuf<int32_t> e1_next;  // day of each unit's next E1 event
   // the external transfers of a replicate-day touch a sizeable share of its
   // nodes (on average at least one node in 16 as a source): the E2 kernel
   // then stages the replicate's state in shared memory, else it works on
@@ -428,7 +442,7 @@ struct sg_model {
   // SISe_sp neighbour lists and the second phi buffer of the coupled step
   DevBuf<int64_t> nb_ptr;
   DevBuf<int32_t> nb_idx;
-  DevBuf<double> nb_dist, v2;
+  DevBuf<double> nb_rate, v2;  // D / distance; second phi buffer
   bool has_nb = false;
   uint64_t nb_version = 0;
   // solver (SG_SOLVER_SSM or SG_SOLVER_AEM) and the channel state of 'aem'
@@ -582,6 +596,15 @@ static int model_create(const sg_desc *d, sg_model **out, bool generic) {
   const size_t nl = (size_t)d->n_ldata * d->n_nodes;
   std::vector<double> ld(d->ldata ? d->ldata : nullptr, d->ldata ? d->ldata + nl : nullptr);
   int rc = upload(m->ldata, ld);
+  if (!rc && d->n_v > 0 && d->n_ldata >= 4) {
+    std::vector<int4> ends((size_t)d->n_nodes);
+    for (size_t i = 0; i < ends.size(); ++i) {
+      const double *e = ld.data() + i * (size_t)d->n_ldata;
+      ends[i] = make_int4(season_end_int(e[0]), season_end_int(e[1]), season_end_int(e[2]),
+                          season_end_int(e[3]));
+    }
+    rc = upload(m->ends, ends);
+  }
   if (!rc) rc = m->err.ensure(1);
   if (!rc) rc = m->cnt.ensure(1);
   if (!rc && !(m->h_err = static_cast<SgDevError *>(pinned_pool().get(sizeof(SgDevError)))))
@@ -665,6 +688,7 @@ extern "C" int sg_model_tables(const sg_model *m, int32_t *S, int32_t *G) {
 extern "C" void sg_model_destroy(sg_model *m) {
   if (!m) return;
   m->ldata.release();
+  m->ends.release();
   m->ev_arena.release();
   m->e1_cur.release();
   m->e1_next.release();
@@ -676,7 +700,7 @@ extern "C" void sg_model_destroy(sg_model *m) {
   if (m->side_fork) cudaEventDestroy(m->side_fork);
   if (m->side_join) cudaEventDestroy(m->side_join);
   m->emu_logits.release(); m->emu_flag.release(); m->emu_delta.release();
-  m->nb_ptr.release(); m->nb_idx.release(); m->nb_dist.release(); m->v2.release();
+  m->nb_ptr.release(); m->nb_idx.release(); m->nb_rate.release(); m->v2.release();
   m->aem_a.release(); m->aem_tau.release(); m->aem_cnt.release();
   m->out_u_colptr.release(); m->out_v_colptr.release();
   m->out_u_row.release(); m->out_v_row.release();
@@ -757,10 +781,7 @@ static int ensure_plan(sg_model *m, int32_t t0, int32_t t_end, int32_t slots) {
     off = (off + bytes + 255) & ~(size_t)255;
     return o;
   };
-  const size_t o_type = place(n), o_shift = place(n), o_sel = place(n),
-               o_node = place(4 * n), o_dest = place(4 * n), o_cnt = place(4 * n),
-               o_prop = place(8 * n), o_idx = place(8 * n),
-               o_wev = place(8 * P.wave_ev.size()), o_woff = place(8 * P.e2_wave_off.size()),
+  const size_t o_rec = place(sizeof(SgEvent) * n), o_wev = place(8 * P.wave_ev.size()), o_woff = place(8 * P.e2_wave_off.size()),
                o_e1d = place(4 * P.e1_day.size()), o_e1o = place(8 * P.e1_node_off.size());
   const size_t total = std::max<size_t>(off, 256);
   std::lock_guard<std::mutex> stage_lock(g_stage_mu);
@@ -770,9 +791,7 @@ static int ensure_plan(sg_model *m, int32_t t0, int32_t t_end, int32_t slots) {
     h = m->ev_stage.data();
   }
   {
-    gather_events(m->ev, P, (int8_t *)(h + o_type), (int8_t *)(h + o_shift), h + o_sel,
-                  (int32_t *)(h + o_node), (int32_t *)(h + o_dest), (int32_t *)(h + o_cnt),
-                  (double *)(h + o_prop), (int64_t *)(h + o_idx));
+    gather_events(m->ev, P, (SgEvent *)(h + o_rec));
     auto put = [&](size_t o, const void *src, size_t bytes) {
       if (bytes) std::memcpy(h + o, src, bytes);
     };
@@ -787,14 +806,7 @@ static int ensure_plan(sg_model *m, int32_t t0, int32_t t_end, int32_t slots) {
     return SG_ERR_CUDA;
   }
   unsigned char *d = m->ev_arena.p;
-  m->e_type = (int8_t *)(d + o_type);
-  m->e_shift = (int8_t *)(d + o_shift);
-  m->e_select = d + o_sel;
-  m->e_node = (int32_t *)(d + o_node);
-  m->e_dest = (int32_t *)(d + o_dest);
-  m->e_n = (int32_t *)(d + o_cnt);
-  m->e_prop = (double *)(d + o_prop);
-  m->e_index = (int64_t *)(d + o_idx);
+  m->e_rec = (SgEvent *)(d + o_rec);
   m->wave_ev = (int64_t *)(d + o_wev);
   m->wave_off = (int64_t *)(d + o_woff);
   m->e1_day = (int32_t *)(d + o_e1d);
@@ -1061,8 +1073,8 @@ static void enqueue_run(sg_model *m, const DayArgs &da0, const EvArgs &ea0, int3
   cudaMemsetAsync(m->err.p, 0, sizeof(SgDevError), st);
   cudaMemsetAsync(m->cnt.p, 0, sizeof(SgCounters), st);
   cudaMemsetAsync(m->e1_cur.p, 0, sizeof(int32_t) * (size_t)std::max(1, Nn * n_rep), st);
-  if (da0.npb > kDayBlock && da0.ev.e1_node_off && Nn > 0) {
-    // the sparse schedule's per-unit day of the next E1 event
+  if (da0.ev.e1_node_off && Nn > 0) {
+    // each unit's day of its next E1 event
     const long long units = (long long)Nn * n_rep;
     const unsigned g = (unsigned)std::min<long long>(4096, (units + 255) / 256);
     k_e1_next_init<<<std::max(1u, g), 256, 0, st>>>(da0.ev.e1_node_off, da0.ev.e1_day, Nn,
@@ -1119,7 +1131,8 @@ static void enqueue_run(sg_model *m, const DayArgs &da0, const EvArgs &ea0, int3
     pa.ldata = m->ldata.p;
     pa.nb_ptr = m->has_nb ? m->nb_ptr.p : nullptr;
     pa.nb_idx = m->nb_idx.p;
-    pa.nb_dist = m->nb_dist.p;
+    pa.nb_rate = m->nb_rate.p;
+    pa.ends = m->ends.p;
     pa.U = da0.U;
     pa.V = da0.V;
     pa.out = da0.out;
@@ -1156,7 +1169,7 @@ static void enqueue_run(sg_model *m, const DayArgs &da0, const EvArgs &ea0, int3
       pa.T = T;
       {
         LaunchTimer lt(m, st, 0);
-        launch_pdl(k_pts_sp, (unsigned)((units + 127) / 128), 128, 0, st, tb, pa);
+        launch_pdl(k_pts_sp, (unsigned)((units * kPtsLanes + 127) / 128), 128, 0, st, tb, pa);
       }
       ++launches;
       std::swap(vc, vn);
@@ -1507,13 +1520,12 @@ extern "C" int sg_run(sg_model *m, const int32_t *tspan, int32_t n_tspan, uint64
     m->graph_ok = false;
   }
 
-  const EvDev evd{m->e_type, m->e_select, m->e_shift, m->e_node, m->e_dest,
-                  m->e_n,    m->e_prop,   m->e_index, m->e1_day,
-                  P.n_e1 > 0 ? m->e1_node_off : nullptr};
+  const EvDev evd{m->e_rec, m->e1_day, P.n_e1 > 0 ? m->e1_node_off : nullptr};
   DayArgs da{};
   da.u = m->u.p;
   da.v = m->v.p;
   da.ldata = m->ldata.p;
+  da.ends = m->ends.p;
   da.U = d_U;
   da.V = d_V;
   da.rec = m->rec.p;
@@ -1529,6 +1541,9 @@ extern "C" int sg_run(sg_model *m, const int32_t *tspan, int32_t n_tspan, uint64
   da.fast = filter_applies(tb) ? 1 : 0;
   set_warp_rule(da, m->heavy_after);
   da.npb = m->npb > 0 ? m->npb : default_npb((long long)Nn * n_rep);
+  // aem: in blocks of a few nodes every node's firings start on its own warp
+  // (1,600 SISe herds: the longest node's chain of firings sets the day)
+  if (aem && m->heavy_after < 0 && da.npb <= 8) da.heavy_after = 0;
   // the sparse-activity schedule (nodes_per_block > kDayBlock) is for the
   // direct method on the built-in kinds with the day / E2 kernel pair;
   // elsewhere such a split falls back to full thread-per-node blocks
@@ -2345,9 +2360,11 @@ extern "C" int sg_set_neighbors(sg_model *m, const int64_t *ptr, const int32_t *
   try {
     std::vector<int64_t> p(ptr, ptr + Nn + 1);
     std::vector<int32_t> ix(idx ? idx : nullptr, idx ? idx + nnz : nullptr);
-    std::vector<double> ds(dist ? dist : nullptr, dist ? dist + nnz : nullptr);
+    // D / d_k of the coupled step (one IEEE division, as on the device)
+    std::vector<double> rate((size_t)nnz);
+    for (int64_t k = 0; k < nnz; ++k) rate[(size_t)k] = m->tb.gdata[7] / dist[k];
     if ((rc = upload(m->nb_ptr, p)) || (rc = upload(m->nb_idx, ix)) ||
-        (rc = upload(m->nb_dist, ds)))
+        (rc = upload(m->nb_rate, rate)))
       return rc;
   } catch (const std::bad_alloc &) {
     return SG_ERR_NOMEM;

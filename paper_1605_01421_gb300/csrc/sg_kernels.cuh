@@ -32,17 +32,22 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // Kernels
 // ---------------------------------------------------------------------------
 
-// Events of the plan, structure of arrays in planned order (E1 part first).
+// Events of the plan in planned order (E1 part first).
 struct EvDev {
-  const int8_t *type;
-  const uint8_t *select;
-  const int8_t *shift;       // -1 = no shift
-  const int32_t *node, *dest, *n;
-  const double *proportion;
-  const int64_t *index;      // position in the caller's list (random stream key)
-  const int32_t *e1_day;     // day index of each E1 event
+  const SgEvent *rec;
+  const int32_t *e1_day;       // day index of each E1 event
   const int64_t *e1_node_off;  // [slots * Nn + 1]; nullptr when there are none
 };
+
+__device__ __forceinline__ SgEvent load_event(const SgEvent *p) {
+  union {
+    int4 v[2];
+    SgEvent e;
+  } r;
+  r.v[0] = __ldg(reinterpret_cast<const int4 *>(p));
+  r.v[1] = __ldg(reinterpret_cast<const int4 *>(p) + 1);
+  return r.e;
+}
 
 // Output selection (Sec. 3.2 result slots U_sparse and V_sparse, and the
 // prevalence summary): compressed-column patterns with the layouts of U
@@ -150,11 +155,12 @@ struct DayArgs {
   int *u;              // [R][Nn][C] working counts
   double *v;           // [R][Nn][NV] working continuous state
   const double *ldata; // [Nn][n_ldata]
+  const int4 *ends;    // [Nn]: the season ends as integers (null: from ldata)
   int32_t *U;          // [R][M][Nn][C]
   double *V;           // [R][M][Nn][NV]
   const int32_t *rec;  // [days + 1]: tspan slot of T = t0 + i, or -1
   int32_t *e1_cur;     // [R][Nn]: next E1 event, relative to the node's list
-  int32_t *e1_next;    // [R][Nn]: day index of that event (sparse schedule)
+  int32_t *e1_next;    // [R][Nn]: day index of that event, or SG_NO_DAY
   EvDev ev;
   int32_t t0, M, n_rep, slots;
   // global index of the run's replicate 0 (a shard of a larger job): every
@@ -211,6 +217,22 @@ struct DayArgs {
   // its post time step, so one launch covers all days; 0: off
   int32_t e2_inblock;
 };
+
+// A node's season ends as integers (the conversion from ldata is a dozen FP64
+// instructions, so it is done once per model).
+__device__ __forceinline__ void load_ends(const int4 *ends, const double *ldata,
+                                          const SgTables &tb, int node, int *ld) {
+  if (ends) {
+    const int4 e = __ldg(ends + node);
+    ld[0] = e.x;
+    ld[1] = e.y;
+    ld[2] = e.z;
+    ld[3] = e.w;
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) ld[i] = season_end_int(ldata[(long long)node * tb.n_ldata + i]);
+  }
+}
 
 // %globaltimer (ns).
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -282,12 +304,57 @@ __device__ __forceinline__ bool grid_barrier(unsigned int *bar, int n_blocks, Sg
 // launch, so it is read and written at L2 only (ld / st .cg) and added to
 // with atomics; a wave never samples a node another event of the wave
 // touches.  Same arithmetic and random stream as the E2 kernel.
+// The day's events and wave bounds may have been staged in shared memory
+// (E2Stage) while the day's SSA ran.
+constexpr int kE2StageEv = 128, kE2StageWaves = 31;
+struct E2Stage {
+  SgEvent ev[kE2StageEv];
+  long long wave[kE2StageWaves + 1];  // bounds of waves w0 .. w0 + n_waves
+  long long w0, w1, lo;               // the day's waves, first staged event
+  int n_waves, n_ev;                  // 0: nothing staged
+};
+
+// Staged by one warp, the events by asynchronous copies that the block waits
+// for (cp.async.wait_all and a barrier) before e2_rep_block.
+__device__ __forceinline__ void e2_stage(E2Stage &s, const DayArgs &a, long long w0,
+                                         long long w1) {
+  const int lane = threadIdx.x & 31;
+  const int nw = (int)min(w1 - w0, (long long)kE2StageWaves);
+  if (lane <= nw) s.wave[lane] = a.wave_ev[w0 + lane];
+  __syncwarp();
+  const long long lo = s.wave[0];
+  const int n = (int)min(s.wave[nw] - lo, (long long)kE2StageEv);
+  if (lane == 0) {
+    s.w0 = w0;
+    s.w1 = w1;
+    s.lo = lo;
+    s.n_waves = nw;
+    s.n_ev = n;
+  }
+  for (int i = lane; i < 2 * n; i += 32)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(reinterpret_cast<int4 *>(s.ev) + i)),
+                 "l"(reinterpret_cast<const int4 *>(a.ev.rec + lo) + i)
+                 : "memory");
+}
+
 template <int C>
 __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int T,
-                             long long w0, long long w1) {
+                             long long w0, long long w1, const E2Stage *stage = nullptr) {
+  auto event = [&](long long j) {
+    if (stage && j >= stage->lo && j < stage->lo + stage->n_ev) return stage->ev[j - stage->lo];
+    return load_event(a.ev.rec + j);
+  };
+  auto bound = [&](long long w) {
+    if (stage && w >= stage->w0 && w <= stage->w0 + stage->n_waves)
+      return stage->wave[w - stage->w0];
+    return (long long)a.wave_ev[w];
+  };
   // a run that already failed does nothing (one thread reads, the barrier
-  // makes the answer the block's)
-  if (__syncthreads_or(threadIdx.x == 0 && *(volatile int32_t *)&a.err->code != 0)) return;
+  // makes the answer the block's); with the events staged the caller has
+  // checked this day
+  if (!stage && __syncthreads_or(threadIdx.x == 0 && *(volatile int32_t *)&a.err->code != 0))
+    return;
   int *state = a.u + (long long)rep * tb.n_nodes * C;
   const uint64_t seed = ((uint64_t)a.k1 << 32) | a.k0;
   constexpr int kHv = 256;  // large transfers of a wave left to the warps
@@ -299,12 +366,13 @@ __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int 
   if (threadIdx.x == 0) s_nhv = 0;
   __syncthreads();
   for (long long w = w0; w < w1; ++w) {
-    const long long lo = a.wave_ev[w], hi = a.wave_ev[w + 1];
+    const long long lo = bound(w), hi = bound(w + 1);
     for (long long j = lo + threadIdx.x; j < hi; j += blockDim.x) {
-      const int src = a.ev.node[j];
+      const SgEvent ev = event(j);
+      const int src = ev.node;
       int *un = state + (long long)src * C;
-      const uint32_t mask = tb.Emask[a.ev.select[j]];
-      const long long idx = a.ev.index[j];
+      const uint32_t mask = tb.Emask[ev.select];
+      const long long idx = ev.index;
       int cur[C];
       long long total = 0;
 #pragma unroll
@@ -312,9 +380,8 @@ __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int 
         cur[p] = __ldcg(un + p);
         if ((mask >> p) & 1u) total += cur[p];
       }
-      const int n = a.ev.n[j];
       const long long k =
-          n > 0 ? (long long)n : (long long)round(a.ev.proportion[j] * (double)total);
+          ev.n > 0 ? (long long)ev.n : (long long)round(ev.proportion * (double)total);
       if (k < 0 || k > total) {
         report(a.err, SG_ERR_EVENT_UNDERFLOW, a.rep0 + rep, src, T, idx);
         bad = true;
@@ -351,8 +418,8 @@ __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int 
           }
         }
       }
-      const int q_sh = a.ev.shift[j];
-      int *ud = state + (long long)a.ev.dest[j] * C;
+      const int q_sh = ev.shift;
+      int *ud = state + (long long)ev.dest * C;
 #pragma unroll
       for (int p = 0; p < C; ++p)
         if (moved[p] != 0) __stcg(un + p, cur[p] - moved[p]);
@@ -371,9 +438,10 @@ __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int 
       // wave touches their source nodes)
       for (int h = warp; h < nhv; h += nwarps) {
         const long long j = s_hv[h];
-        const int src = a.ev.node[j];
+        const SgEvent ev = event(j);
+        const int src = ev.node;
         int *un = state + (long long)src * C;
-        const uint32_t mask = tb.Emask[a.ev.select[j]];
+        const uint32_t mask = tb.Emask[ev.select];
         int cur[C];
         long long total = 0;
 #pragma unroll
@@ -381,15 +449,14 @@ __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int 
           cur[p] = __ldcg(un + p);
           if ((mask >> p) & 1u) total += cur[p];
         }
-        const int n = a.ev.n[j];
         const long long k =
-            n > 0 ? (long long)n : (long long)round(a.ev.proportion[j] * (double)total);
+            ev.n > 0 ? (long long)ev.n : (long long)round(ev.proportion * (double)total);
         int moved[C];
-        urn_warp<C>(cur, mask, (uint32_t)k, (uint32_t)total, seed, a.ev.index[j], a.rep0 + rep,
+        urn_warp<C>(cur, mask, (uint32_t)k, (uint32_t)total, seed, ev.index, a.rep0 + rep,
                     moved);
         if (lane == 0) {
-          const int q_sh = a.ev.shift[j];
-          int *ud = state + (long long)a.ev.dest[j] * C;
+          const int q_sh = ev.shift;
+          int *ud = state + (long long)ev.dest * C;
 #pragma unroll
           for (int p = 0; p < C; ++p)
             if (moved[p] != 0) __stcg(un + p, cur[p] - moved[p]);
@@ -1017,11 +1084,19 @@ __device__ __forceinline__ int aem_draw(uint32_t &c, uint32_t node, uint32_t j, 
   return 0;
 }
 
+// a == b for rates (no NaN), by integer instructions: an FP64 comparison
+// holds the FP64 pipe as long as any FP64 operation.
+__device__ __forceinline__ bool same_rate(double a, double b) {
+  const unsigned long long x = (unsigned long long)__double_as_longlong(a);
+  const unsigned long long y = (unsigned long long)__double_as_longlong(b);
+  return x == y || ((x | y) << 1) == 0ull;
+}
+
 // Channel j's new rate a_new at time t (the update rule above).
 __device__ __forceinline__ int aem_update(double t, double a_new, double &a, double &tau,
                                           uint32_t &c, uint32_t node, uint32_t j, uint32_t tag,
                                           uint32_t k0, uint32_t k1, unsigned long long &drawn) {
-  if (a_new == a) return 0;
+  if (same_rate(a_new, a)) return 0;
   if (gt0(a) && gt0(a_new)) {
     tau = t + (a / a_new) * (tau - t);
   } else if (gt0(a_new)) {
@@ -1064,7 +1139,7 @@ __device__ __forceinline__ int aem_earliest(const double *tau, double &best) {
   best = __longlong_as_double(0x7ff0000000000000ll);
 #pragma unroll
   for (int j = 0; j < T; ++j) {
-    if (tau[j] < best) {
+    if (order_key(tau[j]) < order_key(best)) {
       best = tau[j];
       mu = j;
     }
@@ -1088,7 +1163,7 @@ __device__ __forceinline__ int aem_steps(int *u, const double *kf, double *a, do
   for (int b = 0;; ++b) {
     double best;
     const int mu = aem_earliest<T>(tau, best);
-    if (mu < 0 || best >= Tn) return AEM_DONE;
+    if (mu < 0 || order_key(best) >= order_key(Tn)) return AEM_DONE;
     if (nfired >= SG_MAX_DRAWS) return SG_ERR_STEP_LIMIT;
     if (b == budget) return AEM_HEAVY;
     ++nfired;
@@ -1117,7 +1192,7 @@ __device__ __forceinline__ int aem_steps(int *u, const double *kf, double *a, do
         } else {
           tau[k] = inf;
         }
-      } else if (!(w == a[k])) {
+      } else if (!same_rate(w, a[k])) {
         if (gt0(a[k]) && gt0(w)) {
           tau[k] = t + (a[k] / w) * (tau[k] - t);
         } else if (gt0(w)) {
@@ -1154,13 +1229,17 @@ struct AemSlots {
                                : kDayBlock;
 };
 
-// The rest of a heavy node-day by a whole warp.  Every channel's next draws
-// depend only on its counter, so lane l holds the Exp(1) value of draw
-// c_j + (l mod B) of channel j = l / B (B = 32 / T lanes per channel), all
-// computed at once; the firing loop runs on all lanes in step and takes a
-// channel's next value from its lane.  When a channel has used its B values
-// the table is recomputed from the current counters.  Same operations, in
-// the same order, as the thread path.
+// The rest of a node-day by a whole warp.  Every channel's next draws depend
+// only on its counter, so lane l holds the Exp(1) value of draw c_j +
+// (l mod B) of channel j = l / B (B = 32 / T lanes per channel), all computed
+// at once; when a channel has used its B values the table is recomputed from
+// the current counters.  Lane j < T also holds channel j's rate, firing time
+// and counter: after a firing the channels that change (the fired one with
+// its new draw, the others by the rescaling rule) share one FP64 division and
+// three more operations, and the earliest channel is found by integer
+// comparison.  Bound by the FP64 pipe, 14 operations a firing of two channels
+// (one channel after the other 30).  Same operations on every value, in the
+// same order, as the thread path.
 template <int KIND>
 __device__ void aem_warp(AemSlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK,
                                  ModelTraits<KIND>::T> &hs,
@@ -1169,77 +1248,104 @@ __device__ void aem_warp(AemSlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK,
   using M = ModelTraits<KIND>;
   constexpr int C = M::C, T = M::T, NK = M::NK;
   constexpr int B = 32 / T;
+  constexpr unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int jl = lane / B, il = lane - jl * B;
+  const bool mine = lane < T;  // this lane holds channel `lane`
   int u[C];
-  double kf[NK], a[T], tau[T];
-  uint32_t c[T];
-  int used[T];
+  double kf[NK];
 #pragma unroll
   for (int p = 0; p < C; ++p) u[p] = hs.u[p];
 #pragma unroll
   for (int i = 0; i < NK; ++i) kf[i] = hs.kf[i];
-#pragma unroll
-  for (int j = 0; j < T; ++j) {
-    a[j] = hs.a[j];
-    tau[j] = hs.tau[j];
-    c[j] = hs.c[j];
-    used[j] = B;  // no table yet
-  }
-  double t = hs.t;
+  double a = mine ? hs.a[lane] : 0.0;
+  double tau = mine ? hs.tau[lane] : 0.0;
+  uint32_t c = mine ? hs.c[lane] : 0u;
+  int used = B;  // no table yet
   uint32_t nfired = hs.nfired;
   const uint32_t node = (uint32_t)hs.node;
   const uint32_t tag = (SG_STREAM_AEM << 24) | (uint32_t)hs.rep;
+  const long long Tkey = order_key(Tn), never = 0x7ff0000000000000ll;
   double myE = 0.0;
   unsigned long long f = 0, dr = 0;
-  auto draw = [&](int j, double &E) -> int {
-    uint32_t cj = 0;
-    int uj = 0;
+  int code = 0;
+  for (;;) {
+    const long long key = order_key(tau);
+    long long best = never;
+    int mu = -1;
 #pragma unroll
-    for (int q = 0; q < T; ++q)
-      if (q == j) {
-        cj = c[q];
-        uj = used[q];
+    for (int j = 0; j < T; ++j) {
+      const long long k = __shfl_sync(full, key, j);
+      if (k < best) {
+        best = k;
+        mu = j;
       }
-    if (cj == 0xffffffffu) return SG_ERR_STEP_LIMIT;
-    if (uj == B) {
-      // recompute the table from every channel's current counter
-      if (jl < T) {
-        uint32_t cl = 0;
-#pragma unroll
-        for (int q = 0; q < T; ++q)
-          if (q == jl) cl = c[q];
-        const uint32_t ci = cl + (uint32_t)il;
-        // draws past the counter's end are never used (the counter check
-        // above stops first); compute something harmless for them
-        const U4 x = philox10(U4{ci < cl ? cl : ci, node, (uint32_t)jl, tag}, k0, k1);
-        myE = -log_pos(u01_open(x.x, x.y));
-      }
-#pragma unroll
-      for (int q = 0; q < T; ++q) used[q] = 0;
-      uj = 0;
     }
-    E = __shfl_sync(0xffffffffu, myE, j * B + uj);
+    if (mu < 0 || best >= Tkey) break;
+    if (nfired >= SG_MAX_DRAWS) {
+      code = SG_ERR_STEP_LIMIT;
+      break;
+    }
+    ++nfired;
+    const double t = __shfl_sync(full, tau, mu);
 #pragma unroll
-    for (int q = 0; q < T; ++q)
-      if (q == j) {
-        ++c[q];
-        ++used[q];
+    for (int p = 0; p < C; ++p) u[p] += tb.S[mu][p];
+    ++f;
+    const uint32_t dep = tb.dep[mu];
+    double w = a;
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k < T; ++k) {
+      if ((dep >> k) & 1u) {
+        const double x = M::rate_k(k, u, kf, tb.gdata);
+        bad = bad || bad_rate(x);
+        if (lane == k) w = x;
       }
-    ++dr;
-    return 0;
-  };
-  const int rc = aem_steps<KIND>(u, kf, a, tau, c, t, nfired, Tn, tb, f, -1, draw);
+    }
+    if (bad) {
+      code = SG_ERR_RATE;
+      break;
+    }
+    const bool changes = mine && (lane == mu || !same_rate(w, a));
+    const bool awake = changes && gt0(w);
+    // the fired channel and the ones that wake take a draw
+    const bool draws = awake && (lane == mu || !gt0(a));
+    if (__any_sync(full, draws && c == 0xffffffffu)) {
+      code = SG_ERR_STEP_LIMIT;
+      break;
+    }
+    if (__any_sync(full, draws && used == B)) {
+      const uint32_t cl = __shfl_sync(full, c, jl < T ? jl : 0);
+      const uint32_t ci = cl + (uint32_t)il;
+      // draws past the counter's end are never used (the check above stops
+      // first); compute something harmless for them
+      const U4 x = philox10(U4{ci < cl ? cl : ci, node, (uint32_t)jl, tag}, k0, k1);
+      myE = -log_pos(u01_open(x.x, x.y));
+      used = 0;
+    }
+    const double E = __shfl_sync(full, myE, (lane * B + used) & 31);
+    if (draws) {
+      ++c;
+      ++used;
+    }
+    dr += __popc(__ballot_sync(full, draws));
+    const double q = (draws ? E : a) / w;
+    const double step = draws ? q : q * (tau - t);
+    const double next = t + step;
+    if (changes) {
+      tau = awake ? next : __longlong_as_double(never);
+      a = w;
+    }
+  }
+  if (mine) {
+    hs.a[lane] = a;
+    hs.tau[lane] = tau;
+    hs.c[lane] = c;
+  }
   if (lane == 0) {
 #pragma unroll
     for (int p = 0; p < C; ++p) hs.u[p] = u[p];
-#pragma unroll
-    for (int j = 0; j < T; ++j) {
-      hs.a[j] = a[j];
-      hs.tau[j] = tau[j];
-      hs.c[j] = c[j];
-    }
-    hs.code = rc < 0 ? rc : 0;
+    hs.code = code;
     fired += f;
     drawn += dr;
   }
@@ -1250,7 +1356,7 @@ __device__ void aem_warp(AemSlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK,
 // stream (a function of the seed, the list index and the replicate only), so
 // that they can be fetched and computed ahead of the event.
 struct E1Rec {
-  int type, n, shift;
+  int type, n, shift, next;
   uint32_t mask;
   long long idx;
   double prop;
@@ -1260,12 +1366,14 @@ struct E1Rec {
 __device__ __forceinline__ E1Rec load_e1(const SgTables &tb, const EvDev &ev, long long j, int rep,
                                          uint32_t k0, uint32_t k1) {
   E1Rec r;
-  r.type = ev.type[j];
-  r.mask = tb.Emask[ev.select[j]];
-  r.n = ev.n[j];
-  r.shift = ev.shift[j];
-  r.idx = ev.index[j];
-  r.prop = ev.proportion[j];
+  const SgEvent e = load_event(ev.rec + j);
+  r.type = e.type;
+  r.mask = tb.Emask[e.select];
+  r.n = e.n;
+  r.shift = e.shift;
+  r.next = e.next;
+  r.idx = e.index;
+  r.prop = e.proportion;
   r.first = philox10(U4{0u, (uint32_t)(unsigned long long)r.idx,
                         (uint32_t)((unsigned long long)r.idx >> 32),
                         (SG_STREAM_EVENTS << 24) | (uint32_t)rep},
@@ -1388,6 +1496,42 @@ __device__ __forceinline__ int apply_e1_warp(int *u, const SgTables &tb, const E
   return 0;
 }
 
+// The E1 events of day index d of the unit of every lane with `pend`, in
+// (time, type, list index) order, from its next one `e` on (already loaded).
+// Warp-uniform: all 32 lanes call it.  Every round each lane with an event
+// left takes it, applied in the thread or (kUrnWarp or more individuals
+// drawn) by the whole warp.  ecur and next_day move along the node's list.
+// Returns the lane's error code (0 if none; e is then the event).
+template <int C>
+__device__ __forceinline__ int e1_events(bool pend, E1Rec &e, int *u, long long &ecur,
+                                         int &next_day, int d, const SgTables &tb,
+                                         const EvDev &ev, int rep, uint32_t k0, uint32_t k1,
+                                         unsigned long long &applied) {
+  const int lane = threadIdx.x & 31;
+  int code = 0;
+  while (__any_sync(0xffffffffu, pend)) {
+    const bool heavy = pend && e1_draws<C>(u, tb, e) >= kUrnWarp;
+    if (pend && !heavy) code = apply_e1<C>(u, tb, e, rep, k0, k1);
+    unsigned hm = __ballot_sync(0xffffffffu, heavy);
+    while (hm) {
+      const int L = __ffs(hm) - 1;
+      hm &= hm - 1;
+      const int rc = apply_e1_warp<C>(u, tb, e, L, rep, k0, k1);
+      if (lane == L) code = rc;
+    }
+    if (pend) {
+      if (code == 0) {
+        ++applied;
+        ++ecur;
+        next_day = e.next;
+      }
+      pend = code == 0 && next_day == d;
+      if (pend) e = load_e1(tb, ev, ecur, rep, k0, k1);
+    }
+  }
+  return code;
+}
+
 // Post time step and recording for unit time Tf (the state after its
 // events).  Returns 0 or SG_ERR_PTS.
 template <int KIND>
@@ -1444,23 +1588,18 @@ k_days(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
 #pragma unroll
   for (int p = 0; p < C; ++p) u[p] = 0;
   v[0] = 0.0;
-  long long ecur = 0, ebase = 0, eend = 0;
-  int next_day = 0x7fffffff;
+  long long ecur = 0, ebase = 0;
+  int next_day = SG_NO_DAY;
   double ch_a[AEM ? T : 1], ch_tau[AEM ? T : 1];  // all events method channels
   uint32_t ch_c[AEM ? T : 1];
   // static inputs first (they overlap the previous kernel's tail)
   if (in_range) {
     rep = (int)(gid / Nn);
     node = (int)(gid - (long long)rep * Nn);
-    if (NV > 0) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        ld[i] = season_end_int(a.ldata[(long long)node * tb.n_ldata + i]);
-    }
+    if (NV > 0) load_ends(a.ends, a.ldata, tb, node, ld);
     if (a.ev.e1_node_off) {
       const long long key = (long long)(a.slots > 1 ? rep : 0) * Nn + node;
       ebase = a.ev.e1_node_off[key];
-      eend = a.ev.e1_node_off[key + 1];
     }
   }
   pdl_wait();
@@ -1474,7 +1613,7 @@ k_days(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
     for (int q = 0; q < NV; ++q) v[q] = a.v[gid * NV + q];
     if (a.ev.e1_node_off) {
       ecur = ebase + a.e1_cur[gid];
-      if (ecur < eend) next_day = a.ev.e1_day[ecur];
+      next_day = a.e1_next[gid];
     }
     if constexpr (AEM) {
 #pragma unroll
@@ -1650,57 +1789,15 @@ k_days(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
         bad_day = Td;
       }
     }
-    // this node's E1 events of day Td, in (time, type, list index) order:
-    // each round every lane with an event left takes its next one, applied
-    // in the thread, or by the whole warp when it draws kUrnWarp or more
-    // individuals (every thread of the block reaches this loop)
+    // this node's E1 events of day Td (every thread of the block gets here)
     {
-      bool pend = e1_today && code == 0;
-      bool first = true;
-      const int lane = threadIdx.x & 31;
-      while (__any_sync(0xffffffffu, pend)) {
-        E1Rec e;
-        bool heavy = false;
-        if (pend) {
-          if (ecur < eend && a.ev.e1_day[ecur] == d) {
-            e = first ? pre : load_e1(tb, a.ev, ecur, grep, a.k0, a.k1);
-            first = false;
-            heavy = e1_draws<C>(u, tb, e) >= kUrnWarp;
-            if (!heavy) {
-              const int rc = apply_e1<C>(u, tb, e, grep, a.k0, a.k1);
-              if (rc) {
-                code = rc;
-                bad_day = Td;
-                bad_event = a.ev.index[ecur];
-                pend = false;
-              } else {
-                ++applied;
-                ++ecur;
-              }
-            }
-          } else {
-            pend = false;
-          }
-        }
-        unsigned hm = __ballot_sync(0xffffffffu, heavy);
-        while (hm) {
-          const int L = __ffs(hm) - 1;
-          hm &= hm - 1;
-          const int rc = apply_e1_warp<C>(u, tb, e, L, grep, a.k0, a.k1);
-          if (lane == L) {
-            if (rc) {
-              code = rc;
-              bad_day = Td;
-              bad_event = a.ev.index[ecur];
-              pend = false;
-            } else {
-              ++applied;
-              ++ecur;
-            }
-          }
-        }
+      const int rc = e1_events<C>(e1_today && code == 0, pre, u, ecur, next_day, d, tb, a.ev,
+                                  grep, a.k0, a.k1, applied);
+      if (rc) {
+        code = rc;
+        bad_day = Td;
+        bad_event = pre.idx;
       }
-      if (e1_today) next_day = ecur < eend ? a.ev.e1_day[ecur] : 0x7fffffff;
     }
     if (a.grid_bar && a.wave_off) {
       // persistent run: the day's external transfers between two grid
@@ -1747,7 +1844,10 @@ k_days(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
     for (int p = 0; p < C; ++p) a.u[gid * C + p] = u[p];
 #pragma unroll
     for (int q = 0; q < NV; ++q) a.v[gid * NV + q] = v[q];
-    if (a.ev.e1_node_off) a.e1_cur[gid] = (int32_t)(ecur - ebase);
+    if (a.ev.e1_node_off) {
+      a.e1_cur[gid] = (int32_t)(ecur - ebase);
+      a.e1_next[gid] = next_day;
+    }
     if constexpr (AEM) {
 #pragma unroll
       for (int j = 0; j < T; ++j) {
@@ -1845,12 +1945,6 @@ __device__ __forceinline__ bool quiescent(const int *u, const double *v) {
   }
 }
 
-__device__ __forceinline__ void load_ends(const DayArgs &a, const SgTables &tb, int node,
-                                          int *ld) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i) ld[i] = season_end_int(a.ldata[(long long)node * tb.n_ldata + i]);
-}
-
 // Recording of a unit whose post time step leaves it unchanged (tspan
 // slot m >= 0): dense U / V and the sparse entries.
 template <int C, int NV>
@@ -1894,7 +1988,7 @@ __device__ __forceinline__ int sparse_finish(int Tf, const int *u, double *v, bo
     return 0;
   }
   int ld[4] = {0, 0, 0, 0};
-  if (NV > 0) load_ends(a, tb, node, ld);
+  if (NV > 0) load_ends(a.ends, a.ldata, tb, node, ld);
   const int code = finish_step<KIND>(Tf, u, v, ld, tb, a, rep, node);
   if (code) report(a.err, code, a.rep0 + rep, node, Tf, -1);
 #pragma unroll
@@ -1903,91 +1997,51 @@ __device__ __forceinline__ int sparse_finish(int Tf, const int *u, double *v, bo
 }
 
 // E1 events of day index d (unit time Td) of the unit of every lane with
-// `has`, in (time, type, list index) order, for the sparse schedule (state
-// in device memory).  Warp-uniform: all 32 lanes call it.  Every round each
-// lane with an event left takes its next one, applied in the thread or
-// (kUrnWarp or more individuals drawn) by the whole warp.  Returns the
-// lane's error code (0 if none).
+// `has`, whose next event is of that day, for the sparse schedule (state in
+// device memory).  Warp-uniform.  Returns the lane's error code (0 if none).
 template <int C>
 __device__ __forceinline__ int sparse_e1(bool has, long long gid, int rep, int node, int Td,
                                          int d, const SgTables &tb, const DayArgs &a,
                                          uint32_t k0, uint32_t k1,
                                          unsigned long long &applied) {
-  const int lane = threadIdx.x & 31;
   const int Nn = tb.n_nodes;
-  long long ecur = 0, eend = 0, ebase = 0;
-  int code = 0;
-  int u[C];
+  long long ecur = 0, ebase = 0;
+  int u[C], next_day = d;
 #pragma unroll
   for (int p = 0; p < C; ++p) u[p] = 0;
+  const int grep = a.rep0 + rep;
+  E1Rec e;
   if (has) {
     const long long key = (long long)(a.slots > 1 ? rep : 0) * Nn + node;
     ebase = a.ev.e1_node_off[key];
-    eend = a.ev.e1_node_off[key + 1];
     ecur = ebase + a.e1_cur[gid];
 #pragma unroll
     for (int p = 0; p < C; ++p) u[p] = a.u[gid * C + p];
+    e = load_e1(tb, a.ev, ecur, grep, k0, k1);
   }
-  const int grep = a.rep0 + rep;
-  bool pend = has;
-  while (__any_sync(0xffffffffu, pend)) {
-    E1Rec e;
-    bool heavy = false;
-    if (pend) {
-      if (ecur < eend && a.ev.e1_day[ecur] == d) {
-        e = load_e1(tb, a.ev, ecur, grep, k0, k1);
-        heavy = e1_draws<C>(u, tb, e) >= kUrnWarp;
-        if (!heavy) {
-          const int rc = apply_e1<C>(u, tb, e, grep, k0, k1);
-          if (rc) {
-            code = rc;
-            report(a.err, rc, grep, node, Td, a.ev.index[ecur]);
-            pend = false;
-          } else {
-            ++applied;
-            ++ecur;
-          }
-        }
-      } else {
-        pend = false;
-      }
-    }
-    unsigned hm = __ballot_sync(0xffffffffu, heavy);
-    while (hm) {
-      const int L = __ffs(hm) - 1;
-      hm &= hm - 1;
-      const int rc = apply_e1_warp<C>(u, tb, e, L, grep, k0, k1);
-      if (lane == L) {
-        if (rc) {
-          code = rc;
-          report(a.err, rc, grep, node, Td, a.ev.index[ecur]);
-          pend = false;
-        } else {
-          ++applied;
-          ++ecur;
-        }
-      }
-    }
-  }
+  const int code =
+      e1_events<C>(has, e, u, ecur, next_day, d, tb, a.ev, grep, k0, k1, applied);
+  if (code) report(a.err, code, grep, node, Td, e.idx);
   if (has) {
 #pragma unroll
     for (int p = 0; p < C; ++p) a.u[gid * C + p] = u[p];
     a.e1_cur[gid] = (int32_t)(ecur - ebase);
-    a.e1_next[gid] = ecur < eend ? a.ev.e1_day[ecur] : 0x7fffffff;
+    a.e1_next[gid] = next_day;
   }
   return code;
 }
 
 // E1 events of day Td of the units marked in a chunk's bitmaps: units with
 // events today (e1bits) that took SSA draws (actbits) when `act`, else those
-// that did not.  A warp takes 32 words (1,024 units) at a time from *take,
+// that did not.  A warp takes `words` words (at most 32, of 32 units each) at a time from *take,
 // counts the marked units of each word, and gives the k-th marked unit of
 // the take to lane k mod 32 in round k / 32 (word by a search over the
 // warp's prefix counts, bit by halving), so the lanes stay full however
 // sparse the marks are.  Warp-uniform; called by every lane of a warp.
 template <int C>
 __device__ __forceinline__ void sparse_e1_bits(const uint32_t *e1bits, const uint32_t *actbits,
-                                               bool act, int *take, int nw, long long gbase,
+                                               bool act, int *take, int words, int nw,
+                                               long long gbase,
                                                int Td, int d, const SgTables &tb,
                                                const DayArgs &a, uint32_t k0, uint32_t k1,
                                                unsigned long long &applied) {
@@ -1995,12 +2049,12 @@ __device__ __forceinline__ void sparse_e1_bits(const uint32_t *e1bits, const uin
   const int Nn = tb.n_nodes;
   for (;;) {
     int g = 0;
-    if (lane == 0) g = atomicAdd(take, 32);
+    if (lane == 0) g = atomicAdd(take, words);
     g = __shfl_sync(0xffffffffu, g, 0);
     if (g >= nw) break;
     const int wi = g + lane;
     uint32_t m = 0;
-    if (wi < nw) m = e1bits[wi] & (act ? actbits[wi] : ~actbits[wi]);
+    if (lane < words && wi < nw) m = e1bits[wi] & (act ? actbits[wi] : ~actbits[wi]);
     const int cnt = __popc(m);
     int incl = cnt;
 #pragma unroll
@@ -2063,7 +2117,7 @@ struct UnitPos {
 };
 
 template <int KIND>
-__global__ void __launch_bounds__(kSparseBlock)
+__global__ void __launch_bounds__(kSparseBlock, 2)
 k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
   using M = ModelTraits<KIND>;
   constexpr int C = M::C, T = M::T, NV = M::NV, NK = M::NK;
@@ -2074,6 +2128,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
   __shared__ uint32_t s_actbits[kSparseChunk / 32];  // units taking SSA draws today
   __shared__ uint32_t s_e1bits[kSparseChunk / 32];   // units with E1 events today
   __shared__ int s_nact, s_nheavy, s_stop, s_next, s_nnq, s_e1take, s_e1late, s_nshort;
+  __shared__ __align__(16) E2Stage s_e2;  // the day's transfers of the block's first replicate
   pdl_trigger();
   const int Nn = tb.n_nodes;
   const long long total = (long long)Nn * a.n_rep;
@@ -2150,7 +2205,105 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
       //     +0) has an empty day and, at the launch's start, only its record
       //     of Td - 1 to write; the others are listed
       const int m_prev = fin_prev ? a.rec[Td - 1 - a.t0] : -1;
-      {
+      bool paired = false;
+      if constexpr (KIND != SG_SIR) {
+        // Compartments come in (S, I) pairs and nothing but dense output is
+        // recorded: the counts are read and recorded as they lie in memory,
+        // 8 bytes a lane, 256 consecutive bytes a warp instruction (a unit
+        // per lane touches each 32-byte sector up to six times: 5,000 units
+        // of 24 bytes took 14 us a day).  Every unit's counts are recorded
+        // here; the post time step of the listed ones changes phi only.
+        paired = !a.out.prev && a.out.u_nnz == 0 && a.out.v_nnz == 0 &&
+                 (((uintptr_t)a.U) & 7) == 0;
+        if (paired) {
+          constexpr int H = C / 2;  // pairs of a unit
+          UnitPos pos;              // the warp's first unit of the step
+          pos.set(g0 + c0 + warp * 32, Nn);
+          const int2 *state = reinterpret_cast<const int2 *>(a.u) + (g0 + c0) * H;
+#pragma unroll 1
+          for (int b0 = 0; b0 < cn; b0 += 4 * kSparseBlock) {
+            int2 w[4][H];
+            double v[4];
+            int nday[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const int ub = b0 + k * kSparseBlock + warp * 32, i = ub + lane;
+#pragma unroll
+              for (int j = 0; j < H; ++j) {
+                const int q = j * 32 + lane;
+                w[k][j] = make_int2(0, 0);
+                if (q < (cn - ub) * H) w[k][j] = state[(long long)ub * H + q];
+              }
+              v[k] = 0.0;
+              nday[k] = -1;
+              if (i < cn) {
+                if (NV > 0) v[k] = a.v[g0 + c0 + i];
+                if (has_e1) nday[k] = a.e1_next[g0 + c0 + i];
+              }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const int ub = b0 + k * kSparseBlock + warp * 32, i = ub + lane;
+              const bool in = i < cn;
+              // one bit per pair with an infected animal; a unit's H bits
+              uint32_t inf[3] = {0u, 0u, 0u};
+#pragma unroll
+              for (int j = 0; j < H; ++j) inf[j] = __ballot_sync(0xffffffffu, w[k][j].y != 0);
+              uint32_t mine;
+              if (H == 1) {
+                mine = (inf[0] >> lane) & 1u;
+              } else {
+                const int bit = 3 * lane;
+                const uint32_t lo = bit < 32 ? inf[0] : bit < 64 ? inf[1] : inf[2];
+                const uint32_t hi = bit < 32 ? inf[1] : bit < 64 ? inf[2] : 0u;
+                mine = __funnelshift_r(lo, hi, bit & 31) & 7u;
+              }
+              const bool q0 = in && quiet && mine == 0u && __double_as_longlong(v[k]) == 0;
+              const uint32_t bw = __ballot_sync(0xffffffffu, nday[k] == d);
+              const uint32_t lw = __ballot_sync(0xffffffffu, in && !q0);
+              int at = 0;
+              if (lane == 0) {
+                if (ub < kSparseChunk) s_e1bits[ub / 32] = bw;
+                if (lw) at = atomicAdd(&s_nnq, __popc(lw));
+              }
+              at = __shfl_sync(0xffffffffu, at, 0);
+              if (in && !q0) s_nq[at + __popc(lw & ((1u << lane) - 1u))] = (uint16_t)i;
+              if (m_prev >= 0 && ub < cn) {
+                // streaming stores: the trajectory leaves the state in L2
+                const long long unit =
+                    ((long long)pos.rep * a.M + m_prev) * Nn + pos.node;
+                if (pos.node + 32 <= Nn) {
+                  int2 *U = reinterpret_cast<int2 *>(a.U) + unit * H;
+#pragma unroll
+                  for (int j = 0; j < H; ++j) {
+                    const int q = j * 32 + lane;
+                    if (a.U && q < (cn - ub) * H) __stcs(U + q, w[k][j]);
+                  }
+                  if (NV > 0 && a.V && q0) __stcs(a.V + unit + lane, v[k]);
+                } else {
+#pragma unroll
+                  for (int j = 0; j < H; ++j) {
+                    const int q = j * 32 + lane, x = q / H;
+                    if (!a.U || ub + x >= cn) continue;
+                    UnitPos to = pos;
+                    to.advance(x, Nn);
+                    reinterpret_cast<int2 *>(
+                        a.U)[(((long long)to.rep * a.M + m_prev) * Nn + to.node) * H +
+                             (q - x * H)] = w[k][j];
+                  }
+                  if (NV > 0 && a.V && q0) {
+                    UnitPos to = pos;
+                    to.advance(lane, Nn);
+                    a.V[((long long)to.rep * a.M + m_prev) * Nn + to.node] = v[k];
+                  }
+                }
+              }
+              pos.advance(kSparseBlock, Nn);
+            }
+          }
+        }
+      }
+      if (!paired) {
         UnitPos pos;
         pos.set(g0 + c0 + tid, Nn);
 #pragma unroll 1
@@ -2271,9 +2424,15 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
         }
       }
       __syncthreads();
+      const int nw_e1 = (cn + 31) >> 5;
+      const int e1_words = min(32, max(2, (nw_e1 + 2 * nwarps - 1) / (2 * nwarps)));
       const int n_long = s_nact;
       const int na = n_long + s_nshort;
       const int n_direct = min(s_nheavy, kSparseHeavy);
+      if (a.e2_inblock && c0 == 0 && warp == nwarps - 1) {
+        const long long k = (long long)d * a.slots + (a.slots > 1 ? g0 / Nn : 0);
+        if (nub > 0) e2_stage(s_e2, a, a.wave_off[k], a.wave_off[k + 1]);
+      }
       // long days go to warps if there are few of them, else to the list's
       // front
       const bool own = n_direct > a.warp_max;
@@ -2344,11 +2503,13 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
         }
       }
       // a warp with no SSA work left applies the E1 events of day Td of the
-      // chunk's units that take no draw today (1,024 units per take, their
-      // units with events compacted onto the lanes); the units that take
+      // chunk's units that take no draw today (their units with events
+      // compacted onto the lanes; about two takes a warp, so that every warp
+      // gets some: a round of events is a chain of memory latencies); the
+      // units that take
       // draws come after the SSA (their events follow their day's
       // transitions)
-      if (has_e1) sparse_e1_bits<C>(s_e1bits, s_actbits, false, &s_e1take, (cn + 31) >> 5,
+      if (has_e1) sparse_e1_bits<C>(s_e1bits, s_actbits, false, &s_e1take, e1_words, nw_e1,
                                     g0 + c0, Td, d, tb, a, k0, k1, applied);
       __syncthreads();
       // the warp slots not run yet: all of them when every warp had list
@@ -2371,7 +2532,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
       __syncthreads();
       // 3. E1 events of day Td of the units that took draws today
       if (has_e1) {
-        sparse_e1_bits<C>(s_e1bits, s_actbits, true, &s_e1late, (cn + 31) >> 5, g0 + c0, Td,
+        sparse_e1_bits<C>(s_e1bits, s_actbits, true, &s_e1late, e1_words, nw_e1, g0 + c0, Td,
                           d, tb, a, k0, k1, applied);
         __syncthreads();
       }
@@ -2379,15 +2540,24 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
     if (a.e2_inblock) {
       // this block's replicates' external transfers of Td (the wave plan of
       // day d; no other block touches their nodes)
-      for (long long r = g0 / Nn; nub > 0 && r * Nn < g0 + nub; ++r) {
-        const long long k = (long long)d * a.slots + (a.slots > 1 ? r : 0);
-        const long long w0 = a.wave_off[k], w1 = a.wave_off[k + 1];
-        if (w0 < w1) e2_rep_block<C>(tb, a, (int)r, Td, w0, w1);
-      }
-      // a failed transfer ends the run before the day's post time step
-      if (tid == 0) s_stop = *(volatile int32_t *)&a.err->code != 0;
+      asm volatile("cp.async.wait_all;" ::: "memory");
       __syncthreads();
-      if (s_stop) break;
+      for (long long r = g0 / Nn; nub > 0 && r * Nn < g0 + nub; ++r) {
+        long long w0 = s_e2.w0, w1 = s_e2.w1;
+        if (a.slots > 1 && r != g0 / Nn) {
+          const long long k = (long long)d * a.slots + r;
+          w0 = a.wave_off[k];
+          w1 = a.wave_off[k + 1];
+        }
+        if (w0 < w1) e2_rep_block<C>(tb, a, (int)r, Td, w0, w1, &s_e2);
+      }
+      // a failed transfer ends the run before the day's post time step (of
+      // which the next day's check takes care but on the last one)
+      if (Td + 1 == a.T_end) {
+        if (tid == 0) s_stop = *(volatile int32_t *)&a.err->code != 0;
+        __syncthreads();
+        if (s_stop) break;
+      }
     }
     // then, unless deferred to the next day's first passes or the next
     // launch, the post time step and recording of Td for every unit
@@ -2506,8 +2676,8 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
   }
 }
 
-// Day index of each unit's first E1 event (or 0x7fffffff), the sparse
-// schedule's per-unit test for "events today" (its E1 cursors start at 0).
+// Day index of each unit's first E1 event (or SG_NO_DAY), the per-unit test
+// for "events today" (the E1 cursors start at 0).
 __global__ void k_e1_next_init(const int64_t *__restrict__ e1_node_off,
                                const int32_t *__restrict__ e1_day, int Nn, int n_rep,
                                int slots, int32_t *e1_next) {
@@ -2517,7 +2687,7 @@ __global__ void k_e1_next_init(const int64_t *__restrict__ e1_node_off,
     const int rep = (int)(g / Nn), node = (int)(g - (long long)rep * Nn);
     const long long key = (long long)(slots > 1 ? rep : 0) * Nn + node;
     const long long b = e1_node_off[key], e = e1_node_off[key + 1];
-    e1_next[g] = b < e ? e1_day[b] : 0x7fffffff;
+    e1_next[g] = b < e ? e1_day[b] : SG_NO_DAY;
   }
 }
 
@@ -2611,13 +2781,14 @@ k_events_e2(const SgTables tb, const EvArgs a, const int64_t *__restrict__ wave_
     const long long pend = min(pos + (long long)kE2Cap, s_wave[wn]);
     for (long long i = threadIdx.x; i < pend - pos; i += blockDim.x) {
       const long long j = pos + i;
-      s_node[i] = a.ev.node[j];
-      s_dest[i] = a.ev.dest[j];
-      s_n[i] = a.ev.n[j];
-      s_sel[i] = a.ev.select[j];
-      s_shift[i] = a.ev.shift[j];
-      s_prop[i] = a.ev.proportion[j];
-      const long long idx = a.ev.index[j];
+      const SgEvent ev = load_event(a.ev.rec + j);
+      s_node[i] = ev.node;
+      s_dest[i] = ev.dest;
+      s_n[i] = ev.n;
+      s_sel[i] = ev.select;
+      s_shift[i] = ev.shift;
+      s_prop[i] = ev.proportion;
+      const long long idx = ev.index;
       s_idx[i] = idx;
       const U4 f = philox10(U4{0u, (uint32_t)(unsigned long long)idx,
                                (uint32_t)((unsigned long long)idx >> 32), tag},

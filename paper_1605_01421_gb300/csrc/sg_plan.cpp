@@ -356,23 +356,30 @@ int build_plan(const EventTable &ev, int32_t n_nodes, int32_t t0, int32_t t_end,
   return SG_OK;
 }
 
-void gather_events(const EventTable &ev, const Plan &P, int8_t *type, int8_t *shift,
-                   uint8_t *select, int32_t *node, int32_t *dest, int32_t *n, double *proportion,
-                   int64_t *index) {
+void gather_events(const EventTable &ev, const Plan &P, SgEvent *out) {
   const int64_t m = (int64_t)P.order.size();
   const int T = plan_threads(m);
   run_threads(T, [&](int t) {
     const int64_t lo = m * t / T, hi = m * (t + 1) / T;
     for (int64_t i = lo; i < hi; ++i) {
       const int64_t e = P.order[i];
-      type[i] = (int8_t)ev.type[e];
-      shift[i] = (int8_t)(ev.shift[e] < 0 ? -1 : ev.shift[e]);
-      select[i] = (uint8_t)ev.select[e];
-      node[i] = ev.node[e];
-      dest[i] = ev.dest[e];
-      n[i] = ev.n[e];
-      proportion[i] = ev.proportion[e];
-      index[i] = e;
+      SgEvent r{};
+      r.node = ev.node[e];
+      r.dest = ev.dest[e];
+      r.n = ev.n[e];
+      r.type = (int8_t)ev.type[e];
+      r.select = (uint8_t)ev.select[e];
+      r.shift = (int8_t)(ev.shift[e] < 0 ? -1 : ev.shift[e]);
+      r.proportion = ev.proportion[e];
+      r.index = e;
+      if (i < P.n_e1) {
+        // the next event of the same list, if any, has the same node and
+        // slot (lists are consecutive and never empty between two events)
+        const bool more = i + 1 < P.n_e1 && ev.node[P.order[i + 1]] == ev.node[e] &&
+                          (P.slots == 1 || ev.rep[P.order[i + 1]] == ev.rep[e]);
+        r.next = more ? P.e1_day[i + 1] : SG_NO_DAY;
+      }
+      out[i] = r;
     }
   });
 }
