@@ -1928,7 +1928,8 @@ k_days(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
 // ---------------------------------------------------------------------------
 constexpr int kSparseBlock = 256;   // threads of the sparse-schedule day kernel
 constexpr int kSparseChunk = 8192;  // units per pass through the active list
-constexpr int kSparseHeavy = 64;    // warp hand-off slots per pass
+constexpr int kSparseHeavy = 64;    // warp hand-off slots per pass, of which long
+constexpr int kSparseDirect = 48;   // days take at most these; the others are for redone days
 
 // A unit whose day is certainly empty: no infected animal and phi == +0
 // (bit pattern 0).  Exact only with finite model parameters (DayArgs::quiet).
@@ -2127,7 +2128,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
   __shared__ HeavySlot<C, NK> s_heavy[kSparseHeavy];
   __shared__ uint32_t s_actbits[kSparseChunk / 32];  // units taking SSA draws today
   __shared__ uint32_t s_e1bits[kSparseChunk / 32];   // units with E1 events today
-  __shared__ int s_nact, s_nheavy, s_stop, s_next, s_nnq, s_e1take, s_e1late, s_nshort;
+  __shared__ int s_nact, s_nheavy, s_stop, s_next, s_nnq, s_e1take, s_e1late, s_nshort, s_nredo;
   __shared__ __align__(16) E2Stage s_e2;  // the day's transfers of the block's first replicate
   pdl_trigger();
   const int Nn = tb.n_nodes;
@@ -2197,6 +2198,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
         s_e1take = 0;
         s_e1late = 0;
         s_nshort = 0;
+        s_nredo = 0;
       }
       for (int q = tid; q < kSparseChunk / 32; q += kSparseBlock) s_actbits[q] = 0u;
       __syncthreads();
@@ -2400,9 +2402,9 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
               report(a.err, SG_ERR_RATE, a.rep0 + rep, node, Td, -1);
             } else if (fires) {
               atomicOr(&s_actbits[(i - c0) >> 5], 1u << ((i - c0) & 31));
-              int slot = kSparseHeavy;
+              int slot = kSparseDirect;
               if (!(lam < a.warp_rate)) slot = atomicAdd(&s_nheavy, 1);
-              if (slot < kSparseHeavy) {
+              if (slot < kSparseDirect) {
                 HeavySlot<C, NK> &hs = s_heavy[slot];
 #pragma unroll
                 for (int q = 0; q < NK; ++q) hs.kf[q] = kf[q];
@@ -2428,7 +2430,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
       const int e1_words = min(32, max(2, (nw_e1 + 2 * nwarps - 1) / (2 * nwarps)));
       const int n_long = s_nact;
       const int na = n_long + s_nshort;
-      const int n_direct = min(s_nheavy, kSparseHeavy);
+      const int n_direct = min(s_nheavy, kSparseDirect);
       if (a.e2_inblock && c0 == 0 && warp == nwarps - 1) {
         const long long k = (long long)d * a.slots + (a.slots > 1 ? g0 / Nn : 0);
         if (nub > 0) e2_stage(s_e2, a, a.wave_off[k], a.wave_off[k + 1]);
@@ -2480,7 +2482,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
                          : ssa_exact<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1,
                                            a.heavy_after, tb, fired, drawn);
           if (r == SSA_REDO) {
-            if (slot < 0) slot = atomicAdd(&s_nheavy, 1);
+            if (slot < 0) slot = n_direct + atomicAdd(&s_nredo, 1);
             if (slot < kSparseHeavy) {
               HeavySlot<C, NK> &hs = s_heavy[slot];
 #pragma unroll
@@ -2515,7 +2517,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
       // the warp slots not run yet: all of them when every warp had list
       // units, else those the thread list handed over
       const int h0 = list_warps < nwarps && !own ? n_direct : 0;
-      const int nh = min(s_nheavy, kSparseHeavy);
+      const int nh = min(n_direct + s_nredo, kSparseHeavy);
       for (int h = h0 + warp; h < nh; h += nwarps) {
         HeavySlot<C, NK> &hs = s_heavy[h];
         if (hs.rep < 0) continue;
