@@ -56,6 +56,10 @@ L2_BYTES = 129 * 2 ** 20
 #     inversion (T - 1 at most), the rates column n of G marks and the new
 #     lambda (SISe3: 1 + 5 + 5 + 5; SISe: 1 + 1 + 5 + 1; SIS 1 + 1 + 6 + 1;
 #     SIR 1 + 1 + 10 + 1).
+# The kernels take most of a draw's decisions from FP32 intervals that enclose
+# these FP64 values (same results), so the operations counted here are the
+# method's, not FP64 instructions issued, and their rate may pass the FP64
+# instruction rate where every herd is active.
 # Parsed models (transition strings) have no fixed count: no FP64 roofline.
 FP64_OPS = {  # kind: (per node-day, per draw, per transition)
     0: (11, 46, 13),   # SIR
@@ -599,7 +603,9 @@ def bench_gpu(args):
         node_days_job = (w_full.n_nodes * w_full.n_days * w_full.n_rep if sharded
                          else w.n_nodes * w.n_days * n_rep * world)
         e2e = {"value": node_days_job * n_e2e / t_e2e, "unit": UNIT,
-               "h2d_bytes_per_step": int(u0h.nbytes + v0h.nbytes + w.n_events * 35),
+               # a 32-byte record per event, the day of each but the transfers
+               "h2d_bytes_per_step": int(u0h.nbytes + v0h.nbytes + w.n_events * 32
+                                         + 4 * np.count_nonzero(w.events["event"] != 3)),
                "d2h_bytes_per_step": int(Uh.nbytes + Vh.nbytes), "steps": n_e2e,
                "what": "sg_run_host with model creation, event upload and planning per step"}
         del Uh, Vh

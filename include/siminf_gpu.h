@@ -338,11 +338,11 @@ int sg_set_replicate_range(sg_model *m, int32_t rep0, int32_t rep_total);
 int sg_set_tuning(sg_model *m, int32_t nodes_per_block, int32_t heavy_after);
 
 /* Autotuner: for each of nodes_per_block in {4, 8, 16, 32, 64, 128} x
- * heavy_after in {0, 1, 2, 4, 8}, and, where the sparse-activity schedule
+ * heavy_after in {0, 2, 8, 64, 2^20}, and, where the sparse-activity schedule
  * applies, nodes_per_block = the pairs spread over 1, 2 or 4 blocks per SM,
  * 1,024, and one or two whole replicates (when above 128; replicates per
  * block such that at least half a block per SM exists) x heavy_after in
- * {2, 8, 16, 32, 128}, runs the given
+ * {8, 16, 32, 128, 2^20}, runs the given
  * workload (arguments as sg_run) once untimed (capturing its graph when
  * graphs are on) and twice timed, keeps the setting with the fastest timed
  * run in the model and reports it and its time (outputs may be NULL).  U and
@@ -554,6 +554,17 @@ int sg_absmax_bf16(const void *x, int64_t n, float *out, void *stream);
  * d loss / d logits / B as BF16 (leading dimension ldd; columns 387.. are 0). */
 int sg_mlp_ce_loss(const float *logits, int32_t ldl, const int32_t *targets, int32_t B,
                    void *dlogits, int32_t ldd, double *loss_sum, void *stream);
+/* The network's layers over B rows in one call.  BF16: act[l] (l < 3, B x 256
+ * BF16) and logits (B x 392 FP32) are written, and, with pre not NULL, the
+ * pre-activations pre[l] (B x 256 FP32).  E4M3: layer 1 from BF16 operands
+ * W0, layers 2-4 from W8[l] with row scales wscale[l] and input scales
+ * act_scale[l]; buf_a, buf_b: B x 256 bytes each. */
+int sg_mlp_forward(const void *feat, int32_t B, const void *const *W, const float *const *b,
+                   void *const *act, float *const *pre, float *logits, void *stream);
+int sg_mlp_forward_fp8(const void *feat, int32_t B, const void *W0, const void *const *W8,
+                       const float *const *wscale, const float *act_scale,
+                       const float *const *b, void *buf_a, void *buf_b, float *logits,
+                       void *stream);
 /* Mean cross-entropy gradients of the network over B rows (a multiple of 8)
  * in one call: forward pass, loss, backward pass.  feat: B x 16 BF16;
  * targets: B x 3 int32; W[l], b[l] (l < 4): BF16 weights (out x in) and FP32

@@ -171,7 +171,7 @@ EXPORTS = ["sg_model_create", "sg_set_events", "sg_run", "sg_run_host",
            "sg_run_noalloc", "sg_set_tuning", "sg_autotune", "sg_set_graphs",
            "sg_gemm_bf16", "sg_mlp_ce_loss", "sg_gelu_backward", "sg_transpose_bf16",
            "sg_colsum_bf16", "sg_adam_step", "sg_emu_features", "sg_emu_targets",
-           "sg_emu_sample", "sg_mlp_gradients", "sg_mlp_gradients_scratch",
+           "sg_emu_sample", "sg_mlp_forward", "sg_mlp_forward_fp8", "sg_mlp_gradients", "sg_mlp_gradients_scratch",
            "sg_emulator_set", "sg_set_neighbors", "sg_set_solver",
            "sg_set_output", "sg_model_create_parsed", "sg_model_tables",
            "sg_set_fused_events", "sg_set_persistent", "sg_gemm_fp8", "sg_quant_fp8_rows",
@@ -257,6 +257,11 @@ def lib(path: str | None = None):
         pp = ctypes.POINTER(vp)
         L.sg_mlp_gradients.argtypes = [vp, vp, i32, pp, pp, pp, pp, vp, vp, i64, vp]
         L.sg_mlp_gradients.restype = ctypes.c_int
+        L.sg_mlp_forward.argtypes = [vp, i32, pp, pp, pp, pp, vp, vp]
+        L.sg_mlp_forward.restype = ctypes.c_int
+        L.sg_mlp_forward_fp8.argtypes = [vp, i32, vp, pp, pp, ctypes.POINTER(f32), pp, vp, vp,
+                                         vp, vp]
+        L.sg_mlp_forward_fp8.restype = ctypes.c_int
         L.sg_mlp_gradients_scratch.argtypes = [i32]
         L.sg_mlp_gradients_scratch.restype = i64
         L.sg_gelu_backward.argtypes = [vp, vp, i64, vp, vp]

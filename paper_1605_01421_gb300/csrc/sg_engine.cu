@@ -2093,14 +2093,15 @@ extern "C" int sg_autotune(sg_model *m, const int32_t *tspan, int32_t n_tspan, u
                            int32_t *d_U, double *d_V, void *stream, int32_t *npb_out,
                            int32_t *heavy_after_out, double *ms_out) {
   if (!m) return SG_ERR_ARG;
-  // 4 and 8 nodes per block give every heavy node its own warp (workloads
-  // where most node-days take thousands of draws); more than kDayBlock
+  // 4 and 8 nodes per block give every long day its own warp (workloads
+  // where most node-days take thousands of draws), the largest hand-over
+  // leaves every day to its thread; more than kDayBlock
   // selects the sparse-activity schedule: units spread over 1, 2 or 4
   // blocks per SM, fixed 1,024-unit blocks, or one or two whole replicates
   // per block
   std::vector<std::pair<int32_t, int32_t>> cand;
   for (int32_t npb : {4, 8, 16, 32, 64, 128})
-    for (int32_t h : {0, 1, 2, 4, 8}) cand.emplace_back(npb, h);
+    for (int32_t h : {0, 2, 8, 64, 1 << 20}) cand.emplace_back(npb, h);
   {
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -2127,7 +2128,7 @@ extern "C" int sg_autotune(sg_model *m, const int32_t *tspan, int32_t n_tspan, u
                            (k == SG_SIR || k == SG_SIS || k == SG_SISE || k == SG_SISE3);
     if (!sparse_ok) sp.clear();
     for (int32_t npb : sp)
-      for (int32_t h : {2, 8, 16, 32, 128}) cand.emplace_back(npb, h);
+      for (int32_t h : {8, 16, 32, 128, 1 << 20}) cand.emplace_back(npb, h);
   }
   cudaStream_t st = (cudaStream_t)stream;
   cudaEvent_t e0, e1;

@@ -228,9 +228,10 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
   }
   if (ok) {
     // Epilogue.  Warp w reads TMEM lanes 32 (w % 4) .. + 31 (tile rows) and
-    // the columns of half w / 4.  FP32 results go out as 16-byte vectors;
-    // BF16 results are staged in shared memory (the stage buffers are free
-    // now) and then written row by row, each warp storing whole rows.
+    // half w / 4 of each 64 columns.  Results are staged in shared memory (the
+    // stage buffers are free now) and then written row by row, each warp
+    // storing whole row segments: a lane holds a tile row, so its own stores
+    // would be 16 bytes each, 32 rows apart (100,000 x 392 logits: 125 us).
     tc::tc_fence_after();
     constexpr int kPitch = BN * 2 + 16;  // bytes per staged row (bank offset)
     unsigned char *stage = smem;
@@ -238,13 +239,39 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
     const int lr = q * 32 + lane;
     const int row = m0 + lr;
     const bool vec32 = g.C32 && (g.ldc32 % 4) == 0 && (((uintptr_t)g.C32) & 15) == 0;
-    for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 16) {
+    constexpr int kPitch32 = 64 + 4;     // floats per staged row of 64 columns
+    constexpr int kPitch8 = BN + 16;     // bytes per staged E4M3 row
+    constexpr int kStage16 = kBM * kPitch, kStage32 = kBM * kPitch32 * 4;
+    constexpr int kSmem = NBUF * (kAStage + kBStage);
+    // what fits beside each other (wide tiles: not FP32 or E4M3 beside BF16)
+    const bool st32 = vec32 && (!g.C16 || kStage16 + kStage32 <= kSmem);
+    const bool st8 = g.C8 && !g.C16 && (g.ldc8 % 16) == 0 && (((uintptr_t)g.C8) & 15) == 0 &&
+                     kStage32 + kBM * kPitch8 <= kSmem;
+    float *stage32 = reinterpret_cast<float *>(smem + (g.C16 ? kStage16 : 0));
+    unsigned char *stage8 = smem + kStage32;
+    for (int cb = 0; cb < BN; cb += 64) {
+    for (int c = cb + half * 32; c < cb + half * 32 + 32; c += 16) {
       float v[16];
       tc::tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c, v);
       const int nb = n0 + c;
       // pre-activation: accumulator x a_scale b_scale[n] (E4M3) + bias[n],
       // one fused multiply-add
-      float bs[16];
+      float bs[16], sc[16];
+      if constexpr (F8) {
+        if (nb + 16 <= g.N && (((uintptr_t)(g.b_scale + nb)) & 15) == 0) {
+#pragma unroll
+          for (int i = 0; i < 16; i += 4) {
+            const float4 s4 = __ldg(reinterpret_cast<const float4 *>(g.b_scale + nb + i));
+            sc[i] = s4.x;
+            sc[i + 1] = s4.y;
+            sc[i + 2] = s4.z;
+            sc[i + 3] = s4.w;
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) sc[i] = nb + i < g.N ? __ldg(g.b_scale + nb + i) : 0.0f;
+        }
+      }
       if (g.bias && nb + 16 <= g.N && (((uintptr_t)(g.bias + nb)) & 15) == 0) {
 #pragma unroll
         for (int i = 0; i < 16; i += 4) {
@@ -261,10 +288,15 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         float cs = 1.0f;
-        if constexpr (F8) cs = g.a_scale * ((nb + i < g.N) ? __ldg(g.b_scale + nb + i) : 0.0f);
+        if constexpr (F8) cs = g.a_scale * sc[i];
         v[i] = __fmaf_rn(v[i], cs, bs[i]);
       }
-      if (g.C32 && row < g.M) {
+      if (st32) {
+#pragma unroll
+        for (int i = 0; i < 16; i += 4)
+          *reinterpret_cast<float4 *>(stage32 + lr * kPitch32 + (c - cb) + i) =
+              make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+      } else if (g.C32 && row < g.M) {
         float *dst = g.C32 + (long long)row * g.ldc32 + nb;
         if (vec32 && nb + 16 <= g.N) {
 #pragma unroll
@@ -312,7 +344,7 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
         sp[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
         sp[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
       }
-      if (g.C8 && row < g.M) {
+      if (g.C8 && (st8 || row < g.M)) {
         // 16 E4M3 values of this row (the output scale folded into the
         // activation), one 16-byte store when it fits
         const float hs = 0.5f * g.c8_inv_scale;
@@ -323,11 +355,49 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
         const uint4 pk = pack_e4m3_16(y);
         const uint32_t packed[4] = {pk.x, pk.y, pk.z, pk.w};
         uint8_t *dst = g.C8 + (long long)row * g.ldc8 + nb;
-        if (nb + 16 <= g.N && (((uintptr_t)dst) & 15) == 0) {
+        if (st8) {
+          *reinterpret_cast<uint4 *>(stage8 + lr * kPitch8 + c) = pk;
+        } else if (nb + 16 <= g.N && (((uintptr_t)dst) & 15) == 0) {
           *reinterpret_cast<uint4 *>(dst) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
         } else {
           const uint8_t *bytes = reinterpret_cast<const uint8_t *>(packed);
           for (int i = 0; i < 16 && nb + i < g.N; ++i) dst[i] = bytes[i];
+        }
+      }
+    }
+    if (st32) {
+      // 64 columns of every row: 16 lanes a row
+      __syncthreads();
+      for (int idx = tid; idx < kBM * 16; idx += kGemmThreads) {
+        const int r = idx >> 4, j = (idx & 15) * 4;
+        const int grow = m0 + r, col = n0 + cb + j;
+        if (grow >= g.M || col >= g.N) continue;
+        const float4 val = *reinterpret_cast<const float4 *>(stage32 + r * kPitch32 + j);
+        float *dst = g.C32 + (long long)grow * g.ldc32 + col;
+        if (col + 4 <= g.N) {
+          *reinterpret_cast<float4 *>(dst) = val;
+        } else {
+          const float x[4] = {val.x, val.y, val.z, val.w};
+          for (int i = 0; i < 4 && col + i < g.N; ++i) dst[i] = x[i];
+        }
+      }
+      __syncthreads();
+    }
+    }
+    if (st8) {
+      __syncthreads();
+      constexpr int kVecPerRow = BN / 16;
+      for (int idx = tid; idx < kBM * kVecPerRow; idx += kGemmThreads) {
+        const int r = idx / kVecPerRow, j = (idx - r * kVecPerRow) * 16;
+        const int grow = m0 + r, col = n0 + j;
+        if (grow >= g.M || col >= g.N) continue;
+        const uint4 val = *reinterpret_cast<const uint4 *>(stage8 + r * kPitch8 + j);
+        uint8_t *dst = g.C8 + (long long)grow * g.ldc8 + col;
+        if (col + 16 <= g.N) {
+          *reinterpret_cast<uint4 *>(dst) = val;
+        } else {
+          const uint8_t *x = reinterpret_cast<const uint8_t *>(&val);
+          for (int i = 0; i < 16 && col + i < g.N; ++i) dst[i] = x[i];
         }
       }
     }
@@ -1522,6 +1592,68 @@ struct GradScratch {
 };
 
 }  // namespace
+
+extern "C" int sg_mlp_forward(const void *feat, int32_t B, const void *const *W,
+                              const float *const *b, void *const *act, float *const *pre,
+                              float *logits, void *stream) {
+  if (B < 0 || !W || !b || !act || (B > 0 && (!feat || !logits))) return SG_ERR_ARG;
+  cudaStream_t st = (cudaStream_t)stream;
+  const void *x = feat;
+  for (int l = 0; l < 4; ++l) {
+    GemmArgs g{};
+    g.A = (const __nv_bfloat16 *)x;
+    g.Bt = (const __nv_bfloat16 *)W[l];
+    g.lda = g.ldb = g.K = kLayerIn[l];
+    g.M = B;
+    g.N = g.ldc32 = g.ldc16 = kLayerOut[l];
+    g.bias = b[l];
+    g.act = l < 3 ? 1 : 0;
+    g.C32 = l == 3 ? logits : pre ? pre[l] : nullptr;
+    g.C16 = l < 3 ? (__nv_bfloat16 *)act[l] : nullptr;
+    const int rc = sg::gemm_bf16(g, st);
+    if (rc) return rc;
+    if (l < 3) x = act[l];
+  }
+  return sg::gemm_check(st);
+}
+
+extern "C" int sg_mlp_forward_fp8(const void *feat, int32_t B, const void *W0,
+                                  const void *const *W8, const float *const *wscale,
+                                  const float *act_scale, const float *const *b, void *buf_a,
+                                  void *buf_b, float *logits, void *stream) {
+  if (B < 0 || !W0 || !W8 || !wscale || !act_scale || !b ||
+      (B > 0 && (!feat || !buf_a || !buf_b || !logits)))
+    return SG_ERR_ARG;
+  cudaStream_t st = (cudaStream_t)stream;
+  uint8_t *bufs[2] = {(uint8_t *)buf_a, (uint8_t *)buf_b};
+  for (int l = 0; l < 4; ++l) {
+    GemmArgs g{};
+    g.lda = g.ldb = g.K = kLayerIn[l];
+    g.M = B;
+    g.N = g.ldc32 = g.ldc8 = kLayerOut[l];
+    g.bias = b[l];
+    if (l == 0) {
+      g.A = (const __nv_bfloat16 *)feat;
+      g.Bt = (const __nv_bfloat16 *)W0;
+    } else {
+      g.f8 = 1;
+      g.A8 = bufs[(l - 1) & 1];
+      g.B8 = (const uint8_t *)W8[l - 1];
+      g.a_scale = act_scale[l - 1];
+      g.b_scale = wscale[l - 1];
+    }
+    if (l < 3) {
+      g.act = 1;
+      g.C8 = bufs[l & 1];
+      g.c8_inv_scale = 1.0f / act_scale[l];
+    } else {
+      g.C32 = logits;
+    }
+    const int rc = sg::gemm_bf16(g, st);
+    if (rc) return rc;
+  }
+  return sg::gemm_check(st);
+}
 
 extern "C" int64_t sg_mlp_gradients_scratch(int32_t B) {
   return B < 0 ? 0 : (int64_t)GradScratch(nullptr, (size_t)B).bytes;

@@ -32,6 +32,10 @@ def _p(t):
     return ctypes.c_void_p(t.data_ptr()) if t is not None else None
 
 
+def _ptrs(ts):
+    return (ctypes.c_void_p * len(ts))(*[t.data_ptr() for t in ts])
+
+
 def _s():
     return binding._stream_handle(None)
 
@@ -69,17 +73,16 @@ class Emulator:
     def forward(self, feat16, keep=False):
         """Logits (B x 392 FP32); with keep=True also the activations and
         pre-activations the backward pass needs."""
-        x = feat16
-        acts, pres = [feat16], []
-        for li in range(3):
-            pre, post = binding.gemm_bf16(x, self.W16[li], bias=self.b32[li], act=1,
-                                          out32=keep, out16=True)
-            pres.append(pre)
-            acts.append(post)
-            x = post
-        logits, _ = binding.gemm_bf16(x, self.W16[3], bias=self.b32[3], act=0,
-                                      out32=True, out16=False)
-        return logits, acts, pres
+        torch = self.torch
+        B, dev = feat16.shape[0], feat16.device
+        new = lambda n, t: torch.empty((B, n), dtype=t, device=dev)  # noqa: E731
+        post = [new(HID, torch.bfloat16) for _ in range(3)]
+        pres = [new(HID, torch.float32) if keep else None for _ in range(3)]
+        logits = new(NOUT, torch.float32)
+        _check(binding.lib().sg_mlp_forward(
+            binding._dev_ptr(feat16, torch.bfloat16, (B, NIN), "feat16"), B, _ptrs(self.W16),
+            _ptrs(self.b32), _ptrs(post), _ptrs(pres) if keep else None, _p(logits), _s()))
+        return logits, [feat16, *post], pres
 
     # -- FP8 inference ---------------------------------------------------------
     def quantize_fp8(self, calib_feat16, margin=1.0):
@@ -98,21 +101,17 @@ class Emulator:
         self.act_scale = [float(f32(max(binding.absmax_bf16(a), 1e-30) * margin) / f32(448.0))
                           for a in acts[1:4]]
 
-    def _inv(self, li):
-        # the same single-precision reciprocal the engine takes
-        return float(np.float32(1.0) / np.float32(self.act_scale[li]))
-
     def forward_fp8(self, feat16):
         """Logits (B x 392 FP32) of the E4M3 network: the same kernels and
         arguments the engine uses when FP8 inference is switched on."""
-        x8 = binding.gemm_bf16_to_fp8(feat16, self.W16[0], self._inv(0), bias=self.b32[0],
-                                      act=1)
-        for li in (1, 2):
-            _, _, x8 = binding.gemm_fp8(x8, self.act_scale[li - 1], self.W8[li - 1],
-                                        self.wscale[li - 1], bias=self.b32[li], act=1,
-                                        out32=False, out8_inv_scale=self._inv(li))
-        logits, _, _ = binding.gemm_fp8(x8, self.act_scale[2], self.W8[2], self.wscale[2],
-                                        bias=self.b32[3], act=0, out32=True)
+        torch = self.torch
+        B, dev = feat16.shape[0], feat16.device
+        bufs = [torch.empty((B, HID), dtype=torch.uint8, device=dev) for _ in range(2)]
+        logits = torch.empty((B, NOUT), dtype=torch.float32, device=dev)
+        _check(binding.lib().sg_mlp_forward_fp8(
+            binding._dev_ptr(feat16, torch.bfloat16, (B, NIN), "feat16"), B, _p(self.W16[0]),
+            _ptrs(self.W8), _ptrs(self.wscale), (ctypes.c_float * 3)(*self.act_scale),
+            _ptrs(self.b32), _p(bufs[0]), _p(bufs[1]), _p(logits), _s()))
         return logits
 
     # -- backward ------------------------------------------------------------
@@ -128,12 +127,9 @@ class Emulator:
         nb = int(L.sg_mlp_gradients_scratch(B))
         scratch = torch.empty(nb, dtype=torch.uint8, device=self.device)
 
-        def ptrs(ts):
-            return (ctypes.c_void_p * 4)(*[t.data_ptr() for t in ts])
-
         _check(L.sg_mlp_gradients(
             binding._dev_ptr(feat16, torch.bfloat16, (B, NIN), "feat16"),
-            _p(targets), B, ptrs(self.W16), ptrs(self.b32), ptrs(dW), ptrs(db), _p(loss),
+            _p(targets), B, _ptrs(self.W16), _ptrs(self.b32), _ptrs(dW), _ptrs(db), _p(loss),
             _p(scratch), nb, _s()))
         return float(loss.item()) / B, dW, db
 
