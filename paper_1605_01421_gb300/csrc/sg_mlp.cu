@@ -98,9 +98,10 @@ __device__ __forceinline__ uint4 pack_e4m3_16(const float *y) {
 //
 // Training epilogues: with bwd_pre the value is multiplied by GELU's
 // derivative at bwd_pre (the gradient through an activation), and C16T takes
-// a transposed copy of C16 (32 consecutive rows per store of a warp).
+// a transposed copy of C16 in the tiled layout below.
 constexpr int kGemmThreads = 256;
 __device__ __forceinline__ float gelu_grad(float x);
+__device__ __forceinline__ long long tiled_off(int row, int k, int R);
 
 template <int BN, bool F8, int NBUF>
 __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
@@ -332,7 +333,9 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
 #pragma unroll
           for (int i = 0; i < 16; ++i)
             if (nb + i < g.N)
-              g.C16T[(long long)(nb + i) * g.ldc16t + row] = __float2bfloat16_rn(y[i]);
+              *reinterpret_cast<__nv_bfloat16 *>(
+                  reinterpret_cast<unsigned char *>(g.C16T) + tiled_off(nb + i, row, g.N)) =
+                  __float2bfloat16_rn(y[i]);
         }
         uint32_t packed[8];
 #pragma unroll
@@ -430,24 +433,124 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_tc(const __grid_constant_
   gemm_tile<BN, F8, NBUF>(g, blockIdx.x * kBM, blockIdx.y * BN);
 }
 
-// Up to four contractions in one launch, for a training step's weight
-// gradients: (256..392) x (16..256) outputs with K = the batch are a few
-// tiles each, bound by their chain of stages (128 for 8,192 rows), so the
-// chains run side by side: 126 us for the four, 1,260 us one after the other
-// in 128 x 256 tiles.  Bit for bit the result of one at a time (a split K
-// would not be).
-constexpr int kGroupBN = 64, kGroupBuf = 6;
-struct GemmGroup {
-  GemmArgs g[4];
-  int n, first[5];  // tiles of contraction i: first[i] .. first[i + 1] - 1
+// Operands of the weight gradients, laid out as the tensor core reads them:
+// element (row, k) of an R x K matrix (R a multiple of 8, K padded to whole
+// steps of 64 with zeros) at byte ((k / 64) (R / 8) + row / 8) 1024 +
+// (k % 64 / 8) 128 + (row % 8) 16 + (k % 8) 2, so the rows r0 .. of one step
+// are consecutive and come in with one bulk copy.
+__device__ __forceinline__ long long tiled_off(int row, int k, int R) {
+  return (((long long)(k >> 6) * (R >> 3) + (row >> 3)) << 10) + ((k & 63) >> 3) * 128 +
+         (row & 7) * 16 + (k & 7) * 2;
+}
+
+// Up to four contractions C = A . B^T of tiled operands in one launch: the
+// weight gradients of a training step, (256..392) x (16..256) outputs with K
+// = the batch.  They are a few tiles each, bound by their chain of steps (128
+// for 8,192 rows), so the chains run side by side.  One thread queues the
+// bulk copies of the next kGroupBuf - 1 steps, another issues the MMAs; with
+// per-thread 16-byte copies from row-major operands an SM kept ~24 KB a
+// microsecond in flight (126 us for the four; one after the other in 128 x
+// 256 tiles 1,260 us).  Each output is the same chain of additions as on its
+// own (a split K would not be).
+constexpr int kGroupBN = 64, kGroupBuf = 8;
+struct GroupArgs {
+  const unsigned char *A[4], *B[4];  // tiled, M x K and N x K
+  float *C[4];                       // M x N, row-major
+  int M[4], N[4], K, n, first[5];    // tiles of contraction i: first[i] .. first[i + 1] - 1
+  int *err;
 };
 __global__ void __launch_bounds__(kGemmThreads)
-k_gemm_group(const __grid_constant__ GemmGroup q) {
+k_gemm_group(const __grid_constant__ GroupArgs q) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  constexpr uint32_t kAStage = kBM * 128, kBStage = kGroupBN * 128;
+  __shared__ __align__(8) uint64_t full[kGroupBuf], empty[kGroupBuf], done;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int i = 0;
   while (i + 1 < q.n && (int)blockIdx.x >= q.first[i + 1]) ++i;
-  const GemmArgs g = q.g[i];
-  const int t = (int)blockIdx.x - q.first[i], nt = (g.N + kGroupBN - 1) / kGroupBN;
-  gemm_tile<kGroupBN, false, kGroupBuf>(g, (t / nt) * kBM, (t % nt) * kGroupBN);
+  const int M = q.M[i], N = q.N[i];
+  const int t = (int)blockIdx.x - q.first[i], nt = (N + kGroupBN - 1) / kGroupBN;
+  const int m0 = (t / nt) * kBM, n0 = (t % nt) * kGroupBN;
+  if (tid == 0) {
+    for (int b = 0; b < kGroupBuf; ++b) {
+      tc::mbar_init(&full[b], 1);
+      tc::mbar_init(&empty[b], 1);
+    }
+    tc::mbar_init(&done, 1);
+    tc::fence_mbar_init();
+    s_fail = 0;
+  }
+  if (warp == 0) tc::tmem_alloc(&tmem_slot, kGroupBN);
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  const int steps = (q.K + 63) >> 6;
+  unsigned char *sA = smem, *sB = smem + kGroupBuf * kAStage;
+  if (tid == 0) {
+    // producer: rows past M or N are not copied (they only reach outputs
+    // that are not written)
+    const uint32_t ab = (uint32_t)min(kBM, M - m0) * 128, bb = (uint32_t)min(kGroupBN, N - n0) * 128;
+    const unsigned char *A = q.A[i] + (long long)m0 * 128, *B = q.B[i] + (long long)n0 * 128;
+    for (int k = 0; k < steps; ++k) {
+      const int b = k % kGroupBuf;
+      if (k >= kGroupBuf &&
+          !tc::mbar_wait(&empty[b], ((k / kGroupBuf) - 1) & 1, kWaitLimit)) {
+        s_fail = 1;
+        break;
+      }
+      tc::mbar_arrive_expect_tx(&full[b], ab + bb);
+      tc::bulk_g2s(sA + b * kAStage, A + (long long)k * M * 128, ab, &full[b]);
+      tc::bulk_g2s(sB + b * kBStage, B + (long long)k * N * 128, bb, &full[b]);
+    }
+  } else if (tid == 32) {
+    constexpr uint32_t idesc = tc::idesc_bf16_f32(kBM, kGroupBN);
+    bool ok = true;
+    for (int k = 0; k < steps; ++k) {
+      const int b = k % kGroupBuf;
+      if (!tc::mbar_wait(&full[b], (k / kGroupBuf) & 1, kWaitLimit)) {
+        ok = false;
+        break;
+      }
+      tc::tc_fence_after();
+      const uint32_t a0 = tc::smem_u32(sA + b * kAStage), b0 = tc::smem_u32(sB + b * kBStage);
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk)
+        tc::mma_bf16(tmem, tc::smem_desc(a0 + kk * 256, 128, 1024),
+                     tc::smem_desc(b0 + kk * 256, 128, 1024), idesc, (k > 0 || kk > 0) ? 1u : 0u);
+      tc::mma_commit(&empty[b]);
+    }
+    tc::mma_commit(&done);
+    if (!ok) s_fail = 1;
+  }
+  __syncwarp();
+  // every MMA issued is done (bounded; also where a wait gave up)
+  if (!tc::mbar_wait(&done, 0, kWaitLimit)) s_fail = 1;
+  __syncthreads();
+  if (s_fail) {
+    if (tid == 0) {
+      // bulk copies still in flight land before the block leaves
+      for (int b = 0; b < min(kGroupBuf, steps); ++b)
+        tc::mbar_wait(&full[b], ((steps - 1 - b) / kGroupBuf) & 1, 1u << 16);
+      atomicExch(q.err, SG_ERR_TIMEOUT);
+    }
+  } else {
+    tc::tc_fence_after();
+    const int w = warp & 3, half = warp >> 2, row = m0 + w * 32 + lane;
+    for (int c = half * 32; c < half * 32 + 32; c += 16) {
+      float v[16];
+      tc::tmem_ld16(tmem + ((uint32_t)(w * 32) << 16) + (uint32_t)c, v);
+      if (row < M) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (n0 + c + j < N) q.C[i][(long long)row * N + n0 + c + j] = v[j];
+      }
+    }
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, kGroupBN);
 }
 
 std::mutex g_err_mu;
@@ -509,11 +612,11 @@ void launch_gemm_tiles(const GemmArgs &g, cudaStream_t st) {
     launch_gemm<64, F8, 4>(g, st);
 }
 
-void launch_gemm_group(GemmGroup &q, cudaStream_t st) {
+void launch_gemm_group(GroupArgs &q, cudaStream_t st) {
   q.first[0] = 0;
   for (int i = 0; i < q.n; ++i)
-    q.first[i + 1] = q.first[i] + (q.g[i].M + kBM - 1) / kBM *
-                                      ((q.g[i].N + kGroupBN - 1) / kGroupBN);
+    q.first[i + 1] =
+        q.first[i] + (q.M[i] + kBM - 1) / kBM * ((q.N[i] + kGroupBN - 1) / kGroupBN);
   static unsigned long long attr_set = 0;
   allow_smem(k_gemm_group, gemm_smem(kGroupBN, kGroupBuf), attr_set);
   k_gemm_group<<<q.first[q.n], kGemmThreads, gemm_smem(kGroupBN, kGroupBuf), st>>>(q);
@@ -1495,6 +1598,7 @@ struct TransposeJobs {
   const __nv_bfloat16 *src[4];
   __nv_bfloat16 *dst[4];
   int rows[4], cols[4];
+  bool tiled[4];  // dst in the tiled layout (cols x rows), else row-major
 };
 __global__ void __launch_bounds__(256) k_transpose_jobs(const TransposeJobs t) {
   __shared__ __nv_bfloat16 tile[64][66];
@@ -1517,14 +1621,17 @@ __global__ void __launch_bounds__(256) k_transpose_jobs(const TransposeJobs t) {
 #pragma unroll
   for (int i = 0; i < 64; i += 8) {
     const int c = i + ty;
-    if (c0 + c < cols && r0 + tx < rows)
-      *reinterpret_cast<__nv_bfloat162 *>(t.dst[z] + (long long)(c0 + c) * rows + r0 + tx) =
-          __halves2bfloat162(tile[tx][c], tile[tx + 1][c]);
+    if (c0 + c < cols && r0 + tx < rows) {
+      __nv_bfloat16 *d = t.tiled[z]
+                             ? t.dst[z] + tiled_off(c0 + c, r0 + tx, cols) / 2
+                             : t.dst[z] + (long long)(c0 + c) * rows + r0 + tx;
+      *reinterpret_cast<__nv_bfloat162 *>(d) = __halves2bfloat162(tile[tx][c], tile[tx + 1][c]);
+    }
   }
 }
 
-// Sums of the rows (length n) of up to four matrices, one block per row: the
-// bias gradients from the transposed deltas.
+// Sums of the rows of up to four tiled matrices (n columns, padded with
+// zeros), one block per row: the bias gradients from the deltas.
 struct RowsumJobs {
   const __nv_bfloat16 *src[4];
   float *dst[4];
@@ -1534,21 +1641,17 @@ __global__ void __launch_bounds__(256) k_rowsum_jobs(const RowsumJobs t, int n) 
   __shared__ float s_sum[8];
   int r = blockIdx.x, z = 0;
   while (z < 3 && r >= t.rows[z]) r -= t.rows[z++];
-  const __nv_bfloat16 *x = t.src[z] + (long long)r * n;
+  const unsigned char *x = reinterpret_cast<const unsigned char *>(t.src[z]);
   float sum = 0.0f;
-  if ((n & 7) == 0) {
-    for (int i = threadIdx.x * 8; i < n; i += 256 * 8) {
-      const uint4 v = *reinterpret_cast<const uint4 *>(x + i);
-      const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
+  for (int k = threadIdx.x * 8; k < n; k += 256 * 8) {
+    const uint4 v = *reinterpret_cast<const uint4 *>(x + tiled_off(r, k, t.rows[z]));
+    const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float2 f = __bfloat1622float2(h[k]);
-        sum += f.x;
-        sum += f.y;
-      }
+    for (int j = 0; j < 4; ++j) {
+      const float2 f = __bfloat1622float2(h[j]);
+      sum += f.x;
+      sum += f.y;
     }
-  } else {
-    for (int i = threadIdx.x; i < n; i += 256) sum += __bfloat162float(x[i]);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -1570,6 +1673,7 @@ struct GradScratch {
   __nv_bfloat16 *act[3], *in_t[4], *delta[4], *delta_t[4], *w_t[4];
   size_t bytes;
   GradScratch(unsigned char *base, size_t B) {
+    const size_t Bp = (B + 63) / 64 * 64;  // the tiled operands' padded K
     size_t off = 0;
     auto place = [&](size_t n) {
       unsigned char *p = base + off;
@@ -1582,9 +1686,9 @@ struct GradScratch {
       act[l] = (__nv_bfloat16 *)place(B * kEmuHidden * 2);
     }
     for (int l = 0; l < 4; ++l) {
-      in_t[l] = (__nv_bfloat16 *)place(B * kLayerIn[l] * 2);
+      in_t[l] = (__nv_bfloat16 *)place(Bp * kLayerIn[l] * 2);
       delta[l] = (__nv_bfloat16 *)place(B * kLayerOut[l] * 2);
-      delta_t[l] = (__nv_bfloat16 *)place(B * kLayerOut[l] * 2);
+      delta_t[l] = (__nv_bfloat16 *)place(Bp * kLayerOut[l] * 2);
       w_t[l] = (__nv_bfloat16 *)place((size_t)kLayerOut[l] * kLayerIn[l] * 2);
     }
     bytes = off;
@@ -1663,7 +1767,7 @@ extern "C" int sg_mlp_gradients(const void *feat, const int32_t *targets, int32_
                                 const void *const *W, const float *const *b, float *const *dW,
                                 float *const *db, double *loss_sum, void *scratch,
                                 int64_t scratch_bytes, void *stream) {
-  // rows of the transposed operands are the batch: a multiple of 8 of them
+  // the weight gradients contract over the batch: whole 16-byte chunks of it
   if (B < 8 || B % 8 != 0 || !feat || !targets || !W || !b || !dW || !db || !loss_sum ||
       !scratch || ((uintptr_t)scratch & 255) != 0 ||
       scratch_bytes < sg_mlp_gradients_scratch(B))
@@ -1673,12 +1777,21 @@ extern "C" int sg_mlp_gradients(const void *feat, const int32_t *targets, int32_
   cudaStream_t st = (cudaStream_t)stream;
   const GradScratch s((unsigned char *)scratch, (size_t)B);
   cudaMemsetAsync(loss_sum, 0, sizeof(double), st);
+  if (B % 64) {
+    // the last step's rows past the batch contribute zeros
+    const size_t step = (size_t)(B / 64) * 64;
+    for (int l = 0; l < 4; ++l) {
+      cudaMemsetAsync(s.in_t[l] + step * kLayerIn[l], 0, (size_t)128 * kLayerIn[l], st);
+      cudaMemsetAsync(s.delta_t[l] + step * kLayerOut[l], 0, (size_t)128 * kLayerOut[l], st);
+    }
+  }
   // transposes of the features and of the weights that the backward pass reads
   TransposeJobs t{};
   t.src[0] = (const __nv_bfloat16 *)feat;
   t.dst[0] = s.in_t[0];
   t.rows[0] = B;
   t.cols[0] = kEmuIn;
+  t.tiled[0] = true;
   for (int l = 1; l < 4; ++l) {
     t.src[l] = (const __nv_bfloat16 *)W[l];
     t.dst[l] = s.w_t[l];
@@ -1686,10 +1799,10 @@ extern "C" int sg_mlp_gradients(const void *feat, const int32_t *targets, int32_
     t.cols[l] = kLayerIn[l];
   }
   k_transpose_jobs<<<dim3((unsigned)((std::max(B, kEmuOut) + 63) / 64), 4, 4), 256, 0, st>>>(t);
-  GemmGroup q{};
-  int rc = gemm_err_buf(&q.g[0].err);
-  auto shape = [&](const __nv_bfloat16 *A, const __nv_bfloat16 *Bt, int M, int N, int K,
-                   GemmArgs &g) {
+  GroupArgs q{};
+  int rc = gemm_err_buf(&q.err);
+  auto gemm = [&](const __nv_bfloat16 *A, const __nv_bfloat16 *Bt, int M, int N, int K,
+                  GemmArgs g) {
     g.A = A;
     g.lda = K;
     g.Bt = Bt;
@@ -1698,10 +1811,6 @@ extern "C" int sg_mlp_gradients(const void *feat, const int32_t *targets, int32_
     g.N = N;
     g.K = K;
     g.ldc32 = g.ldc16 = N;
-  };
-  auto gemm = [&](const __nv_bfloat16 *A, const __nv_bfloat16 *Bt, int M, int N, int K,
-                  GemmArgs g) {
-    shape(A, Bt, M, N, K, g);
     if (!rc) rc = sg::gemm_bf16(g, st);
   };
   // forward: pre-activations, activations and their transposes
@@ -1714,7 +1823,6 @@ extern "C" int sg_mlp_gradients(const void *feat, const int32_t *targets, int32_
       g.C32 = s.pre[l];
       g.C16 = s.act[l];
       g.C16T = s.in_t[l + 1];
-      g.ldc16t = B;
     } else {
       g.C32 = s.logits;
     }
@@ -1728,20 +1836,23 @@ extern "C" int sg_mlp_gradients(const void *feat, const int32_t *targets, int32_
   d.dst[0] = s.delta_t[3];
   d.rows[0] = B;
   d.cols[0] = kEmuOut;
+  d.tiled[0] = true;
   k_transpose_jobs<<<dim3((B + 63) / 64, (kEmuOut + 63) / 64, 1), 256, 0, st>>>(d);
   for (int l = 3; l > 0; --l) {
     GemmArgs h{};
     h.C16 = s.delta[l - 1];
     h.C16T = s.delta_t[l - 1];
-    h.ldc16t = B;
     h.bwd_pre = s.pre[l - 1];
     gemm(s.delta[l], s.w_t[l], B, kLayerIn[l], kLayerOut[l], h);
   }
   q.n = 4;
+  q.K = B;
   for (int l = 0; l < 4; ++l) {
-    q.g[l].err = q.g[0].err;
-    q.g[l].C32 = dW[l];
-    shape(s.delta_t[l], s.in_t[l], kLayerOut[l], kLayerIn[l], B, q.g[l]);
+    q.A[l] = (const unsigned char *)s.delta_t[l];
+    q.B[l] = (const unsigned char *)s.in_t[l];
+    q.C[l] = dW[l];
+    q.M[l] = kLayerOut[l];
+    q.N[l] = kLayerIn[l];
   }
   if (!rc) launch_gemm_group(q, st);
   RowsumJobs r{};

@@ -38,10 +38,9 @@ struct GemmArgs {
   int ldc8;
   float c8_inv_scale;
   // training: C16 = value * GELU'(bwd_pre) (bwd_pre: M x N FP32, row-major);
-  // C16T: transposed copy of C16 (N x ldc16t)
+  // C16T: transposed copy of C16 (N x M) in the tiled layout of sg_mlp.cu
   const float *bwd_pre;
   __nv_bfloat16 *C16T;
-  int ldc16t;
 };
 
 int gemm_bf16(const GemmArgs &g, cudaStream_t st);
