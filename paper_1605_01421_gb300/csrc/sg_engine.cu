@@ -393,6 +393,7 @@ struct sg_model {
   // then stages the replicate's state in shared memory, else it works on
   // the state in device memory (L2)
   bool e2_dense = true;
+  int e2_threads = kE2Small;  // threads of the E2 kernel
   DevBuf<int> u;
   DevBuf<double> v;
   DevBuf<int32_t> rec;
@@ -1013,10 +1014,10 @@ static void launch_e2(sg_model *m, const EvArgs &ea, long long wb, long long we,
                            (int)kE2SmemStateMax);
       attr_set |= 1ull << dev;
     }
-    launch_pdl(k_events_e2<KIND, true>, (unsigned)n_rep, kE2Block, bytes, st, m->tb, ea,
+    launch_pdl(k_events_e2<KIND, true>, (unsigned)n_rep, (unsigned)m->e2_threads, bytes, st, m->tb, ea,
                (const int64_t *)m->wave_ev, wb, we, (const int64_t *)m->wave_off, day, slots);
   } else {
-    launch_pdl(k_events_e2<KIND, false>, (unsigned)n_rep, kE2Block, 0, st, m->tb, ea,
+    launch_pdl(k_events_e2<KIND, false>, (unsigned)n_rep, (unsigned)m->e2_threads, 0, st, m->tb, ea,
                (const int64_t *)m->wave_ev, wb, we, (const int64_t *)m->wave_off, day, slots);
   }
 }
@@ -1036,7 +1037,7 @@ static void launch_e2_kind(sg_model *m, const EvArgs &ea, long long wb, long lon
     long long b = wb, e = we;
     int dd = day, sl = slots;
     void *args[] = {&tb, &a, &wev, &b, &e, &woff, &dd, &sl};
-    launch_jit(k, (unsigned)n_rep, kE2Block, in_smem ? bytes : 0, st, args, true);
+    launch_jit(k, (unsigned)n_rep, (unsigned)m->e2_threads, in_smem ? bytes : 0, st, args, true);
     return;
   }
   switch (m->tb.kind) {
@@ -1457,6 +1458,7 @@ extern "C" int sg_run(sg_model *m, const int32_t *tspan, int32_t n_tspan, uint64
       std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - host_t0).count();
   const Plan &P = m->plan;
   m->e2_dense = days > 0 && P.n_e2 * 16 >= (long long)days * slots * Nn;
+  m->e2_threads = P.n_e2 > (long long)days * slots * kE2Small ? kE2Block : kE2Small;
 
   const long long per_rep_u = (long long)Nn * C, per_rep_v = (long long)Nn * NV;
   if ((rc = m->u.ensure((size_t)(per_rep_u * n_rep))) ||

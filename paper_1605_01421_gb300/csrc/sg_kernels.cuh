@@ -14,7 +14,11 @@
 namespace sg {
 
 constexpr int kDayBlock = 128;
-constexpr int kE2Block = 256;
+// Threads of the E2 kernel: the launch takes kE2Block when a replicate has more
+// than kE2Small transfers a day (37,000 herds, 740 transfers a day: 14.7 ms a
+// year with 256 threads, 13.3 with 512), else kE2Small (1,600 herds, 195 a
+// day: 6.1 ms with either).
+constexpr int kE2Block = 512, kE2Small = 256;
 
 // Programmatic dependent launch: the day kernels and the E2 kernels are
 // launched so that the next kernel in the stream may start while the
@@ -968,7 +972,7 @@ __device__ __noinline__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTrait
       double lam = w[0];
 #pragma unroll
       for (int j = 1; j < T; ++j) lam = lam + w[j];
-      const double tau = nE / lam;
+      const double tau = nE / (gt0(lam) ? lam : 1.0);  // unused where lambda = 0
       const unsigned pos_mask = __ballot_sync(full, gt0(lam));
       const unsigned bad_mask = __ballot_sync(full, bad);
       int l = 0;
@@ -1238,7 +1242,8 @@ struct AemSlots {
 // its new draw, the others by the rescaling rule) share one FP64 division and
 // three more operations, and the earliest channel is found by integer
 // comparison.  Bound by the FP64 pipe, 14 operations a firing of two channels
-// (one channel after the other 30).  Same operations on every value, in the
+// (one channel after the other 30): 1,600 SISe herds x 365 days 13.9 ms, by one
+// channel after the other 18.4 ms.  Same operations on every value, in the
 // same order, as the thread path.
 template <int KIND>
 __device__ void aem_warp(AemSlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK,
@@ -1329,7 +1334,9 @@ __device__ void aem_warp(AemSlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK,
       ++used;
     }
     dr += __popc(__ballot_sync(full, draws));
-    const double q = (draws ? E : a) / w;
+    // lanes without a change divide 1 by 1: an operand of zero in any lane
+    // sends the warp through the division's slow path
+    const double q = (draws ? E : awake ? a : 1.0) / (awake ? w : 1.0);
     const double step = draws ? q : q * (tau - t);
     const double next = t + step;
     if (changes) {
@@ -2720,7 +2727,7 @@ __device__ __forceinline__ void copy_words(int *dst, const int *src, int n) {
   for (int i = head + threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
 }
 
-constexpr int kE2Cap = 512;      // events staged in shared memory per chunk
+constexpr int kE2Cap = 896;      // events staged in shared memory per chunk
 constexpr int kE2WaveCap = 128;  // wave bounds staged per chunk
 
 // E2 events of one day: block r runs replicate r's external transfers
