@@ -271,7 +271,7 @@ def time_oracle(w, budget_s=10.0, max_runs=50):
 
 def _kernel_sources_sha1():
     h = hashlib.sha1()
-    for f in ("sg_common.h", "sg_device.cuh", "sg_kernels.cuh"):
+    for f in ("sg_common.h", "sg_device.cuh", "sg_filter.cuh", "sg_kernels.cuh"):
         with open(os.path.join(_ROOT, "paper_1605_01421_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
@@ -285,29 +285,29 @@ def _kernel_sources_sha1():
 # the capture's bytes per node-day scale it to the timed launch.  The
 # capture command:
 #   python bench.py --workload batched --days 30 --steps 1 --warmup 1
-#       --cpu-seconds 0 --e2e 0 --extras 0 --tuning 5000,16, under
+#       --cpu-seconds 0 --e2e 0 --extras 0 --tuning 5000,32, under
 #   ncu --section SpeedOfLight --section ComputeWorkloadAnalysis
 #       --section MemoryWorkloadAnalysis --section WarpStateStats
 #       --section SchedulerStats --section Occupancy --section LaunchStats
 #       --metrics dram__bytes_read.sum,dram__bytes_write.sum
 #       --clock-control none -k regex:k_days_sparse -s 1 -c 1
 DAY_KERNEL_NCU = {
-    "sources_sha1": "7c3a1bfdd76c0c8c69c09a955fc3d411772b05ab",
+    "sources_sha1": "6e1b2800a6b6cd20574bfc00c9eed37e0b9bc71c",
     "workload": "SISe3 256 replicates x 5000 nodes x 30 days, own events per replicate",
     "tuning": [5000, 32],
-    "duration_us": 2249.0,
-    "dram_bytes_read": 2896477000,
-    "dram_bytes_write": 1507242000,
-    "dram_bytes_per_node_day": 114.68,
+    "duration_us": 1675.1,
+    "dram_bytes_read": 789000704,
+    "dram_bytes_write": 1361758000,
+    "dram_bytes_per_node_day": 56.01,
     "algorithmic_bytes_per_node_day": 68,
-    "issue_active_pct": 19.23,
-    "fp64_pipe_active_pct": 14.09,
-    "warps_active_pct": 21.11,
-    "stall_barrier_per_issue": 7.70,
-    "stall_long_scoreboard_per_issue": 3.10,
-    "stall_wait_per_issue": 2.75,
-    "l1_hit_pct": 69.9,
-    "l2_hit_pct": 26.4,
+    "issue_active_pct": 29.37,
+    "fp64_pipe_active_pct": 7.78,
+    "warps_active_pct": 21.15,
+    "stall_barrier_per_issue": 3.76,
+    "stall_long_scoreboard_per_issue": 1.63,
+    "stall_wait_per_issue": 2.40,
+    "l1_hit_pct": 32.0,
+    "l2_hit_pct": 45.4,
 }
 
 

@@ -380,7 +380,7 @@ struct sg_model {
   SgEvent *e_rec = nullptr;
   int32_t *e1_day = nullptr;
   int64_t *wave_ev = nullptr, *wave_off = nullptr, *e1_node_off = nullptr;
-  int32_t heavy_after = -1;  // draws a thread takes before its warp takes
+  int32_t heavy_after = -1;  // hand-over of long days to warps (sg_set_tuning)
   int32_t npb = -1;          // nodes per block; -1 = chosen from the size
   // sg_set_replicate_range: the runs cover global replicates rep0 .. rep0 +
   // n_rep - 1 of a job with rep_total replicates (0: a whole job, rep0 = 0)

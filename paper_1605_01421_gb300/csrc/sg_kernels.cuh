@@ -177,7 +177,8 @@ struct DayArgs {
   int32_t T_begin, T_end;  // SSA toward T = T_begin .. T_end - 1
   int32_t finish_first;    // finish unit step T_begin - 1 before the SSA
   int32_t finish_last;     // finish unit step T_end - 1 after the SSA
-  int32_t heavy_after;     // draws a thread takes before its warp takes over
+  int32_t heavy_after;     // aem, or a caller's own S or G: draws a thread takes
+                           // before a warp takes over
   // 1: the model's S and G are its kind's own and its parameters finite and
   // not negative, so the intervals of sg_filter.cuh apply
   int32_t fast;
@@ -2358,7 +2359,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
       __syncthreads();
       // 1b. the listed units: finish of Td - 1 (launch start only), rates;
       //     units with lambda > 0 go to the thread list, or, expecting
-      //     heavy_after transitions or more, straight to a warp slot
+      //     warp_rate transitions or more, straight to a warp slot
       {
         const int nq = s_nnq;
 #pragma unroll 1
