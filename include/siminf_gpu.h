@@ -569,9 +569,9 @@ int sg_mlp_forward_fp8(const void *feat, int32_t B, const void *W0, const void *
  * in one call: forward pass, loss, backward pass.  feat: B x 16 BF16;
  * targets: B x 3 int32; W[l], b[l] (l < 4): BF16 weights (out x in) and FP32
  * biases; dW[l], db[l]: FP32 gradients (out); *loss_sum (device double): the
- * summed loss (out).  scratch: at least sg_mlp_gradients_scratch(B) bytes on
- * the device, 256-byte aligned. */
-int64_t sg_mlp_gradients_scratch(int32_t B);
+ * summed loss (out).  scratch: on the device, 256-byte aligned, at least as
+ * many bytes as sg_mlp_gradients_scratch says. */
+int sg_mlp_gradients_scratch(int32_t B, int64_t *bytes);
 int sg_mlp_gradients(const void *feat, const int32_t *targets, int32_t B, const void *const *W,
                      const float *const *b, float *const *dW, float *const *db,
                      double *loss_sum, void *scratch, int64_t scratch_bytes, void *stream);

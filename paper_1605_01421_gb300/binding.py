@@ -262,8 +262,8 @@ def lib(path: str | None = None):
         L.sg_mlp_forward_fp8.argtypes = [vp, i32, vp, pp, pp, ctypes.POINTER(f32), pp, vp, vp,
                                          vp, vp]
         L.sg_mlp_forward_fp8.restype = ctypes.c_int
-        L.sg_mlp_gradients_scratch.argtypes = [i32]
-        L.sg_mlp_gradients_scratch.restype = i64
+        L.sg_mlp_gradients_scratch.argtypes = [i32, ctypes.POINTER(i64)]
+        L.sg_mlp_gradients_scratch.restype = ctypes.c_int
         L.sg_gelu_backward.argtypes = [vp, vp, i64, vp, vp]
         L.sg_transpose_bf16.argtypes = [vp, i32, i32, vp, vp]
         L.sg_colsum_bf16.argtypes = [vp, i32, i32, vp, vp]

@@ -1759,8 +1759,10 @@ extern "C" int sg_mlp_forward_fp8(const void *feat, int32_t B, const void *W0,
   return sg::gemm_check(st);
 }
 
-extern "C" int64_t sg_mlp_gradients_scratch(int32_t B) {
-  return B < 0 ? 0 : (int64_t)GradScratch(nullptr, (size_t)B).bytes;
+extern "C" int sg_mlp_gradients_scratch(int32_t B, int64_t *bytes) {
+  if (B < 0 || !bytes) return SG_ERR_ARG;
+  *bytes = (int64_t)GradScratch(nullptr, (size_t)B).bytes;
+  return SG_OK;
 }
 
 extern "C" int sg_mlp_gradients(const void *feat, const int32_t *targets, int32_t B,
@@ -1770,7 +1772,7 @@ extern "C" int sg_mlp_gradients(const void *feat, const int32_t *targets, int32_
   // the weight gradients contract over the batch: whole 16-byte chunks of it
   if (B < 8 || B % 8 != 0 || !feat || !targets || !W || !b || !dW || !db || !loss_sum ||
       !scratch || ((uintptr_t)scratch & 255) != 0 ||
-      scratch_bytes < sg_mlp_gradients_scratch(B))
+      scratch_bytes < (int64_t)GradScratch(nullptr, (size_t)B).bytes)
     return SG_ERR_ARG;
   for (int l = 0; l < 4; ++l)
     if (!W[l] || !b[l] || !dW[l] || !db[l]) return SG_ERR_ARG;

@@ -124,13 +124,14 @@ class Emulator:
         dW = [torch.empty((o, i), dtype=torch.float32, device=self.device) for o, i in DIMS]
         db = [torch.empty(o, dtype=torch.float32, device=self.device) for o, _ in DIMS]
         loss = torch.empty(1, dtype=torch.float64, device=self.device)
-        nb = int(L.sg_mlp_gradients_scratch(B))
-        scratch = torch.empty(nb, dtype=torch.uint8, device=self.device)
+        nb = ctypes.c_int64()
+        _check(L.sg_mlp_gradients_scratch(B, ctypes.byref(nb)))
+        scratch = torch.empty(nb.value, dtype=torch.uint8, device=self.device)
 
         _check(L.sg_mlp_gradients(
             binding._dev_ptr(feat16, torch.bfloat16, (B, NIN), "feat16"),
             _p(targets), B, _ptrs(self.W16), _ptrs(self.b32), _ptrs(dW), _ptrs(db), _p(loss),
-            _p(scratch), nb, _s()))
+            _p(scratch), nb.value, _s()))
         return float(loss.item()) / B, dW, db
 
     def adam(self, dW, db, lr, b1=0.9, b2=0.999, eps=1e-8):
