@@ -331,7 +331,8 @@ int sg_set_replicate_range(sg_model *m, int32_t rep0, int32_t rep_total);
  * pairs exceed two full 128-pair blocks per SM, one replicate per block
  * when there are at least as many replicates as SMs (and more than 128
  * nodes), else two blocks per SM; otherwise 128 pairs per block (fewer for
- * small problems, so that about two blocks per SM exist).  By default a
+ * small problems, so that about two blocks per SM exist; one node per block
+ * for up to 16 per SM without external transfers).  By default a
  * node expecting 16 transitions or more goes to a warp if its block has at
  * most 8 of them (S, G other than the kind's own: after 32, 8 and 2 draws in
  * these three cases; aem: after 2). */
