@@ -88,6 +88,17 @@ __device__ __forceinline__ Itv itv_mul_pos(Itv a, Itv b) {
 __device__ __forceinline__ Itv itv_scale(Itv a, float b) {
   return Itv{__fmul_rd(a.lo, b), __fmul_ru(a.hi, b)};
 }
+// a * b for an interval b >= 0
+__device__ __forceinline__ Itv itv_scale(Itv a, Itv b) {
+  return Itv{__fmul_rd(a.lo, a.lo >= 0.0f ? b.lo : b.hi),
+             __fmul_ru(a.hi, a.hi >= 0.0f ? b.hi : b.lo)};
+}
+// a count: any int32 >= 0, else NaN
+__device__ __forceinline__ Itv itv_count(int n) {
+  return n >= 0 ? Itv{__int2float_rd(n), __int2float_ru(n)} : itv_nan();
+}
+__device__ __forceinline__ Itv itv_of(float x) { return Itv{x, x}; }
+__device__ __forceinline__ Itv itv_of(Itv x) { return x; }
 __device__ __forceinline__ Itv itv_mul(Itv a, Itv b) {
   if (!(fabsf(a.lo) < kItvMax && fabsf(a.hi) < kItvMax && fabsf(b.lo) < kItvMax &&
         fabsf(b.hi) < kItvMax))
@@ -270,6 +281,59 @@ template <> struct Filter<SG_SISE3> {
       x[2 * a] -= y;
       x[2 * a + 1] += y;
     }
+  }
+};
+
+// The rates as intervals for any counts, kept as int32: a count above 2^24 is
+// an interval itself.  Moves are the model's S.  Used where a day's counts
+// may leave the range in which FP32 holds them exactly (a model from
+// transition strings can grow by 127 a transition).
+template <int KIND> struct FilterWide {
+  using M = ModelTraits<KIND>;
+  static constexpr bool kPhi = KIND == SG_SISE || KIND == SG_SISE_SP || KIND == SG_SISE3;
+  int x[M::C];
+  Itv k[M::NK];
+  __device__ __forceinline__ void load(const int *u, const double *kf) {
+#pragma unroll
+    for (int p = 0; p < M::C; ++p) x[p] = u[p];
+#pragma unroll
+    for (int i = 0; i < M::NK; ++i) k[i] = kPhi ? itv_nonneg(kf[i]) : Itv{0.0f, 0.0f};
+  }
+  __device__ __forceinline__ bool sums(Itv *P, const SgTables &tb) const {
+    Itv c[M::C];
+#pragma unroll
+    for (int p = 0; p < M::C; ++p) c[p] = itv_count(x[p]);
+    if constexpr (KIND == SG_GENERIC) {
+      return M::sums_itv(c, P);
+    } else {
+      auto g = [&](int i) { return Itv{tb.g_lo[i], tb.g_hi[i]}; };
+      if constexpr (KIND == SG_SISE3) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const Itv w = itv_mul_pos(k[a], c[2 * a]);
+          P[2 * a] = a == 0 ? w : itv_add(P[2 * a - 1], w);
+          P[2 * a + 1] = itv_add(P[2 * a], itv_mul_pos(g(3 + a), c[2 * a + 1]));
+        }
+      } else {
+        if constexpr (KIND == SG_SIR) {
+          // the rate is 0 in an empty node
+          const long long n = (long long)x[0] + x[1] + x[2];
+          const float lo = fmaxf(__ll2float_rd(n), 1.0f), hi = fmaxf(__ll2float_ru(n), 1.0f);
+          P[0] = itv_div_pos(itv_mul_pos(itv_mul_pos(g(0), c[0]), c[1]), Itv{lo, hi});
+          P[0] = x[2] >= 0 ? P[0] : itv_nan();
+        } else if constexpr (KIND == SG_SIS) {
+          P[0] = itv_mul_pos(itv_mul_pos(g(0), c[0]), c[1]);
+        } else {
+          P[0] = itv_mul_pos(k[0], c[0]);
+        }
+        P[1] = itv_add(P[0], itv_mul_pos(g(1), c[1]));
+      }
+      return true;
+    }
+  }
+  __device__ __forceinline__ void fire(int n, const SgTables &tb) {
+#pragma unroll
+    for (int p = 0; p < M::C; ++p) x[p] += tb.S[n][p];
   }
 };
 

@@ -884,7 +884,8 @@ __device__ __forceinline__ int ssa_window(int *u, const double *kf, uint32_t nod
 //
 // With the kind's own tables (`fast`): the transitions of up to 32 draws are
 // walked first, selected from intervals (they depend on the draws' r2 and
-// the counts, not on the times), and lane l keeps the counts before draw l;
+// the counts, not on the times), and lane l keeps the counts before draw l,
+// as int32, which a day may take anywhere;
 // then every lane evaluates its draw in FP64 -- rates, lambda and E / lambda,
 // 32 logarithms and divisions for the price of one -- and the times are
 // added up in order, which tells where the day ends.  A draw walked beyond
@@ -926,8 +927,9 @@ __device__ __noinline__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTrait
     __syncwarp();
     return;
   }
-  Filter<KIND> F;
-  if (fast && F.load(u, kf, tb)) {
+  if (fast) {
+    FilterWide<KIND> F;
+    F.load(u, kf);
     bool done = false;
     while (!done && code == 0) {
       const U4 x = philox10(U4{c + (uint32_t)lane, node, Td, tag}, k0, k1);
@@ -945,16 +947,13 @@ __device__ __noinline__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTrait
         const bool good = F.sums(P, tb) && P[T - 1].lo >= kItvMin && P[T - 1].hi <= kItvMax;
         const uint32_t w2 = __shfl_sync(full, x.z, walked), w3 = __shfl_sync(full, x.w, walked);
         const float e = __shfl_sync(full, e_lo, walked);
-        int v[C];
-#pragma unroll
-        for (int p = 0; p < C; ++p) v[p] = (int)F.x[p];
         if (lane == walked) {
 #pragma unroll
-          for (int p = 0; p < C; ++p) us[p] = v[p];
+          for (int p = 0; p < C; ++p) us[p] = F.x[p];
         }
         ++walked;
         int n = good ? itv_select<T>(P, itv_r2(w3)) : -1;
-        if (n < 0) n = select_exact<KIND>(v, kf, w2, w3, tb);
+        if (n < 0) n = select_exact<KIND>(F.x, kf, w2, w3, tb);
         if (good) left -= e * rcp_lo(P[T - 1].hi);
         if (n < 0 || left < 0.0f) {
           open = false;
@@ -1009,14 +1008,14 @@ __device__ __noinline__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTrait
           // the event of the last draw, which the walk left out
           const uint32_t w2 = __shfl_sync(full, x.z, src), w3 = __shfl_sync(full, x.w, src);
           const int n = select_exact<KIND>(u, kf, w2, w3, tb);
-          F.load(u, kf, tb);
+          F.load(u, kf);
           F.fire(n, tb);
 #pragma unroll
-          for (int p = 0; p < C; ++p) u[p] = (int)F.x[p];
+          for (int p = 0; p < C; ++p) u[p] = F.x[p];
         }
       } else {
 #pragma unroll
-        for (int p = 0; p < C; ++p) u[p] = (int)F.x[p];
+        for (int p = 0; p < C; ++p) u[p] = F.x[p];
       }
     }
   } else {

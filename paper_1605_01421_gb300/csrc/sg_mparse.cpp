@@ -223,8 +223,9 @@ std::string code(const Node *n, const double *gd) {
 // The same expression on FP32 intervals that enclose its FP64 value
 // (sg_filter.cuh).  Subexpressions of constants are evaluated here in FP64
 // (with the very operations of the propensity) and become constant
-// intervals; counts x[] are exact and not negative, and products of factors
-// known not to be negative take the two-instruction form.
+// intervals; counts x[] are not negative (FP32 numbers that hold them exactly,
+// or intervals), and products of factors known not to be negative take the
+// two-instruction form.
 struct ItvCode {
   std::string text;
   bool constant = false, count = false, nonneg = false;
@@ -254,7 +255,7 @@ ItvCode code_itv(const Node *n, const double *gd) {
     r.count = r.nonneg = true;
     return r;
   }
-  auto itv = [](const ItvCode &c) { return c.count ? "Itv{" + c.text + ", " + c.text + "}" : c.text; };
+  auto itv = [](const ItvCode &c) { return c.count ? "itv_of(" + c.text + ")" : c.text; };
   const ItvCode a = code_itv(n->a.get(), gd);
   if (n->kind == Node::NEG) {
     if (a.constant) return constant(-a.value);
@@ -411,7 +412,7 @@ int mparse(const char *const *transitions, int n_trans, const char *const *compa
     rd.push_back(r);
     out.rate_code.push_back(code(tree.get(), gdata));
     const ItvCode c = code_itv(tree.get(), gdata);
-    out.rate_itv_code.push_back(c.count ? "Itv{" + c.text + ", " + c.text + "}" : c.text);
+    out.rate_itv_code.push_back(c.count ? "itv_of(" + c.text + ")" : c.text);
   }
   // G[k, j] = 1 when propensity k reads a compartment transition j changes
   for (int j = 0; j < n_trans; ++j)
@@ -484,7 +485,8 @@ std::string generic_source(const ParsedModel &pm) {
     s += "      case " + std::to_string(j) + ": return " + pm.rate_code[j] + ";\n";
   s += "    }\n    return 0.0;\n  }\n";
   // running sums of the propensities' intervals (false: one may be negative)
-  s += "  __device__ static __forceinline__ bool sums_itv(const float *x, Itv *P) {\n"
+  s += "  template <class X>\n"
+       "  __device__ static __forceinline__ bool sums_itv(const X *x, Itv *P) {\n"
        "    bool good = true;\n";
   for (int j = 0; j < pm.T; ++j) {
     const std::string k = std::to_string(j);
