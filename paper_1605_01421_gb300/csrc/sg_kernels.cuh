@@ -343,6 +343,18 @@ __device__ __forceinline__ void e2_stage(E2Stage &s, const DayArgs &a, long long
                  : "memory");
 }
 
+// The number of large transfers that a wave left to the warps (the same in
+// every thread), read after the wave's barrier; three counters take turns.  A
+// fast thread may add to the next wave's counter before a slow one has read
+// this wave's, so they differ; the one cleared here was last read before this
+// wave's barrier and is added to after the next one's.
+__device__ __forceinline__ int next_wave(int *count, int &cw) {
+  const int n = count[cw];
+  if (threadIdx.x == 0) count[cw == 0 ? 2 : cw - 1] = 0;
+  cw = cw == 2 ? 0 : cw + 1;
+  return n;
+}
+
 template <int C>
 __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int T,
                              long long w0, long long w1, const E2Stage *stage = nullptr) {
@@ -364,11 +376,12 @@ __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int 
   const uint64_t seed = ((uint64_t)a.k1 << 32) | a.k0;
   constexpr int kHv = 256;  // large transfers of a wave left to the warps
   __shared__ long long s_hv[kHv];
-  __shared__ int s_nhv;
+  __shared__ int s_nhv[3];  // see next_wave
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   unsigned long long applied = 0;
   bool bad = false;
-  if (threadIdx.x == 0) s_nhv = 0;
+  if (threadIdx.x < 3) s_nhv[threadIdx.x] = 0;
+  int cw = 0;
   __syncthreads();
   for (long long w = w0; w < w1; ++w) {
     const long long lo = bound(w), hi = bound(w + 1);
@@ -395,7 +408,7 @@ __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int 
       if (k >= kUrnWarp) {
         // a large transfer: sampled by a warp after this pass (in this
         // thread when the list is full)
-        const int slot = atomicAdd(&s_nhv, 1);
+        const int slot = atomicAdd(&s_nhv[cw], 1);
         if (slot < kHv) {
           s_hv[slot] = j;
           continue;
@@ -435,10 +448,8 @@ __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int 
     }
     // one barrier per wave; its result is the same for every thread
     if (__syncthreads_or(bad)) break;
-    const int nhv = min(s_nhv, kHv);  // the same in every thread
+    const int nhv = min(next_wave(s_nhv, cw), kHv);
     if (nhv > 0) {
-      __syncthreads();  // every thread has read the count
-      if (threadIdx.x == 0) s_nhv = 0;
       // the wave's large transfers, one warp each (no other event of the
       // wave touches their source nodes)
       for (int h = warp; h < nhv; h += nwarps) {
@@ -2753,11 +2764,12 @@ k_events_e2(const SgTables tb, const EvArgs a, const int64_t *__restrict__ wave_
   __shared__ uint4 s_w[kE2Cap];
   __shared__ long long s_wave[kE2WaveCap + 1];
   __shared__ int16_t s_hv[kE2Cap];  // the wave's events left to the warps
-  __shared__ int s_nhv;
+  __shared__ int s_nhv[3];  // see next_wave
   pdl_trigger();
   const int rep = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  if (threadIdx.x == 0) s_nhv = 0;
+  if (threadIdx.x < 3) s_nhv[threadIdx.x] = 0;
+  int cw = 0;
   const int Nn = tb.n_nodes;
   long long w0 = w_begin_shared, w1 = w_end_shared;
   if (slots > 1) {
@@ -2838,7 +2850,7 @@ k_events_e2(const SgTables tb, const EvArgs a, const int64_t *__restrict__ wave_
         }
         if (k >= kUrnWarp) {
           // a large transfer: sampled by a warp after this pass
-          s_hv[atomicAdd(&s_nhv, 1)] = (int16_t)i;
+          s_hv[atomicAdd(&s_nhv[cw], 1)] = (int16_t)i;
           continue;
         }
         int moved[C];
@@ -2880,10 +2892,8 @@ k_events_e2(const SgTables tb, const EvArgs a, const int64_t *__restrict__ wave_
       }
       stop = __syncthreads_or(bad);
       if (stop) break;
-      const int nhv = s_nhv;  // the same in every thread (read after the barrier)
+      const int nhv = next_wave(s_nhv, cw);
       if (nhv > 0) {
-        __syncthreads();  // every thread has read the count
-        if (threadIdx.x == 0) s_nhv = 0;
         // the wave's large transfers, one warp each: no other event of the
         // wave touches their source nodes, so the order does not matter
         for (int h = warp; h < nhv; h += nwarps) {
