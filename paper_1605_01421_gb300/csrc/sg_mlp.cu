@@ -1774,8 +1774,16 @@ extern "C" int sg_mlp_gradients(const void *feat, const int32_t *targets, int32_
       !scratch || ((uintptr_t)scratch & 255) != 0 ||
       scratch_bytes < (int64_t)GradScratch(nullptr, (size_t)B).bytes)
     return SG_ERR_ARG;
-  for (int l = 0; l < 4; ++l)
+  // feat and W are read in 16-byte pieces
+  uintptr_t low = (uintptr_t)feat;
+  for (int l = 0; l < 4; ++l) {
     if (!W[l] || !b[l] || !dW[l] || !db[l]) return SG_ERR_ARG;
+    low |= (uintptr_t)W[l];
+  }
+  if (low & 15) return SG_ERR_ARG;
+  GroupArgs q{};
+  int rc = gemm_err_buf(&q.err);
+  if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   const GradScratch s((unsigned char *)scratch, (size_t)B);
   cudaMemsetAsync(loss_sum, 0, sizeof(double), st);
@@ -1801,8 +1809,6 @@ extern "C" int sg_mlp_gradients(const void *feat, const int32_t *targets, int32_
     t.cols[l] = kLayerIn[l];
   }
   k_transpose_jobs<<<dim3((unsigned)((std::max(B, kEmuOut) + 63) / 64), 4, 4), 256, 0, st>>>(t);
-  GroupArgs q{};
-  int rc = gemm_err_buf(&q.err);
   auto gemm = [&](const __nv_bfloat16 *A, const __nv_bfloat16 *Bt, int M, int N, int K,
                   GemmArgs g) {
     g.A = A;
