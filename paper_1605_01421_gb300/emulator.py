@@ -26,6 +26,7 @@ from . import workloads as W
 
 NIN, HID, NOUT, NUSED, BINS, HALF = 16, 256, 392, 387, 129, 64
 DIMS = [(HID, NIN), (HID, HID), (HID, HID), (NOUT, HID)]  # (out, in) per layer
+OUTS = [(o,) for o, _ in DIMS]
 
 
 def _p(t):
@@ -34,6 +35,19 @@ def _p(t):
 
 def _ptrs(ts):
     return (ctypes.c_void_p * len(ts))(*[t.data_ptr() for t in ts])
+
+
+def _operands(ts, dtype, shapes, name):
+    """Device pointers of a pass's operands, each checked as binding._dev_ptr
+    does (which is called for its message only: a pass takes a dozen)."""
+    if len(ts) != len(shapes):
+        raise ValueError(f"{name} must hold {len(shapes)} tensors, not {len(ts)}")
+    p = (ctypes.c_void_p * len(shapes))()
+    for i, t in enumerate(ts):
+        if not (t.is_cuda and t.dtype is dtype and t.is_contiguous() and t.shape == shapes[i]):
+            binding._dev_ptr(t, dtype, shapes[i], f"{name}[{i}]")
+        p[i] = t.data_ptr()
+    return p
 
 
 def _s():
@@ -80,8 +94,10 @@ class Emulator:
         pres = [new(HID, torch.float32) if keep else None for _ in range(3)]
         logits = new(NOUT, torch.float32)
         _check(binding.lib().sg_mlp_forward(
-            binding._dev_ptr(feat16, torch.bfloat16, (B, NIN), "feat16"), B, _ptrs(self.W16),
-            _ptrs(self.b32), _ptrs(post), _ptrs(pres) if keep else None, _p(logits), _s()))
+            _operands([feat16], torch.bfloat16, [(B, NIN)], "feat16")[0], B,
+            _operands(self.W16, torch.bfloat16, DIMS, "W16"),
+            _operands(self.b32, torch.float32, OUTS, "b32"), _ptrs(post),
+            _ptrs(pres) if keep else None, _p(logits), _s()))
         return logits, [feat16, *post], pres
 
     # -- FP8 inference ---------------------------------------------------------
@@ -106,12 +122,16 @@ class Emulator:
         arguments the engine uses when FP8 inference is switched on."""
         torch = self.torch
         B, dev = feat16.shape[0], feat16.device
-        bufs = [torch.empty((B, HID), dtype=torch.uint8, device=dev) for _ in range(2)]
+        bufs = torch.empty((2, B, HID), dtype=torch.uint8, device=dev)
         logits = torch.empty((B, NOUT), dtype=torch.float32, device=dev)
         _check(binding.lib().sg_mlp_forward_fp8(
-            binding._dev_ptr(feat16, torch.bfloat16, (B, NIN), "feat16"), B, _p(self.W16[0]),
-            _ptrs(self.W8), _ptrs(self.wscale), (ctypes.c_float * 3)(*self.act_scale),
-            _ptrs(self.b32), _p(bufs[0]), _p(bufs[1]), _p(logits), _s()))
+            _operands([feat16], torch.bfloat16, [(B, NIN)], "feat16")[0], B,
+            _operands(self.W16[:1], torch.bfloat16, DIMS[:1], "W16")[0],
+            _operands(self.W8, torch.uint8, DIMS[1:], "W8"),
+            _operands(self.wscale, torch.float32, OUTS[1:], "wscale"),
+            (ctypes.c_float * 3)(*self.act_scale),
+            _operands(self.b32, torch.float32, OUTS, "b32"), bufs.data_ptr(),
+            bufs.data_ptr() + B * HID, _p(logits), _s()))
         return logits
 
     # -- backward ------------------------------------------------------------
@@ -129,8 +149,9 @@ class Emulator:
         scratch = torch.empty(nb.value, dtype=torch.uint8, device=self.device)
 
         _check(L.sg_mlp_gradients(
-            binding._dev_ptr(feat16, torch.bfloat16, (B, NIN), "feat16"),
-            _p(targets), B, _ptrs(self.W16), _ptrs(self.b32), _ptrs(dW), _ptrs(db), _p(loss),
+            _operands([feat16], torch.bfloat16, [(B, NIN)], "feat16")[0], _p(targets), B,
+            _operands(self.W16, torch.bfloat16, DIMS, "W16"),
+            _operands(self.b32, torch.float32, OUTS, "b32"), _ptrs(dW), _ptrs(db), _p(loss),
             _p(scratch), nb.value, _s()))
         return float(loss.item()) / B, dW, db
 
