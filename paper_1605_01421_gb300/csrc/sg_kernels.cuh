@@ -355,8 +355,9 @@ __device__ __forceinline__ int next_wave(int *count, int &cw) {
   return n;
 }
 
+// Returns whether a transfer failed (the same in every thread).
 template <int C>
-__device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int T,
+__device__ bool e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int T,
                              long long w0, long long w1, const E2Stage *stage = nullptr) {
   auto event = [&](long long j) {
     if (stage && j >= stage->lo && j < stage->lo + stage->n_ev) return stage->ev[j - stage->lo];
@@ -368,10 +369,10 @@ __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int 
     return (long long)a.wave_ev[w];
   };
   // a run that already failed does nothing (one thread reads, the barrier
-  // makes the answer the block's); with the events staged the caller has
-  // checked this day
+  // makes the answer the block's); with the events staged the caller knows
+  // whether its own units' day went well
   if (!stage && __syncthreads_or(threadIdx.x == 0 && *(volatile int32_t *)&a.err->code != 0))
-    return;
+    return true;
   int *state = a.u + (long long)rep * tb.n_nodes * C;
   const uint64_t seed = ((uint64_t)a.k1 << 32) | a.k0;
   constexpr int kHv = 256;  // large transfers of a wave left to the warps
@@ -379,7 +380,7 @@ __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int 
   __shared__ int s_nhv[3];  // see next_wave
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   unsigned long long applied = 0;
-  bool bad = false;
+  bool bad = false, failed = false;
   if (threadIdx.x < 3) s_nhv[threadIdx.x] = 0;
   int cw = 0;
   __syncthreads();
@@ -447,7 +448,10 @@ __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int 
       ++applied;
     }
     // one barrier per wave; its result is the same for every thread
-    if (__syncthreads_or(bad)) break;
+    if (__syncthreads_or(bad)) {
+      failed = true;
+      break;
+    }
     const int nhv = min(next_wave(s_nhv, cw), kHv);
     if (nhv > 0) {
       // the wave's large transfers, one warp each (no other event of the
@@ -487,6 +491,7 @@ __device__ void e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int 
     }
   }
   if (applied) atomicAdd(&a.cnt->events, applied);
+  return failed;
 }
 
 // One transition (Appendix A, inversion and update): the smallest n with
@@ -2057,13 +2062,14 @@ __device__ __forceinline__ int sparse_e1(bool has, long long gid, int rep, int n
 // the take to lane k mod 32 in round k / 32 (word by a search over the
 // warp's prefix counts, bit by halving), so the lanes stay full however
 // sparse the marks are.  Warp-uniform; called by every lane of a warp.
+// *failed (shared) is set where an event fails.
 template <int C>
 __device__ __forceinline__ void sparse_e1_bits(const uint32_t *e1bits, const uint32_t *actbits,
                                                bool act, int *take, int words, int nw,
                                                long long gbase,
                                                int Td, int d, const SgTables &tb,
                                                const DayArgs &a, uint32_t k0, uint32_t k1,
-                                               unsigned long long &applied) {
+                                               unsigned long long &applied, int *failed) {
   const int lane = threadIdx.x & 31;
   const int Nn = tb.n_nodes;
   for (;;) {
@@ -2113,7 +2119,7 @@ __device__ __forceinline__ void sparse_e1_bits(const uint32_t *e1bits, const uin
         rep = (int)(gid / Nn);
         node = (int)(gid - (long long)rep * Nn);
       }
-      sparse_e1<C>(has, gid, rep, node, Td, d, tb, a, k0, k1, applied);
+      if (sparse_e1<C>(has, gid, rep, node, Td, d, tb, a, k0, k1, applied)) *failed = 1;
     }
   }
 }
@@ -2147,6 +2153,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
   __shared__ uint32_t s_actbits[kSparseChunk / 32];  // units taking SSA draws today
   __shared__ uint32_t s_e1bits[kSparseChunk / 32];   // units with E1 events today
   __shared__ int s_nact, s_nheavy, s_stop, s_next, s_nnq, s_e1take, s_e1late, s_nshort, s_nredo;
+  __shared__ int s_failed;  // a unit of the block met an error today
   __shared__ __align__(16) E2Stage s_e2;  // the day's transfers of the block's first replicate
   pdl_trigger();
   const int Nn = tb.n_nodes;
@@ -2195,7 +2202,10 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
   }
   for (int Td = a.T_begin; Td < a.T_end; ++Td) {
     // a failed run stops at the next day boundary (the block's verdict)
-    if (tid == 0) s_stop = *(volatile int32_t *)&a.err->code != 0;
+    if (tid == 0) {
+      s_stop = *(volatile int32_t *)&a.err->code != 0;
+      s_failed = 0;
+    }
     __syncthreads();
     if (s_stop) break;
     const double Tn = (double)Td;
@@ -2388,6 +2398,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
           int code = 0;
           if (fin_prev) {
             code = sparse_finish<KIND>(Td - 1, u, v, quiet, tb, a, rep, node, gid);
+            if (code) s_failed = 1;
             if (a.out.prev && m_prev >= 0 && code == 0)
               prevalence_add_unit<C>(a.out, (long long)rep * a.M + m_prev, u);
           }
@@ -2418,6 +2429,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
             }
             if (bad) {
               report(a.err, SG_ERR_RATE, a.rep0 + rep, node, Td, -1);
+              s_failed = 1;
             } else if (fires) {
               atomicOr(&s_actbits[(i - c0) >> 5], 1u << ((i - c0) & 31));
               int slot = kSparseDirect;
@@ -2466,7 +2478,10 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
           __syncwarp();
           ssa_warp<KIND>(hs, Tn, (uint32_t)Td, k0, k1, a.fast, tb, fired, drawn);
           if (lane == 0) {
-            if (hs.code) report(a.err, hs.code, hs.rep, hs.node, Td, -1);
+            if (hs.code) {
+              report(a.err, hs.code, hs.rep, hs.node, Td, -1);
+              s_failed = 1;
+            }
 #pragma unroll
             for (int p = 0; p < C; ++p) a.u[gid * C + p] = hs.u[p];
           }
@@ -2517,7 +2532,10 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
                                 drawn);
           }
           if (slot >= 0 && slot < kSparseHeavy) s_heavy[slot].rep = -1;  // done
-          if (r < 0) report(a.err, r, a.rep0 + rep, node, Td, -1);
+          if (r < 0) {
+            report(a.err, r, a.rep0 + rep, node, Td, -1);
+            s_failed = 1;
+          }
 #pragma unroll
           for (int p = 0; p < C; ++p) a.u[gid * C + p] = u[p];
         }
@@ -2530,7 +2548,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
       // draws come after the SSA (their events follow their day's
       // transitions)
       if (has_e1) sparse_e1_bits<C>(s_e1bits, s_actbits, false, &s_e1take, e1_words, nw_e1,
-                                    g0 + c0, Td, d, tb, a, k0, k1, applied);
+                                    g0 + c0, Td, d, tb, a, k0, k1, applied, &s_failed);
       __syncthreads();
       // the warp slots not run yet: all of them when every warp had list
       // units, else those the thread list handed over
@@ -2543,7 +2561,10 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
         __syncwarp();
         ssa_warp<KIND>(hs, Tn, (uint32_t)Td, k0, k1, a.fast, tb, fired, drawn);
         if (lane == 0) {
-          if (hs.code) report(a.err, hs.code, hs.rep, hs.node, Td, -1);
+          if (hs.code) {
+            report(a.err, hs.code, hs.rep, hs.node, Td, -1);
+            s_failed = 1;
+          }
 #pragma unroll
           for (int p = 0; p < C; ++p) a.u[gid * C + p] = hs.u[p];
         }
@@ -2553,23 +2574,25 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
       // 3. E1 events of day Td of the units that took draws today
       if (has_e1) {
         sparse_e1_bits<C>(s_e1bits, s_actbits, true, &s_e1late, e1_words, nw_e1, g0 + c0, Td,
-                          d, tb, a, k0, k1, applied);
+                          d, tb, a, k0, k1, applied, &s_failed);
         __syncthreads();
       }
     }
     if (a.e2_inblock) {
       // this block's replicates' external transfers of Td (the wave plan of
-      // day d; no other block touches their nodes)
+      // day d; no other block touches their nodes); none after an error of
+      // one of its units today
       asm volatile("cp.async.wait_all;" ::: "memory");
       __syncthreads();
-      for (long long r = g0 / Nn; nub > 0 && r * Nn < g0 + nub; ++r) {
+      bool stop = s_failed != 0;
+      for (long long r = g0 / Nn; !stop && nub > 0 && r * Nn < g0 + nub; ++r) {
         long long w0 = s_e2.w0, w1 = s_e2.w1;
         if (a.slots > 1 && r != g0 / Nn) {
           const long long k = (long long)d * a.slots + r;
           w0 = a.wave_off[k];
           w1 = a.wave_off[k + 1];
         }
-        if (w0 < w1) e2_rep_block<C>(tb, a, (int)r, Td, w0, w1, &s_e2);
+        if (w0 < w1) stop = e2_rep_block<C>(tb, a, (int)r, Td, w0, w1, &s_e2);
       }
       // a failed transfer ends the run before the day's post time step (of
       // which the next day's check takes care but on the last one)
