@@ -895,13 +895,50 @@ __device__ __forceinline__ int ssa_window(int *u, const double *kf, uint32_t nod
   }
 }
 
+// The transitions of up to 32 draws from the counts in F on, each selected
+// from intervals or in FP64: lane l of `us` gets the counts before draw l,
+// F.x the ones after the last walked draw.  x: lane l's Philox words of draw
+// l, e_lo its waiting time's lower end, left: what is left of the day, rounded
+// up.  Returns whether a state after the last walked draw exists (not where
+// nothing can fire, or the day is surely over).
+template <int KIND, typename F_t>
+__device__ __forceinline__ bool walk_draws(F_t &F, const U4 &x, float e_lo, float left,
+                                           const double *kf, const SgTables &tb, int *us,
+                                           int &walked) {
+  using M = ModelTraits<KIND>;
+  constexpr int C = M::C, T = M::T;
+  constexpr unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  for (walked = 0; walked < 32;) {
+    Itv P[T];
+    const bool good = F.sums(P, tb) && P[T - 1].lo >= kItvMin && P[T - 1].hi <= kItvMax;
+    const uint32_t w2 = __shfl_sync(full, x.z, walked), w3 = __shfl_sync(full, x.w, walked);
+    const float e = __shfl_sync(full, e_lo, walked);
+    int v[C];
+#pragma unroll
+    for (int p = 0; p < C; ++p) v[p] = (int)F.x[p];
+    if (lane == walked) {
+#pragma unroll
+      for (int p = 0; p < C; ++p) us[p] = v[p];
+    }
+    ++walked;
+    int n = good ? itv_select<T>(P, itv_r2(w3)) : -1;
+    if (n < 0) n = select_exact<KIND>(v, kf, w2, w3, tb);
+    if (good) left -= e * rcp_lo(P[T - 1].hi);
+    if (n < 0 || left < 0.0f) return false;
+    F.fire(n, tb);
+  }
+  return true;
+}
+
 // Direct SSA of one unit by a whole warp: from intervals (ssa_window), and
 // where they leave an event's time open, with exact times.
 //
 // With the kind's own tables (`fast`): the transitions of up to 32 draws are
 // walked first, selected from intervals (they depend on the draws' r2 and
-// the counts, not on the times), and lane l keeps the counts before draw l,
-// as int32, which a day may take anywhere;
+// the counts, not on the times), and lane l keeps the counts before draw l
+// (a day may take them anywhere in int32: FP32 counts are loaded anew for
+// every 32 draws, and where they would not be exact FilterWide takes over);
 // then every lane evaluates its draw in FP64 -- rates, lambda and E / lambda,
 // 32 logarithms and divisions for the price of one -- and the times are
 // added up in order, which tells where the day ends.  A draw walked beyond
@@ -944,38 +981,29 @@ __device__ __noinline__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTrait
     return;
   }
   if (fast) {
-    FilterWide<KIND> F;
-    F.load(u, kf);
     bool done = false;
     while (!done && code == 0) {
       const U4 x = philox10(U4{c + (uint32_t)lane, node, Td, tag}, k0, k1);
       const double nE = -log_pos(u01_open(x.x, x.y));
       // walk the transitions; stop early once the day is surely over
       const float e_lo = itv_neglog(x.x, x.y).lo;
-      float left = (float)(Tn - t) * (1.0f + 0x1.0p-20f);
-      int us[C];
+      const float left = (float)(Tn - t) * (1.0f + 0x1.0p-20f);
+      int us[C], end[C], walked;
 #pragma unroll
       for (int p = 0; p < C; ++p) us[p] = u[p];
-      int walked = 0;
-      bool open = true;  // a state after the last walked draw exists
-      while (walked < 32) {
-        Itv P[T];
-        const bool good = F.sums(P, tb) && P[T - 1].lo >= kItvMin && P[T - 1].hi <= kItvMax;
-        const uint32_t w2 = __shfl_sync(full, x.z, walked), w3 = __shfl_sync(full, x.w, walked);
-        const float e = __shfl_sync(full, e_lo, walked);
-        if (lane == walked) {
+      bool open;
+      Filter<KIND> N;
+      if (N.load(u, kf, tb)) {
+        // 32 transitions leave the counts below 2^24
+        open = walk_draws<KIND>(N, x, e_lo, left, kf, tb, us, walked);
 #pragma unroll
-          for (int p = 0; p < C; ++p) us[p] = F.x[p];
-        }
-        ++walked;
-        int n = good ? itv_select<T>(P, itv_r2(w3)) : -1;
-        if (n < 0) n = select_exact<KIND>(F.x, kf, w2, w3, tb);
-        if (good) left -= e * rcp_lo(P[T - 1].hi);
-        if (n < 0 || left < 0.0f) {
-          open = false;
-          break;
-        }
-        F.fire(n, tb);
+        for (int p = 0; p < C; ++p) end[p] = (int)N.x[p];
+      } else {
+        FilterWide<KIND> W;
+        W.load(u, kf);
+        open = walk_draws<KIND>(W, x, e_lo, left, kf, tb, us, walked);
+#pragma unroll
+        for (int p = 0; p < C; ++p) end[p] = W.x[p];
       }
       // lane l < walked: draw c + l exactly
       double w[T];
@@ -1024,14 +1052,12 @@ __device__ __noinline__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTrait
           // the event of the last draw, which the walk left out
           const uint32_t w2 = __shfl_sync(full, x.z, src), w3 = __shfl_sync(full, x.w, src);
           const int n = select_exact<KIND>(u, kf, w2, w3, tb);
-          F.load(u, kf);
-          F.fire(n, tb);
 #pragma unroll
-          for (int p = 0; p < C; ++p) u[p] = F.x[p];
+          for (int p = 0; p < C; ++p) u[p] += tb.S[n][p];
         }
       } else {
 #pragma unroll
-        for (int p = 0; p < C; ++p) u[p] = F.x[p];
+        for (int p = 0; p < C; ++p) u[p] = end[p];
       }
     }
   } else {
