@@ -309,12 +309,13 @@ int sg_set_kernel_timing(sg_model *m, int enable);
 int sg_set_replicate_range(sg_model *m, int32_t rep0, int32_t rep_total);
 
 /* Work split of the SSA day kernel.  With nodes_per_block in 1..128 each
- * block of 128 threads owns that many (replicate, node) pairs, one per
- * thread, kept in registers for a run of days; a node that expects
- * heavy_after transitions or more in a day (a rate at the day's start; for
- * S or G other than the kind's own and for aem: that has taken heavy_after
- * draws) is handed to one of the block's warps, whose 32 lanes evaluate 32
- * draws at once.  With
+ * block of 128 threads (one warp for nodes_per_block = 1) owns that many
+ * (replicate, node) pairs, one per thread, kept in registers for a run of
+ * days; a node that expects heavy_after transitions or more in a day (a rate
+ * at the day's start; where G leaves a rate as it was although a transition
+ * changed what it reads, where a rate parameter is negative or not finite,
+ * and for aem: that has taken heavy_after draws) is handed to one of the
+ * block's warps, whose 32 lanes evaluate 32 draws at once.  With
  * nodes_per_block > 128 (up to 2^22; the direct method on the built-in
  * kinds without emulator or persistent schedule -- elsewhere it
  * means 128) the sparse-activity schedule runs instead: each block of 256
@@ -334,8 +335,9 @@ int sg_set_replicate_range(sg_model *m, int32_t rep0, int32_t rep_total);
  * small problems, so that about two blocks per SM exist; one node per block
  * for up to 16 per SM without external transfers).  By default a
  * node expecting 16 transitions or more goes to a warp if its block has at
- * most 8 of them (S, G other than the kind's own: after 32, 8 and 2 draws in
- * these three cases; aem: after 2). */
+ * most 8 of them (where draws count, as above: after 32 in the
+ * sparse-activity schedule, else after 2; aem: after 0 in blocks of up to
+ * eight nodes, else after 2). */
 int sg_set_tuning(sg_model *m, int32_t nodes_per_block, int32_t heavy_after);
 
 /* Autotuner: for each of nodes_per_block in {4, 8, 16, 32, 64, 128} x

@@ -505,31 +505,35 @@ static void set_gdata(SgTables &tb, const sg_desc *d) {
   }
 }
 
-// Whether the day kernels may decide draws from intervals (sg_filter.cuh):
-// the transitions are the kind's own, G marks at least the rates that each
-// one changes (then every rate equals its value at the current counts), and
-// the rate parameters are not negative (NaN intervals catch the rest).
-// Models from transition strings derive both from the strings.
-static bool filter_applies(const SgTables &tb) {
-  if (tb.kind == SG_GENERIC) return true;
+// Whether the day kernels may decide draws from intervals (DayArgs::fast): G
+// marks at least the rates that each transition changes (then every rate
+// equals its value at the current counts), and the rate parameters are not
+// negative (NaN intervals catch the rest).  1 if S is the kind's own, 2 if it
+// is another.  Models from transition strings derive both from the strings.
+static int filter_mode(const SgTables &tb) {
+  if (tb.kind == SG_GENERIC) return 1;
   const bool three = tb.kind == SG_SISE3;
   const int n_rates = three ? 6 : 2;
-  for (int j = 0; j < tb.n_trans; ++j) {
-    int8_t want[SG_MAX_COMP] = {};
-    if (tb.kind == SG_SIR) {
-      want[j] = -1;
-      want[j + 1] = 1;
-    } else {
-      want[j] = -1;
-      want[j ^ 1] = 1;
-    }
-    if (std::memcmp(want, tb.S[j], sizeof want) != 0) return false;
-    const uint32_t need = three ? 3u << (j & ~1) : 3u;
-    if ((tb.dep[j] & need) != need) return false;
-  }
   for (int i = 0; i < n_rates; ++i)
-    if (!(tb.g_lo[i] >= 0.0f)) return false;
-  return true;
+    if (!(tb.g_lo[i] >= 0.0f)) return 0;
+  int mode = 1;
+  for (int j = 0; j < tb.n_trans; ++j) {
+    int8_t own[SG_MAX_COMP] = {};
+    own[j] = -1;
+    own[tb.kind == SG_SIR ? j + 1 : j ^ 1] = 1;
+    if (std::memcmp(own, tb.S[j], sizeof own) != 0) mode = 2;
+    for (int k = 0; k < tb.n_trans; ++k) {
+      // the compartments that rate k reads
+      uint32_t reads = 1u << k;
+      if (k == 0 && tb.kind == SG_SIR) reads = 7u;
+      if (k == 0 && tb.kind == SG_SIS) reads = 3u;
+      bool changes = false;
+      for (int p = 0; p < tb.n_comp; ++p)
+        changes = changes || (((reads >> p) & 1u) && tb.S[j][p] != 0);
+      if (changes && !((tb.dep[j] >> k) & 1u)) return 0;
+    }
+  }
+  return mode;
 }
 
 static int model_create(const sg_desc *d, sg_model **out, bool generic);
@@ -866,7 +870,8 @@ static void launch_days(sg_model *m, const DayArgs &a, cudaStream_t st) {
     // sparse-activity schedule (sg_run only sets npb > kDayBlock where it
     // applies: direct method, built-in kinds without a coupled post step)
     if constexpr (KIND == SG_SIR || KIND == SG_SIS || KIND == SG_SISE || KIND == SG_SISE3)
-      launch_pdl(k_days_sparse<KIND>, grid, kSparseBlock, 0, st, m->tb, a);
+      launch_pdl(a.fast == 1 ? k_days_sparse<KIND, false> : k_days_sparse<KIND, true>, grid,
+                 kSparseBlock, 0, st, m->tb, a);
   } else {
     launch_pdl(k_days<KIND, false>, grid, day_threads(a), 0, st, m->tb, a);
   }
@@ -1543,7 +1548,7 @@ extern "C" int sg_run(sg_model *m, const int32_t *tspan, int32_t n_tspan, uint64
   da.slots = slots;
   da.rep0 = m->rep0;
   da.heavy_after = m->heavy_after >= 0 ? m->heavy_after : 2;
-  da.fast = filter_applies(tb) ? 1 : 0;
+  da.fast = filter_mode(tb);
   set_warp_rule(da, m->heavy_after);
   da.npb = m->npb > 0 ? m->npb : default_npb((long long)Nn * n_rep);
   // a run without external transfers is one launch: where every node can
@@ -1579,7 +1584,9 @@ extern "C" int sg_run(sg_model *m, const int32_t *tspan, int32_t n_tspan, uint64
     if (units > 2LL * kDayBlock * sms) {
       const bool whole = n_rep >= sms && Nn > kDayBlock;
       da.npb = whole ? Nn : (int32_t)((units + 2LL * sms - 1) / (2LL * sms));
-      if (m->heavy_after < 0) da.heavy_after = whole ? 32 : 8;
+      // (draws before a warp starts the day anew, where intervals do not
+      // apply; 100,000 SISe herds with a stale rate: 3.4 ms, at 8 draws 8.1)
+      if (m->heavy_after < 0) da.heavy_after = 32;
     }
   }
   {
@@ -2028,7 +2035,7 @@ extern "C" int sg_run_noalloc(const sg_desc *d, const double *d_ldata, const int
       da.n_rep = n_rep;
       da.slots = 1;
       da.heavy_after = 2;
-      da.fast = filter_applies(tb) ? 1 : 0;
+      da.fast = filter_mode(tb);
       set_warp_rule(da, -1);
       da.npb = default_npb((long long)Nn * n_rep);
       da.emu = nullptr;

@@ -146,8 +146,8 @@ __device__ __forceinline__ Itv itv_r2(uint32_t w3) {
 // The kind's rates as intervals.  load() takes the counts and the day's rate
 // factors (ModelTraits::prepare) and tells whether the intervals apply;
 // sums() gives the running sums of the rates in index order; fire(n) moves
-// the counts x by transition n of the kind's own S (the host only sets
-// DayArgs::fast when the model's S and G are the kind's).  Counts of the
+// the counts x by transition n of the kind's own S (used only where
+// DayArgs::fast says that the model's S is the kind's).  Counts of the
 // built-in kinds are kept as FP32: their transitions keep every node's total,
 // so with each count below 2^20 at the start they stay exact.
 //
@@ -284,20 +284,22 @@ template <> struct Filter<SG_SISE3> {
   }
 };
 
-// The rates as intervals for any counts, kept as int32: a count above 2^24 is
-// an interval itself.  Moves are the model's S.  Used where a day's counts
-// may leave the range in which FP32 holds them exactly (a model from
-// transition strings can grow by 127 a transition).
+// The rates as intervals for any counts, kept as int32 (a count above 2^24 is
+// an interval itself), moved by the model's S.  Used for a caller's own S, for
+// counts beyond Filter's, and where a day may take the counts out of the
+// range in which FP32 holds them exactly (a model from transition strings can
+// grow by 127 a transition).
 template <int KIND> struct FilterWide {
   using M = ModelTraits<KIND>;
   static constexpr bool kPhi = KIND == SG_SISE || KIND == SG_SISE_SP || KIND == SG_SISE3;
   int x[M::C];
   Itv k[M::NK];
-  __device__ __forceinline__ void load(const int *u, const double *kf) {
+  __device__ __forceinline__ bool load(const int *u, const double *kf, const SgTables &) {
 #pragma unroll
     for (int p = 0; p < M::C; ++p) x[p] = u[p];
 #pragma unroll
     for (int i = 0; i < M::NK; ++i) k[i] = kPhi ? itv_nonneg(kf[i]) : Itv{0.0f, 0.0f};
+    return true;
   }
   __device__ __forceinline__ bool sums(Itv *P, const SgTables &tb) const {
     Itv c[M::C];

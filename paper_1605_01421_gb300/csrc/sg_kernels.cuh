@@ -177,10 +177,11 @@ struct DayArgs {
   int32_t T_begin, T_end;  // SSA toward T = T_begin .. T_end - 1
   int32_t finish_first;    // finish unit step T_begin - 1 before the SSA
   int32_t finish_last;     // finish unit step T_end - 1 after the SSA
-  int32_t heavy_after;     // aem, or a caller's own S or G: draws a thread takes
-                           // before a warp takes over
-  // 1: the model's S and G are its kind's own and its parameters finite and
-  // not negative, so the intervals of sg_filter.cuh apply
+  int32_t heavy_after;     // aem, or intervals that do not apply: draws a thread
+                           // takes before a warp takes over
+  // the intervals of sg_filter.cuh apply: parameters finite and not negative,
+  // every rate a function of the counts (G marks at least the rates that each
+  // transition changes), and S the kind's own (1) or a caller's (2); 0: not
   int32_t fast;
   float warp_rate;         // expected transitions from which a unit's day goes to a warp,
   int32_t warp_max;        // if the block has at most this many such units
@@ -689,14 +690,14 @@ __device__ __forceinline__ uint32_t day_units_hi(float t) {
 // beside it.  Bound by issue where every lane has a unit (100,000 endemic
 // SISe3 herds x 20 days, 130 M draws: 2.9 ms, in FP64 43.0 ms), elsewhere by
 // the latency of the longest unit (100 SIR nodes x 99 days: 0.23 ms, 1.33 ms).
-template <int KIND>
+template <int KIND, typename F_t = Filter<KIND>>
 __device__ __forceinline__ int ssa_filter(int *u, const double *kf, uint32_t node, uint32_t Td,
                                           uint32_t tag, uint32_t k0, uint32_t k1,
                                           const SgTables &tb, unsigned long long &fired,
                                           unsigned long long &drawn) {
   using M = ModelTraits<KIND>;
   constexpr int T = M::T;
-  Filter<KIND> F;
+  F_t F;
   if (!F.load(u, kf, tb)) return SSA_REDO;
   DayTime t(Td);
   U4 x = philox10(U4{0u, node, Td, tag}, k0, k1);
@@ -740,6 +741,66 @@ __device__ __forceinline__ int ssa_filter(int *u, const double *kf, uint32_t nod
   return SSA_DONE;
 }
 
+// One unit's day in its thread where the kind's own intervals do not apply, by
+// FilterWide (own: a caller's own S) or with exact times.  Out of line, so that
+// k_days keeps its registers for ssa_filter.  u and kf are copies that the
+// caller makes for this call; n[0] and n[1] get the day's transitions and draws.
+template <int KIND>
+__device__ __noinline__ int ssa_general(int *u, const double *kf, uint32_t node, uint32_t Td,
+                                        uint32_t tag, uint32_t k0, uint32_t k1, bool own,
+                                        int budget, const SgTables &tb, unsigned long long *n) {
+  unsigned long long f = 0, d = 0;
+  const int r = own ? ssa_filter<KIND, FilterWide<KIND>>(u, kf, node, Td, tag, k0, k1, tb, f, d)
+                    : ssa_exact<KIND>(u, kf, node, Td, tag, k0, k1, budget, tb, f, d);
+  n[0] = f;
+  n[1] = d;
+  return r;
+}
+
+// One unit's day in its thread, by what `fast` says (DayArgs::fast).
+template <int KIND>
+__device__ __forceinline__ int ssa_thread(int *u, const double *kf, uint32_t node, uint32_t Td,
+                                          uint32_t tag, uint32_t k0, uint32_t k1, int fast,
+                                          int budget, const SgTables &tb,
+                                          unsigned long long &fired, unsigned long long &drawn) {
+  using M = ModelTraits<KIND>;
+  // a model from transition strings is always 1
+  if (KIND == SG_GENERIC || fast == 1)
+    return ssa_filter<KIND>(u, kf, node, Td, tag, k0, k1, tb, fired, drawn);
+  int un[M::C];
+  double kn[M::NK];
+  unsigned long long n[2];
+#pragma unroll
+  for (int p = 0; p < M::C; ++p) un[p] = u[p];
+#pragma unroll
+  for (int i = 0; i < M::NK; ++i) kn[i] = kf[i];
+  const int r = ssa_general<KIND>(un, kn, node, Td, tag, k0, k1, fast == 2, budget, tb, n);
+#pragma unroll
+  for (int p = 0; p < M::C; ++p) u[p] = un[p];
+  fired += n[0];
+  drawn += n[1];
+  return r;
+}
+
+// The day's total rate as an interval; false (lambda not set) where the intervals
+// do not apply.
+template <int KIND>
+__device__ __forceinline__ bool day_rate(const int *u, const double *kf, int fast,
+                                         const SgTables &tb, Itv &lambda) {
+  constexpr int T = ModelTraits<KIND>::T;
+  Itv L[T];
+  bool good = false;
+  if (KIND == SG_GENERIC || fast == 1) {
+    Filter<KIND> F;
+    good = F.load(u, kf, tb) && F.sums(L, tb);
+  } else if (fast == 2) {
+    FilterWide<KIND> F;
+    good = F.load(u, kf, tb) && F.sums(L, tb);
+  }
+  if (good) lambda = L[T - 1];
+  return good;
+}
+
 // Direct SSA of one unit's day by a whole warp, decided from intervals.  The
 // draws depend only on (seed, replicate, node, day, draw index), so lane l
 // holds the random numbers of draw c0 + l.  The states that the next J draws
@@ -758,7 +819,7 @@ template <int T>
 struct Window {
   static constexpr int J = T == 1 ? 8 : T == 2 ? 7 : T <= 6 ? 3 : 2;
 };
-template <int KIND>
+template <int KIND, typename F_t>
 __device__ __forceinline__ int ssa_window(int *u, const double *kf, uint32_t node, uint32_t Td,
                                           uint32_t tag, uint32_t k0, uint32_t k1,
                                           const SgTables &tb, unsigned long long &fired,
@@ -768,11 +829,11 @@ __device__ __forceinline__ int ssa_window(int *u, const double *kf, uint32_t nod
   constexpr unsigned full = 0xffffffffu;
   constexpr int kNone = T, kOpen = T + 1, kBad = T + 2;  // no transition; not settled; no interval
   const int lane = threadIdx.x & 31;
-  Filter<KIND> F;
+  F_t F;
   if (!F.load(u, kf, tb)) return SSA_REDO;
   // this lane's multiset: its size and what it adds to the counts
   int depth = 0;
-  float add[C];
+  decltype(F.x[0] + F.x[0]) add[C];
   {
     int m0 = -1, m1 = -1, n0 = 0, n1 = 0;  // n0 times m0 and n1 times m1
     if (T <= 2) {
@@ -802,7 +863,7 @@ __device__ __forceinline__ int ssa_window(int *u, const double *kf, uint32_t nod
       int y = 0;
       if (m0 >= 0 && n0) y += n0 * tb.S[m0][p];
       if (m1 >= 0 && n1) y += n1 * tb.S[m1][p];
-      add[p] = (float)y;
+      add[p] = y;
     }
   }
   DayTime t(Td);
@@ -821,7 +882,7 @@ __device__ __forceinline__ int ssa_window(int *u, const double *kf, uint32_t nod
       w3 = x.w;
       have = true;
     }
-    Filter<KIND> G = F;
+    F_t G = F;
 #pragma unroll
     for (int p = 0; p < C; ++p) G.x[p] += add[p];
     const int src = (int)(t.d - c0) + depth;
@@ -949,7 +1010,7 @@ __device__ __forceinline__ bool walk_draws(F_t &F, const U4 &x, float e_lo, floa
 // the lanes only compute 32 draws' random numbers at once.
 template <int KIND>
 __device__ __noinline__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK> &hs, double Tn,
-                         uint32_t Td, uint32_t k0, uint32_t k1, bool fast, const SgTables &tb,
+                         uint32_t Td, uint32_t k0, uint32_t k1, int fast, const SgTables &tb,
                          unsigned long long &fired, unsigned long long &drawn) {
   using M = ModelTraits<KIND>;
   constexpr int C = M::C, T = M::T, NK = M::NK;
@@ -968,7 +1029,15 @@ __device__ __noinline__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTrait
   int code = 0;
   unsigned long long f = 0, wf = 0, wd = 0;
   const long long Tkey = order_key(Tn);
-  if (fast && ssa_window<KIND>(u, kf, node, Td, tag, k0, k1, tb, wf, wd) == SSA_DONE) {
+  int r = SSA_REDO;
+  if (fast) {
+    Filter<KIND> N;
+    if (fast == 1 && N.load(u, kf, tb))
+      r = ssa_window<KIND, Filter<KIND>>(u, kf, node, Td, tag, k0, k1, tb, wf, wd);
+    else
+      r = ssa_window<KIND, FilterWide<KIND>>(u, kf, node, Td, tag, k0, k1, tb, wf, wd);
+  }
+  if (r == SSA_DONE) {
     __syncwarp();
     if (lane == 0) {
 #pragma unroll
@@ -980,7 +1049,7 @@ __device__ __noinline__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTrait
     __syncwarp();
     return;
   }
-  if (fast) {
+  if (KIND == SG_GENERIC || fast) {
     bool done = false;
     while (!done && code == 0) {
       const U4 x = philox10(U4{c + (uint32_t)lane, node, Td, tag}, k0, k1);
@@ -993,14 +1062,14 @@ __device__ __noinline__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTrait
       for (int p = 0; p < C; ++p) us[p] = u[p];
       bool open;
       Filter<KIND> N;
-      if (N.load(u, kf, tb)) {
+      if (fast == 1 && N.load(u, kf, tb)) {
         // 32 transitions leave the counts below 2^24
         open = walk_draws<KIND>(N, x, e_lo, left, kf, tb, us, walked);
 #pragma unroll
         for (int p = 0; p < C; ++p) end[p] = (int)N.x[p];
       } else {
         FilterWide<KIND> W;
-        W.load(u, kf);
+        W.load(u, kf, tb);
         open = walk_draws<KIND>(W, x, e_lo, left, kf, tb, us, walked);
 #pragma unroll
         for (int p = 0; p < C; ++p) end[p] = W.x[p];
@@ -1778,9 +1847,8 @@ k_days(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
       };
       if (a.fast && ssa) {
         // a long day goes to a warp if the block has few of them
-        Filter<KIND> F;
-        Itv L[T];
-        if (F.load(u, kf, tb) && F.sums(L, tb) && L[T - 1].lo >= a.warp_rate) {
+        Itv lambda;
+        if (day_rate<KIND>(u, kf, a.fast, tb, lambda) && lambda.lo >= a.warp_rate) {
           my = atomicAdd(&s_nheavy, 1);
           to_slot();
         }
@@ -1789,10 +1857,8 @@ k_days(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
       const bool own = s_nheavy > a.warp_max;
       __syncthreads();
       if (ssa && (my < 0 || own)) {
-        const int r = a.fast ? ssa_filter<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, a.k0,
-                                                a.k1, tb, fired, drawn)
-                             : ssa_exact<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, a.k0,
-                                               a.k1, a.heavy_after, tb, fired, drawn);
+        const int r = ssa_thread<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, a.k0, a.k1,
+                                       a.fast, a.heavy_after, tb, fired, drawn);
         if (r == SSA_REDO) {
           if (my < 0) my = atomicAdd(&s_nheavy, 1);
           to_slot();
@@ -2167,7 +2233,10 @@ struct UnitPos {
   }
 };
 
-template <int KIND>
+// OWN: a caller's own S or G (DayArgs::fast is not 1).  Two kernels, because a
+// branch in the list's loop that leads to a call costs the kind's own tables
+// their registers (256 x 5,000 x 60 days 3.7 ms instead of 3.5).
+template <int KIND, bool OWN>
 __global__ void __launch_bounds__(kSparseBlock, 2)
 k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
   using M = ModelTraits<KIND>;
@@ -2437,7 +2506,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
             float lam;
             Filter<KIND> F;
             Itv L[T];
-            if (a.fast && F.load(u, kf, tb) && F.sums(L, tb) && L[T - 1].hi <= kItvMax) {
+            if (!OWN && F.load(u, kf, tb) && F.sums(L, tb) && L[T - 1].hi <= kItvMax) {
               fires = L[T - 1].hi > 0.0f;
               lam = L[T - 1].lo;
             } else {
@@ -2536,10 +2605,16 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
 #pragma unroll
           for (int q = 0; q < NV; ++q) v[q] = a.v[gid * NV + q];
           M::prepare(v, tb.gdata, kf);
-          int r = a.fast ? ssa_filter<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1,
-                                            tb, fired, drawn)
-                         : ssa_exact<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1,
-                                           a.heavy_after, tb, fired, drawn);
+          int r;
+          if (!OWN)
+            r = ssa_filter<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1, tb, fired,
+                                 drawn);
+          else if (a.fast)
+            r = ssa_filter<KIND, FilterWide<KIND>>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0,
+                                                   k1, tb, fired, drawn);
+          else
+            r = ssa_exact<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1, a.heavy_after,
+                                tb, fired, drawn);
           if (r == SSA_REDO) {
             if (slot < 0) slot = n_direct + atomicAdd(&s_nredo, 1);
             if (slot < kSparseHeavy) {
