@@ -626,6 +626,7 @@ template <int C, int NK>
 struct HeavySlot {
   double kf[NK];
   int32_t node, rep, code;
+  int32_t redo;  // 1: intervals have left the day's end open in its thread
   int32_t u[C];
 };
 
@@ -651,7 +652,9 @@ __device__ __forceinline__ int select_exact(const int *u, const double *kf, uint
 // is that in 2^-6 units, rounded up, and d the number of transitions
 // (at most kFilterDraws, so d * drift < 2^32).
 constexpr uint32_t kDayUnits = 1u << 31;
-constexpr uint32_t kFilterDraws = 1u << 16;  // longer days take exact times
+// Longer days take exact times at once: with n draws the end of the day is left
+// open in n (2.5e-6 + n 5e-10) of the cases, and the attempt is lost.
+constexpr uint32_t kFilterDraws = 1u << 15;
 struct DayTime {
   uint32_t lo = 0, hi = 0, d = 0, drift;
   __device__ __forceinline__ explicit DayTime(uint32_t Td)
@@ -831,6 +834,10 @@ __device__ __forceinline__ int ssa_window(int *u, const double *kf, uint32_t nod
   const int lane = threadIdx.x & 31;
   F_t F;
   if (!F.load(u, kf, tb)) return SSA_REDO;
+  {
+    Itv L[T];
+    if (F.sums(L, tb) && L[T - 1].lo >= (float)kFilterDraws) return SSA_REDO;
+  }
   // this lane's multiset: its size and what it adds to the counts
   int depth = 0;
   decltype(F.x[0] + F.x[0]) add[C];
@@ -1031,11 +1038,14 @@ __device__ __noinline__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTrait
   const long long Tkey = order_key(Tn);
   int r = SSA_REDO;
   if (fast) {
+    // (a thread that gave up has decided from the same intervals)
     Filter<KIND> N;
-    if (fast == 1 && N.load(u, kf, tb))
-      r = ssa_window<KIND, Filter<KIND>>(u, kf, node, Td, tag, k0, k1, tb, wf, wd);
-    else
+    if (fast == 1 && N.load(u, kf, tb)) {
+      if (!hs.redo)
+        r = ssa_window<KIND, Filter<KIND>>(u, kf, node, Td, tag, k0, k1, tb, wf, wd);
+    } else if (fast == 1 || !hs.redo) {
       r = ssa_window<KIND, FilterWide<KIND>>(u, kf, node, Td, tag, k0, k1, tb, wf, wd);
+    }
   }
   if (r == SSA_DONE) {
     __syncwarp();
@@ -1835,8 +1845,9 @@ k_days(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
       const bool ssa = live && code == 0 && !emulated;
       double kf[NK];
       if (ssa) M::prepare(v, tb.gdata, kf);
-      auto to_slot = [&]() {
+      auto to_slot = [&](int redo) {
         HeavySlot<C, NK> &hs = s_heavy[my];
+        hs.redo = redo;
 #pragma unroll
         for (int i = 0; i < NK; ++i) hs.kf[i] = kf[i];
         hs.node = node;
@@ -1850,7 +1861,7 @@ k_days(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
         Itv lambda;
         if (day_rate<KIND>(u, kf, a.fast, tb, lambda) && lambda.lo >= a.warp_rate) {
           my = atomicAdd(&s_nheavy, 1);
-          to_slot();
+          to_slot(0);
         }
       }
       __syncthreads();
@@ -1861,7 +1872,7 @@ k_days(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
                                        a.fast, a.heavy_after, tb, fired, drawn);
         if (r == SSA_REDO) {
           if (my < 0) my = atomicAdd(&s_nheavy, 1);
-          to_slot();
+          to_slot(1);
         } else {
           if (my >= 0) s_heavy[my].rep = -1;  // done
           my = -1;
@@ -2536,6 +2547,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
                 hs.node = node;
                 hs.rep = a.rep0 + rep;
                 hs.code = i;  // the unit, until the warp reports
+                hs.redo = 0;
 #pragma unroll
                 for (int p = 0; p < C; ++p) hs.u[p] = u[p];
               } else if (lam < 2.0f) {
@@ -2624,6 +2636,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
               hs.node = node;
               hs.rep = a.rep0 + rep;
               hs.code = (int32_t)(gid - g0);  // the unit, until the warp reports
+              hs.redo = 1;
 #pragma unroll
               for (int p = 0; p < C; ++p) hs.u[p] = u[p];
               continue;
