@@ -113,13 +113,15 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
   auto sB = [&](int b) { return smem + NBUF * kAStage + (uint32_t)b * kBStage; };
   __shared__ __align__(8) uint64_t bar[NBUF];
   __shared__ uint32_t tmem_slot;
-  __shared__ int s_fail;
+  // a wait of stage s ran out: set in s_fail[s & 1], read after the next
+  // stage's barrier, so that every thread reads the same
+  __shared__ int s_fail[2];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int b = 0; b < NBUF; ++b) tc::mbar_init(&bar[b], 1);
     tc::fence_mbar_init();
-    s_fail = 0;
+    s_fail[0] = s_fail[1] = 0;
   }
   if (warp == 0) tc::tmem_alloc(&tmem_slot, BN);
   tc::tc_fence_before();
@@ -129,6 +131,7 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
   constexpr uint32_t idesc = F8 ? tc::idesc_e4m3_f32(kBM, BN) : tc::idesc_bf16_f32(kBM, BN);
   const int stages = (g.K + kStageK - 1) / kStageK;
   bool ok = true;
+  int issued = 0;  // stages whose MMAs are on their way
 
   // Stage loader: every thread issues its 16-byte asynchronous copies
   // (cp.async) for stage s into buffer s mod NBUF, rows past M / N and
@@ -184,7 +187,7 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
     asm volatile("cp.async.wait_group %0;" ::"n"(NBUF - 2) : "memory");
     tc::fence_async_smem();
     __syncthreads();
-    if (s_fail) {
+    if (s_fail[(s + 1) & 1]) {
       ok = false;
       break;
     }
@@ -203,13 +206,14 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
       }
       tc::mma_commit(&bar[b]);
     }
+    issued = s + 1;
     // the buffer of stage s + NBUF - 1 is free once the MMAs of stage s - 1
     // are done; its loads overlap those of the stages between
     const int nx = s + NBUF - 1;
     if (nx < stages) {
       if (s > 0 &&
           !tc::mbar_wait(&bar[(s - 1) % NBUF], ((s - 1) / NBUF) & 1, kWaitLimit))
-        s_fail = 1;
+        s_fail[s & 1] = 1;
       else
         load_stage(nx);
     }
@@ -218,13 +222,13 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int m0, int n0) {
   // all MMAs done: the last stage's commit completes after every earlier one
   if (ok && stages > 0) {
     const int l = stages - 1;
-    if (!tc::mbar_wait(&bar[l % NBUF], (l / NBUF) & 1, kWaitLimit)) ok = false;
+    ok = !__syncthreads_or(!tc::mbar_wait(&bar[l % NBUF], (l / NBUF) & 1, kWaitLimit));
   }
   if (!ok) {
     if (tid == 0) atomicExch(g.err, SG_ERR_TIMEOUT);
     // copies and MMAs still in flight end (bounded) before the memory is freed
     asm volatile("cp.async.wait_all;" ::: "memory");
-    for (int l = max(0, stages - NBUF); l < stages; ++l)
+    for (int l = max(0, issued - NBUF); l < issued; ++l)
       tc::mbar_wait(&bar[l % NBUF], (l / NBUF) & 1, 1u << 16);
   }
   if (ok) {
@@ -465,7 +469,7 @@ k_gemm_group(const __grid_constant__ GroupArgs q) {
   constexpr uint32_t kAStage = kBM * 128, kBStage = kGroupBN * 128;
   __shared__ __align__(8) uint64_t full[kGroupBuf], empty[kGroupBuf], done;
   __shared__ uint32_t tmem_slot;
-  __shared__ int s_fail;
+  __shared__ int s_fail, s_queued;  // a wait ran out; steps queued
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int i = 0;
   while (i + 1 < q.n && (int)blockIdx.x >= q.first[i + 1]) ++i;
@@ -493,7 +497,8 @@ k_gemm_group(const __grid_constant__ GroupArgs q) {
     // that are not written)
     const uint32_t ab = (uint32_t)min(kBM, M - m0) * 128, bb = (uint32_t)min(kGroupBN, N - n0) * 128;
     const unsigned char *A = q.A[i] + (long long)m0 * 128, *B = q.B[i] + (long long)n0 * 128;
-    for (int k = 0; k < steps; ++k) {
+    int k = 0;
+    for (; k < steps; ++k) {
       const int b = k % kGroupBuf;
       if (k >= kGroupBuf &&
           !tc::mbar_wait(&empty[b], ((k / kGroupBuf) - 1) & 1, kWaitLimit)) {
@@ -504,6 +509,7 @@ k_gemm_group(const __grid_constant__ GroupArgs q) {
       tc::bulk_g2s(sA + b * kAStage, A + (long long)k * M * 128, ab, &full[b]);
       tc::bulk_g2s(sB + b * kBStage, B + (long long)k * N * 128, bb, &full[b]);
     }
+    s_queued = k;
   } else if (tid == 32) {
     constexpr uint32_t idesc = tc::idesc_bf16_f32(kBM, kGroupBN);
     bool ok = true;
@@ -531,8 +537,8 @@ k_gemm_group(const __grid_constant__ GroupArgs q) {
   if (s_fail) {
     if (tid == 0) {
       // bulk copies still in flight land before the block leaves
-      for (int b = 0; b < min(kGroupBuf, steps); ++b)
-        tc::mbar_wait(&full[b], ((steps - 1 - b) / kGroupBuf) & 1, 1u << 16);
+      for (int k = max(0, s_queued - kGroupBuf); k < s_queued; ++k)
+        tc::mbar_wait(&full[k % kGroupBuf], (k / kGroupBuf) & 1, 1u << 16);
       atomicExch(q.err, SG_ERR_TIMEOUT);
     }
   } else {
