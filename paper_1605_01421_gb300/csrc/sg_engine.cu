@@ -870,7 +870,7 @@ static void launch_days(sg_model *m, const DayArgs &a, cudaStream_t st) {
     // sparse-activity schedule (sg_run only sets npb > kDayBlock where it
     // applies: direct method, built-in kinds without a coupled post step)
     if constexpr (KIND == SG_SIR || KIND == SG_SIS || KIND == SG_SISE || KIND == SG_SISE3)
-      launch_pdl(a.fast == 1 ? k_days_sparse<KIND, false> : k_days_sparse<KIND, true>, grid,
+      launch_pdl(a.fast == 2 ? k_days_sparse<KIND, true> : k_days_sparse<KIND, false>, grid,
                  kSparseBlock, 0, st, m->tb, a);
   } else {
     launch_pdl(k_days<KIND, false>, grid, day_threads(a), 0, st, m->tb, a);

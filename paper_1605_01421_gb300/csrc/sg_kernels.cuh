@@ -2244,9 +2244,9 @@ struct UnitPos {
   }
 };
 
-// OWN: a caller's own S or G (DayArgs::fast is not 1).  Two kernels, because a
-// branch in the list's loop that leads to a call costs the kind's own tables
-// their registers (256 x 5,000 x 60 days 3.7 ms instead of 3.5).
+// OWN: a caller's own S (DayArgs::fast is 2).  Two kernels, because a third
+// branch in the list's loop costs the kind's own tables their registers (256 x
+// 5,000 x 60 days 3.6 ms instead of 3.4).
 template <int KIND, bool OWN>
 __global__ void __launch_bounds__(kSparseBlock, 2)
 k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
@@ -2517,7 +2517,7 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
             float lam;
             Filter<KIND> F;
             Itv L[T];
-            if (!OWN && F.load(u, kf, tb) && F.sums(L, tb) && L[T - 1].hi <= kItvMax) {
+            if (!OWN && a.fast && F.load(u, kf, tb) && F.sums(L, tb) && L[T - 1].hi <= kItvMax) {
               fires = L[T - 1].hi > 0.0f;
               lam = L[T - 1].lo;
             } else {
@@ -2618,15 +2618,14 @@ k_days_sparse(const __grid_constant__ SgTables tb, const __grid_constant__ DayAr
           for (int q = 0; q < NV; ++q) v[q] = a.v[gid * NV + q];
           M::prepare(v, tb.gdata, kf);
           int r;
-          if (!OWN)
-            r = ssa_filter<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1, tb, fired,
-                                 drawn);
-          else if (a.fast)
+          if constexpr (OWN)
             r = ssa_filter<KIND, FilterWide<KIND>>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0,
                                                    k1, tb, fired, drawn);
           else
-            r = ssa_exact<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1, a.heavy_after,
-                                tb, fired, drawn);
+            r = a.fast ? ssa_filter<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1, tb,
+                                          fired, drawn)
+                       : ssa_exact<KIND>(u, kf, (uint32_t)node, (uint32_t)Td, tag, k0, k1,
+                                         a.heavy_after, tb, fired, drawn);
           if (r == SSA_REDO) {
             if (slot < 0) slot = n_direct + atomicAdd(&s_nredo, 1);
             if (slot < kSparseHeavy) {
