@@ -23,8 +23,8 @@ _BUILD = os.path.join(_PKG, "_build")
 LIB_PATH = os.path.join(_BUILD, "libsiminf_gpu.so")
 
 SOURCES = ["sg_engine.cu", "sg_plan.cpp", "sg_mlp.cu", "sg_mparse.cpp"]
-HEADERS = ["sg_common.h", "sg_device.cuh", "sg_filter.cuh", "sg_kernels.cuh", "sg_plan.h", "sg_mlp.h", "sg_tc.cuh",
-           "sg_mparse.h"]
+HEADERS = ["sg_common.h", "sg_device.cuh", "sg_filter.cuh", "sg_kernels.cuh", "sg_plan.h",
+           "sg_mlp.h", "sg_tc.cuh", "sg_mparse.h"]
 # The headers the run-time compiler (NVRTC) sees for a model from transition
 # strings, embedded into the library; NVRTC has no C library, so the two
 # standard headers they include are replaced by minimal ones.
@@ -171,7 +171,8 @@ EXPORTS = ["sg_model_create", "sg_set_events", "sg_run", "sg_run_host",
            "sg_run_noalloc", "sg_set_tuning", "sg_autotune", "sg_set_graphs",
            "sg_gemm_bf16", "sg_mlp_ce_loss", "sg_gelu_backward", "sg_transpose_bf16",
            "sg_colsum_bf16", "sg_adam_step", "sg_emu_features", "sg_emu_targets",
-           "sg_emu_sample", "sg_mlp_forward", "sg_mlp_forward_fp8", "sg_mlp_gradients", "sg_mlp_gradients_scratch",
+           "sg_emu_sample", "sg_mlp_forward", "sg_mlp_forward_fp8", "sg_mlp_gradients",
+           "sg_mlp_gradients_scratch",
            "sg_emulator_set", "sg_set_neighbors", "sg_set_solver",
            "sg_set_output", "sg_model_create_parsed", "sg_model_tables",
            "sg_set_fused_events", "sg_set_persistent", "sg_gemm_fp8", "sg_quant_fp8_rows",

@@ -304,14 +304,8 @@ __device__ __forceinline__ bool grid_barrier(unsigned int *bar, int n_blocks, Sg
   return s_ok != 0;
 }
 
-// The external transfers (Sec. 3.3) of replicate `rep` at unit time T, wave by
-// wave, by one block (a block barrier between waves), on the replicate's
-// state in global memory.  The state was written by other blocks of the same
-// launch, so it is read and written at L2 only (ld / st .cg) and added to
-// with atomics; a wave never samples a node another event of the wave
-// touches.  Same arithmetic and random stream as the E2 kernel.
-// The day's events and wave bounds may have been staged in shared memory
-// (E2Stage) while the day's SSA ran.
+// A day's events and wave bounds staged in shared memory while the day's SSA
+// runs, for e2_rep_block.
 constexpr int kE2StageEv = 128, kE2StageWaves = 31;
 struct E2Stage {
   SgEvent ev[kE2StageEv];
@@ -356,7 +350,13 @@ __device__ __forceinline__ int next_wave(int *count, int &cw) {
   return n;
 }
 
-// Returns whether a transfer failed (the same in every thread).
+// The external transfers (Sec. 3.3) of replicate `rep` at unit time T, wave by
+// wave, by one block (a block barrier between waves), on the replicate's
+// state in global memory.  The state was written by other blocks of the same
+// launch, so it is read and written at L2 only (ld / st .cg) and added to
+// with atomics; a wave never samples a node another event of the wave
+// touches.  Same arithmetic and random stream as the E2 kernel.  Returns
+// whether a transfer failed (the same in every thread).
 template <int C>
 __device__ bool e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int T,
                              long long w0, long long w1, const E2Stage *stage = nullptr) {
@@ -495,10 +495,6 @@ __device__ bool e2_rep_block(const SgTables &tb, const DayArgs &a, int rep, int 
   return failed;
 }
 
-// One transition (Appendix A, inversion and update): the smallest n with
-// target <= running sum of the positive rates (last positive one if rounding
-// leaves none), u += S[, n], and the rates that column n of G marks are
-// recomputed.  Returns 0 or SG_ERR_RATE.
 // u += S[, n] and the rates that column n of G marks recomputed; 0 or
 // SG_ERR_RATE.
 template <int KIND>
@@ -519,6 +515,9 @@ __device__ __forceinline__ int apply_transition(int *u, double *w, int n, const 
   return code;
 }
 
+// One transition (Appendix A, inversion and update): the smallest n with
+// target <= running sum of the positive rates (last positive one if rounding
+// leaves none), then apply_transition.
 template <int KIND>
 __device__ __forceinline__ int fire(int *u, double *w, double target, const double *kf,
                                     const SgTables &tb) {
@@ -540,16 +539,14 @@ __device__ __forceinline__ int fire(int *u, double *w, double target, const doub
   return apply_transition<KIND>(u, w, n, kf, tb);
 }
 
-// Prefix sums P_j = (..(w_0 + w_1) + ..) + w_j of the rates in index order,
-// recomputed from index j0 on (the rates below j0 unchanged).  P_(T-1) is
-// lambda as the direct method sums it, and at every positive rate P_j is
+// Prefix sums P_j = (..(w_0 + w_1) + ..) + w_j of the rates in index order.
+// P_(T-1) is lambda as the direct method sums it, and at every positive rate P_j is
 // the running sum of the positive rates that fire() forms (adding a zero
 // rate leaves a sum unchanged, and a sum of zeros plus w is w).
 template <int T>
-__device__ __forceinline__ void rate_prefix(const double *w, double *P, int j0) {
+__device__ __forceinline__ void rate_prefix(const double *w, double *P) {
 #pragma unroll
-  for (int j = 0; j < T; ++j)
-    if (j >= j0) P[j] = j == 0 ? w[0] : P[j - 1] + w[j];
+  for (int j = 0; j < T; ++j) P[j] = j == 0 ? w[0] : P[j - 1] + w[j];
 }
 
 // fire()'s choice of transition from the prefix sums.
@@ -640,7 +637,7 @@ __device__ __forceinline__ int select_exact(const int *u, const double *kf, uint
   double w[M::T], P[M::T];
 #pragma unroll
   for (int j = 0; j < M::T; ++j) w[j] = M::rate_k(j, u, kf, tb.gdata);
-  rate_prefix<M::T>(w, P, 0);
+  rate_prefix<M::T>(w, P);
   if (!gt0(P[M::T - 1])) return -1;
   return select_prefix<M::T>(w, P, P[M::T - 1] * u01_open(w2, w3));
 }
@@ -691,8 +688,8 @@ __device__ __forceinline__ uint32_t day_units_hi(float t) {
 // is 55 FP64 instructions of ~76 issue cycles each).  The random numbers of
 // the next draw do not depend on this one's outcome, so they are computed
 // beside it.  Bound by issue where every lane has a unit (100,000 endemic
-// SISe3 herds x 20 days, 130 M draws: 2.9 ms, in FP64 43.0 ms), elsewhere by
-// the latency of the longest unit (100 SIR nodes x 99 days: 0.23 ms, 1.33 ms).
+// SISe3 herds x 20 days, 130 M draws: 3.2 ms, in FP64 43.0 ms), elsewhere by
+// the latency of the longest unit (100 SIR nodes x 99 days: 0.19 ms, 1.33 ms).
 template <int KIND, typename F_t = Filter<KIND>>
 __device__ __forceinline__ int ssa_filter(int *u, const double *kf, uint32_t node, uint32_t Td,
                                           uint32_t tag, uint32_t k0, uint32_t k1,
@@ -817,7 +814,8 @@ __device__ __forceinline__ bool day_rate(const int *u, const double *kf, int fas
 // Latency bound: a round is one evaluation and J dependent shuffles.  At ten
 // times a thread's instructions it pays for the few units of a block whose
 // day is long (1,000 predator-prey nodes x 30 days, 2,600 draws a node-day:
-// 20 ms, by threads 115 ms; 37,000 SISe3 herds x 365 days: 15 ms, 19 ms).
+// 15.8 ms, by threads 38.7 ms; 37,000 SISe3 herds x 365 days: 13.3 ms, 17.1
+// ms).
 template <int T>
 struct Window {
   static constexpr int J = T == 1 ? 8 : T == 2 ? 7 : T <= 6 ? 3 : 2;
@@ -1016,9 +1014,10 @@ __device__ __forceinline__ bool walk_draws(F_t &F, const U4 &x, float e_lo, floa
 // Otherwise (a caller's own S or G): draw by draw, the rates kept as G says;
 // the lanes only compute 32 draws' random numbers at once.
 template <int KIND>
-__device__ __noinline__ void ssa_warp(HeavySlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK> &hs, double Tn,
-                         uint32_t Td, uint32_t k0, uint32_t k1, int fast, const SgTables &tb,
-                         unsigned long long &fired, unsigned long long &drawn) {
+__device__ __noinline__ void ssa_warp(
+    HeavySlot<ModelTraits<KIND>::C, ModelTraits<KIND>::NK> &hs, double Tn, uint32_t Td,
+    uint32_t k0, uint32_t k1, int fast, const SgTables &tb, unsigned long long &fired,
+    unsigned long long &drawn) {
   using M = ModelTraits<KIND>;
   constexpr int C = M::C, T = M::T, NK = M::NK;
   constexpr unsigned full = 0xffffffffu;
@@ -1337,7 +1336,6 @@ __device__ __forceinline__ int aem_steps(int *u, const double *kf, double *a, do
 // A node handed from its thread to a warp (all events method).
 template <int C, int NK, int T>
 struct AemSlot {
-  double t;
   double kf[NK];
   double a[T], tau[T];
   uint32_t c[T];
@@ -1814,7 +1812,6 @@ k_days(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
           if (slot < kAemSlots) {
             my = slot;
             AemSlot<C, NK, T> &hs = s_aheavy[slot];
-            hs.t = t;
 #pragma unroll
             for (int i = 0; i < NK; ++i) hs.kf[i] = kf[i];
 #pragma unroll
@@ -1885,7 +1882,8 @@ k_days(const __grid_constant__ SgTables tb, const __grid_constant__ DayArgs a) {
     if constexpr (!AEM) {
       const int nh = s_nheavy;
       for (int h = warp; h < nh; h += nwarps)
-        if (s_heavy[h].rep >= 0) ssa_warp<KIND>(s_heavy[h], Tn, (uint32_t)Td, a.k0, a.k1, a.fast, tb, fired, drawn);
+        if (s_heavy[h].rep >= 0)
+          ssa_warp<KIND>(s_heavy[h], Tn, (uint32_t)Td, a.k0, a.k1, a.fast, tb, fired, drawn);
     } else {
       const int nh = min(s_nheavy, kAemSlots);
       for (int h = warp; h < nh; h += nwarps)

@@ -603,8 +603,8 @@ void launch_gemm(const GemmArgs &g, cudaStream_t st) {
   k_gemm_tc<BN, F8, NBUF><<<grid, kGemmThreads, gemm_smem(BN, NBUF), st>>>(g);
 }
 
-// The widest tile that still gives every SM one, else the narrowest (8,192 x
-// 256 x 256 in 64 wide tiles: 20-28 us, most SMs idle).
+// The widest tile that still gives every SM (152) one, else the narrowest:
+// 8,192 x 256 x 256 took 20-28 us as 64 tiles of 256 columns, with 88 SMs idle.
 constexpr int kGemmSms = 152;
 template <bool F8>
 void launch_gemm_tiles(const GemmArgs &g, cudaStream_t st) {
