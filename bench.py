@@ -292,22 +292,22 @@ def _kernel_sources_sha1():
 #       --metrics dram__bytes_read.sum,dram__bytes_write.sum
 #       --clock-control none -k regex:k_days_sparse -s 1 -c 1
 DAY_KERNEL_NCU = {
-    "sources_sha1": "6e1b2800a6b6cd20574bfc00c9eed37e0b9bc71c",
+    "sources_sha1": "e074fcd4464e7ec970afa99782d628103c59c46a",
     "workload": "SISe3 256 replicates x 5000 nodes x 30 days, own events per replicate",
     "tuning": [5000, 32],
-    "duration_us": 1675.1,
-    "dram_bytes_read": 789000704,
-    "dram_bytes_write": 1361758000,
-    "dram_bytes_per_node_day": 56.01,
+    "duration_us": 1657.7,
+    "dram_bytes_read": 786245632,
+    "dram_bytes_write": 1358271000,
+    "dram_bytes_per_node_day": 55.85,
     "algorithmic_bytes_per_node_day": 68,
-    "issue_active_pct": 29.37,
-    "fp64_pipe_active_pct": 7.78,
-    "warps_active_pct": 21.15,
-    "stall_barrier_per_issue": 3.76,
-    "stall_long_scoreboard_per_issue": 1.63,
+    "issue_active_pct": 29.63,
+    "fp64_pipe_active_pct": 7.77,
+    "warps_active_pct": 21.13,
+    "stall_barrier_per_issue": 3.69,
+    "stall_long_scoreboard_per_issue": 1.61,
     "stall_wait_per_issue": 2.40,
     "l1_hit_pct": 32.0,
-    "l2_hit_pct": 45.4,
+    "l2_hit_pct": 45.5,
 }
 
 
